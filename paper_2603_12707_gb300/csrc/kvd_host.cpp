@@ -840,6 +840,7 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         pa.page_stride = stride;
         pa.err = c->err;
         pa.step_no = c->step_no;
+        pa.queues = c->queue;
         // Longest rows first: their items start early and the tail is short.
         pa.use_order = use_order ? 1 : 0;
         if (use_order)
@@ -934,6 +935,8 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     // Consecutive attention launches use different work counters: a chained
     // launch may start while the previous one drains, and each launch resets
     // the counter of the next one once the previous launch has completed.
+    // That order breaks where a graph replays an odd number of launches, so
+    // the step kernels zero both counters and a merge pass its launch's own.
     p.queue = c->queue + (c->attn_launches & 1u);
     p.queue_next = c->queue + ((c->attn_launches + 1u) & 1u);
     p.err = c->err;
@@ -1067,6 +1070,7 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     a.page_stride = c->dev_stride;
     a.err = c->err;
     a.step_no = c->step_no;
+    a.queues = c->queue;
     c->last_stream = st;
     KVD_CUDA(launch_step_device(a, st));
     ++c->launches;

@@ -87,6 +87,7 @@ struct PlanArgs {
     int32_t page_stride;
     int32_t* err;
     uint32_t* step_no;   // step counter, advanced by the launch that builds the plan
+    uint32_t* queues;    // the two work counters of the attention launches, zeroed by that launch
 };
 
 // kv_begin_step_device: the step's lazy allocation and plan, on the device.
@@ -110,6 +111,7 @@ struct StepDevArgs {
     int32_t page_stride;
     int32_t* err;
     uint32_t* step_no;        // step counter, advanced once per step
+    uint32_t* queues;         // the two work counters of the attention launches, zeroed
 };
 
 struct ScatterI32 {

@@ -333,3 +333,48 @@ def test_layer_graph_captured_after_another_replays_as_fast(kvlib):
     st = kd.kv_cache_query(h)
     assert st.device_error == 0
     t.close()
+
+
+@pytest.mark.parametrize("with_step", [True, False])
+@pytest.mark.parametrize("Hq,Hkv", [(8, 8), (56, 8)])
+def test_graph_of_one_layer_hands_out_every_item_on_every_replay(kvlib, Hq, Hkv, with_step):
+    """Consecutive attention launches alternate two work counters; a graph
+    with an odd number of them replays with the same counter, which must be
+    back at zero (more items than resident warps: some are claimed)."""
+    cfg = wl.custom("odd", 1, Hq, Hkv, 128, 16, lens=[1000 + 37 * b for b in range(16)], seed=71)
+    t = Tracked(cfg, extra_tokens=12, split_pages=1)
+    h, B = t.sess.h, cfg.batch
+    ids = torch.tensor(t.sess.seq_ids, dtype=torch.int32, device="cuda")
+    q, kn, vn = wl.step_inputs(cfg, 0, 0, "cuda")
+    out, ref = torch.empty_like(q), torch.empty_like(q)
+    torch.cuda.synchronize()
+    kd.kv_cache_device_steps(h, B)
+    s = torch.cuda.Stream()
+
+    def step(o):
+        kd.kv_begin_step_device(h, B, ids, s)
+        kd.decode_attention_append(h, 0, B, q, kn, vn, o, 0.0, s)
+
+    with torch.cuda.stream(s):
+        step(ref)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        if with_step:
+            kd.kv_begin_step_device(h, B, ids, s)
+        kd.decode_attention_append(h, 0, B, q, kn, vn, out, 0.0, s)
+    for rep in range(4):
+        with torch.cuda.stream(s):
+            if with_step:
+                out.zero_()
+                g.replay()
+                got = out.clone()
+                # the same layer again, launched by itself on the same step
+                kd.decode_attention(h, 0, B, q, ref, 0.0, s)
+            else:
+                out.zero_()
+                g.replay()
+                got = out.clone()
+        s.synchronize()
+        assert torch.equal(got, ref), rep
+    t.close()
