@@ -142,10 +142,11 @@ __global__ void __launch_bounds__(1024)
         const int seq = patch.seq[i], len = patch.new_len[i];
         a.seq_len[seq] = len;
         a.step_seq[patch.b0 + i] = seq;
+        if (a.no_plan) a.rows[patch.b0 + i] = make_int2(seq, len);
         if (patch.new_page[i] >= 0)
             a.page_table[(int64_t)seq * a.max_pages + (len - 1) / kPageSize] = patch.new_page[i];
     }
-    if (!a.build) return;
+    if (!a.build || a.no_plan) return;
     __syncthreads();
     build_split_plan(
         a.batch, a.item_pages, a.chunk_cap, INT_MAX,
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
         }
         if (i < a.batch) {
             a.step_seq[i] = ok ? seq : -1;
+            if (a.no_plan) a.rows[i] = make_int2(ok ? seq : 0, ok ? len : 0);   // no tokens: the row is left out
             if (small) {
                 s_seq[i] = ok ? seq : -1;
                 s_len[i] = ok ? len : 0;
@@ -227,6 +229,7 @@ __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
     }
     __syncthreads();
     if (threadIdx.x == 0) *a.free_top = top0 - min(carry, top0);
+    if (a.no_plan) return;
 
     // Row order: the rank of row b counts the rows with more pages, and the
     // rows with as many pages that come before b (failed rows have none).

@@ -1,0 +1,410 @@
+// Decode attention for steps with few (sequence, KV head) units (sm_103a): a
+// thread-block cluster per unit, no second pass.
+//
+// A unit's pages are cut evenly over all warps of its cluster (C CTAs of W
+// warps).  Each warp streams its pages through its own ring of shared-memory
+// stages and runs the same online softmax as the split pass
+// (kvd_decode_kernel.cuh).  The warps' (o, m, l) then merge by log-sum-exp in
+// two hops: within the CTA through shared memory, and across the cluster
+// through distributed shared memory, where CTA r receives every CTA's dims
+// [r D/C, (r+1) D/C) and writes them as bf16 output.
+//
+// What bounds it: such a layer holds a few MB, 1-2 us of HBM time, so the
+// chain of dependent latencies per layer decides.  The split pass and merge
+// pass pay two dependency hops (~1 us each) and two L2 round trips for the
+// partials; this kernel pays one hop and a cluster barrier.
+#include <algorithm>
+
+#include "kvd_decode_kernel.cuh"
+
+namespace kvd {
+
+namespace {
+
+constexpr int kClusterMaxCtas = 8;   // the portable cluster size
+constexpr int kClusterMaxWarps = 8;
+// Pages a warp brings into L2 before the dependency wait, beyond its ring.
+constexpr int kClusterL2Pages = 8;
+
+template <int D, bool GQA>
+struct ClusterGeo {
+    static constexpr int kStage = Geo<D, GQA>::kStageBytes;
+    static constexpr int kHeads = GQA ? kMaxGroup : 1;
+    static constexpr int kRow = D + 4;                          // floats per head of a warp's staged o (bank spread)
+    static constexpr int kRecv = kHeads * D * 4;                // this CTA's dims from every CTA of the cluster
+    static constexpr int kRecvMl = kClusterMaxCtas * kHeads * 8;
+    static constexpr int kWarpMl = kClusterMaxWarps * kHeads * 8;
+    static_assert(kHeads * kRow * 4 <= kStage, "a warp's staged o fits one stage of its ring");
+    static int smem(int warps, int ring)
+    {
+        return warps * ring * (kStage + 8) + kRecv + kRecvMl + kWarpMl + 8;
+    }
+};
+
+// A warp's unnormalised o ([head][kRow] floats) and (m, l) per head to shared memory.
+template <int D>
+__device__ __forceinline__ void stage_partial(MhaCompute<D>& c, float* wo, float2* wml, int lane)
+{
+    constexpr int CH = MhaCompute<D>::CH;
+    float o[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f2_unpack(c.o2[k], o[2 * k], o[2 * k + 1]);
+#pragma unroll
+    for (int mask = CH; mask < 32; mask <<= 1)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o[k] += __shfl_xor_sync(0xffffffffu, o[k], mask);
+    float l = c.l;
+#pragma unroll
+    for (int mask = 1; mask < 32; mask <<= 1) l += __shfl_xor_sync(0xffffffffu, l, mask);
+    if (c.tsub == 0) {
+        float4* dst = reinterpret_cast<float4*>(wo + c.c * 8);
+        dst[0] = make_float4(o[0], o[1], o[2], o[3]);
+        dst[1] = make_float4(o[4], o[5], o[6], o[7]);
+    }
+    if (lane == 0) wml[0] = make_float2(c.m, l);
+}
+
+template <int D>
+__device__ __forceinline__ void stage_partial(GqaCompute<D>& c, float* wo, float2* wml, int lane)
+{
+    constexpr int ROW = ClusterGeo<D, true>::kRow;
+    float l0 = c.l0, l1 = c.l1;
+#pragma unroll
+    for (int mask = 4; mask < 32; mask <<= 1) {
+        l0 += __shfl_xor_sync(0xffffffffu, l0, mask);
+        l1 += __shfl_xor_sync(0xffffffffu, l1, mask);
+    }
+    const int h0 = 2 * (lane & 3), h1 = h0 + 1, dlo = lane >> 2;
+#pragma unroll
+    for (int mt = 0; mt < GqaCompute<D>::KS; ++mt) {
+        const int d0 = mt * 16 + dlo;
+        wo[h0 * ROW + d0] = c.oacc[mt][0];
+        wo[h1 * ROW + d0] = c.oacc[mt][1];
+        wo[h0 * ROW + d0 + 8] = c.oacc[mt][2];
+        wo[h1 * ROW + d0 + 8] = c.oacc[mt][3];
+    }
+    if (lane < 4) {
+        wml[h0] = make_float2(c.m0, l0);
+        wml[h1] = make_float2(c.m1, l1);
+    }
+}
+
+// Weight of a partial with reference max m against M; a partial without
+// tokens (m = -inf) weighs 0 even when M is -inf too.
+__device__ __forceinline__ float lse_weight(float m, float M) { return m == -INFINITY ? 0.f : ex2(m - M); }
+
+// Keep a value read from the kernel parameters in a register from here on:
+// its first use would otherwise fetch the parameter line at the end of the
+// layer's dependent chain.
+template <class T>
+__device__ __forceinline__ void hold(T*& v) { asm volatile("" : "+l"(v)); }
+__device__ __forceinline__ void hold(int& v) { asm volatile("" : "+r"(v)); }
+
+template <int D, bool GQA, bool FUSED>
+__global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
+    cluster_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv,
+                   const DecodeParams p)
+{
+    using Cg = ClusterGeo<D, GQA>;
+    constexpr int STAGE = Cg::kStage;
+    constexpr int TILE = STAGE / 2;
+    // 128-byte swizzled stages need a 1024-byte aligned base; the kernel has no
+    // static shared memory, so its dynamic part starts at that alignment.
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int W = blockDim.x >> 5, R = p.ring;
+    const int C = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
+    const int log_dc = 31 - __clz(D / C);                                       // C is a power of two
+    uint8_t* ring = smem + warp * R * STAGE;
+    float* recv = reinterpret_cast<float*>(smem + W * R * STAGE);               // [C][G][D / C]
+    float2* recv_ml = reinterpret_cast<float2*>(reinterpret_cast<uint8_t*>(recv) + Cg::kRecv);   // [C][heads]
+    float2* warp_ml = recv_ml + kClusterMaxCtas * Cg::kHeads;                   // [W][heads]
+    uint64_t* recv_bar = reinterpret_cast<uint64_t*>(warp_ml + kClusterMaxWarps * Cg::kHeads);
+    uint64_t* bars = recv_bar + 1 + warp * R;
+    const uint32_t ring_s = smem_addr(ring);
+    int G = GQA ? p.G : 1;
+
+    // The next launch may start at once: it reads nothing this one writes
+    // before its own dependency wait (but for slots that it replaces).
+    griddep_launch_dependents();
+    bool waited = p.early == 0;
+    if (waited) griddep_wait();
+    const int unit = (int)blockIdx.x / C;
+    const int b = unit / p.H_kv, g = unit - b * p.H_kv;
+    const int2 row = p.rows[b];   // (sequence, tokens attended), by the step kernel; no tokens: the row's step failed
+    if (lane == 0) {
+        for (int s = 0; s < R; ++s) mbar_init(smem_addr(&bars[s]), 1);
+        if (warp == 0) mbar_init(smem_addr(recv_bar), 1);
+        fence_mbar_init();
+        if (warp == 0) {   // what the cluster sends this CTA: its dims and (M, L) of every CTA and head
+            prefetch_tensormap(&tmk);
+            if (!p.kv_map) prefetch_tensormap(&tmv);
+            mbar_arrive_expect_tx(smem_addr(recv_bar), G * D * 4 + C * G * 8);
+        }
+    }
+    __syncwarp();
+    cluster_arrive();   // "ready to receive": waited for before the first write to another CTA
+    const int len = row.y;
+    const int np = (len + kPageSize - 1) / kPageSize;
+    int first, n;
+    chunk_range(np, C * W, rank * W + warp, &first, &n);
+    const bool has_last = n > 0 && first + n == np;
+    const int32_t* pt_row = p.page_table + (int64_t)row.x * p.max_pages + first;
+    auto load_window = [&](int w0) { return (w0 + lane < n) ? pt_row[w0 + lane] : 0; };
+    int32_t pid_cur = load_window(0);
+    int32_t pid_next = 0;
+    const uint64_t policy = l2_policy_evict_first();
+    auto load = [&](int32_t pid, int s) {   // page pid into stage s, by one lane
+        if (pid < 0 || pid >= p.num_pages) {
+            atomicOr(p.err, 1);
+            pid = 0;
+        }
+        const uint32_t bar = smem_addr(&bars[s]);
+        const uint32_t dst = ring_s + s * STAGE;
+        const int32_t y = (pid * p.H_kv + g) * kPageSize;
+        mbar_arrive_expect_tx(bar, STAGE);
+        if (p.kv_map) {
+            tma_load_4d(dst, &tmk, 0, y, 0, 0, bar, policy);
+        } else {
+            tma_load_3d(dst, &tmk, 0, y, 0, bar, policy);
+            tma_load_3d(dst + TILE, &tmv, 0, y, 0, bar, policy);
+        }
+    };
+    auto issue = [&](int j, int s) {
+        if ((j & 31) == 8 && j + 24 < n) pid_next = load_window(j + 24);
+        if ((j & 31) == 0 && j > 0) pid_cur = pid_next;
+        const int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
+        if (lane == 0) load(pid, s);
+    };
+    const int pre = min(n, R);
+    if (lane < pre) load(pid_cur, lane);   // lane i: page i into stage i
+    // The pages past the ring into L2: when a stage is free again its next
+    // page is an L2 round trip away.
+    if (p.kv_map) {
+        const int end = min(min(n, 32), R + kClusterL2Pages);
+        if (lane >= R && lane < end && pid_cur >= 0 && pid_cur < p.num_pages)
+            tma_prefetch_l2_4d(&tmk, 0, (pid_cur * p.H_kv + g) * kPageSize, 0, 0);
+    }
+    __syncwarp();
+
+    PlanEntry en{};
+    en.b = b;
+    en.len = len;
+    float scale_log2 = p.scale_log2;
+    uint16_t* out = p.out + ((int64_t)b * p.H_q + g * G) * D;
+    hold(out);
+    hold(G);
+    if (!waited) griddep_wait();
+    using Comp = typename std::conditional<GQA, GqaCompute<D>, MhaCompute<D>>::type;
+    Comp comp;
+    comp.start(p, en, g, lane);
+    uint4 new_kv = make_uint4(0u, 0u, 0u, 0u);
+    if constexpr (FUSED)
+        if (has_last) new_kv = load_new_token<D>(p, en, g, lane);
+
+    uint32_t phase = 0, pending = (1u << pre) - 1u;
+    bool ok = true;
+    // Wait for page j in stage s and put the new token into it if it is the row's last.
+    auto arrived = [&](int j, int s) {
+        const bool w = mbar_wait_bounded(smem_addr(&bars[s]), (phase >> s) & 1u, kWaitLimitNs);
+        if (!__all_sync(0xffffffffu, w)) return false;
+        phase ^= 1u << s;
+        pending &= ~(1u << s);
+        if constexpr (FUSED) {
+            if (has_last && j == n - 1) {   // the page-id window has not moved past this page
+                const int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
+                put_new_token<D>(p, en, g, pid, new_kv, ring + s * STAGE, ring + s * STAGE + TILE, lane);
+            }
+        }
+        return true;
+    };
+    auto refill = [&](int j, int s) {
+        if (j + R < n) {
+            issue(j + R, s);
+            pending |= 1u << s;
+        }
+    };
+    auto after = [&](int s) { return s + 1 == R ? 0 : s + 1; };
+    auto tokens = [&](int j) { return min(kPageSize, len - (first + j) * kPageSize); };
+    int j = 0, s = 0;
+    if constexpr (!GQA) {
+        // two pages at a time: MHA's page is a dependent chain of ~440 cycles
+        for (; ok && j + 1 < n && R > 1; j += 2) {
+            const int s1 = after(s);
+            ok = arrived(j, s) && arrived(j + 1, s1);
+            if (!ok) break;
+            uint8_t* const k[2] = {ring + s * STAGE, ring + s1 * STAGE};
+            uint8_t* const v[2] = {k[0] + TILE, k[1] + TILE};
+            const int valid[2] = {tokens(j), tokens(j + 1)};
+            comp.template pages<2>(k, v, valid, scale_log2);
+            __syncwarp();
+            refill(j, s);
+            refill(j + 1, s1);
+            s = after(s1);
+        }
+    }
+    for (; ok && j < n; ++j) {
+        ok = arrived(j, s);
+        if (!ok) break;
+        const uint32_t sk = ring_s + s * STAGE;
+        comp.page(ring + s * STAGE, ring + s * STAGE + TILE, sk, sk + TILE, tokens(j), scale_log2, lane);
+        __syncwarp();
+        refill(j, s);
+        s = after(s);
+    }
+    if (!ok) {   // let the loads in flight land: their stages are about to be reused
+        if (lane == 0) atomicOr(p.err, 2);
+        for (int i = 0; i < R; ++i)
+            if (pending & (1u << i)) mbar_wait_bounded(smem_addr(&bars[i]), (phase >> i) & 1u, kWaitLimitNs);
+    }
+    __syncwarp();
+
+    // Hop 1: the CTA's warps, four dims of a head at a time; the result goes
+    // to the CTA of the cluster that owns those dims.
+    stage_partial<D>(comp, reinterpret_cast<float*>(ring), warp_ml + warp * Cg::kHeads, lane);
+    __syncthreads();
+    cluster_wait();
+    const uint32_t bar_s = smem_addr(recv_bar);
+    for (int i = threadIdx.x; i < G * (D / 4); i += blockDim.x) {
+        const int h = i / (D / 4), d0 = (i % (D / 4)) * 4;
+        // (fixed bounds, so that every load goes out before the first use)
+        float2 ml[kClusterMaxWarps];
+        float4 v[kClusterMaxWarps];
+#pragma unroll
+        for (int w = 0; w < kClusterMaxWarps; ++w) {
+            ml[w] = make_float2(-INFINITY, 0.f);
+            v[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (w < W) {
+                ml[w] = warp_ml[w * Cg::kHeads + h];
+                v[w] = *reinterpret_cast<const float4*>(smem + w * R * STAGE + (h * Cg::kRow + d0) * 4);
+            }
+        }
+        float M = ml[0].x;
+#pragma unroll
+        for (int w = 1; w < kClusterMaxWarps; ++w) M = fmaxf(M, ml[w].x);
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        float L = 0.f;
+#pragma unroll
+        for (int w = 0; w < kClusterMaxWarps; ++w) {
+            const float e = lse_weight(ml[w].x, M);
+            a.x = fmaf(e, v[w].x, a.x);
+            a.y = fmaf(e, v[w].y, a.y);
+            a.z = fmaf(e, v[w].z, a.z);
+            a.w = fmaf(e, v[w].w, a.w);
+            L = fmaf(e, ml[w].y, L);
+        }
+        const uint32_t dst = (uint32_t)(d0 >> log_dc);
+        const int dd = d0 & ((1 << log_dc) - 1);
+        const uint32_t bar = cluster_map(bar_s, dst);
+        cluster_store_async4(cluster_map(smem_addr(recv + ((rank * G + h) << log_dc) + dd), dst), a, bar);
+        // every CTA gets (M, L) of each head, from the thread of its first dims
+        if (dd == 0) cluster_store_async2(cluster_map(smem_addr(recv_ml + rank * Cg::kHeads + h), dst), M, L, bar);
+    }
+    if (!mbar_wait_bounded_cluster(bar_s, 0, kWaitLimitNs)) {
+        atomicOr(p.err, 2);
+        return;
+    }
+    // Hop 2: this CTA's dims over the cluster, two at a time.
+    if (np == 0) return;   // a row whose step failed: its output is left alone
+    for (int i = threadIdx.x; i < G << (log_dc - 1); i += blockDim.x) {
+        const int h = i >> (log_dc - 1), d0 = (i & ((1 << (log_dc - 1)) - 1)) * 2;
+        float2 ml[kClusterMaxCtas], v[kClusterMaxCtas];
+#pragma unroll
+        for (int c = 0; c < kClusterMaxCtas; ++c) {
+            ml[c] = make_float2(-INFINITY, 0.f);
+            v[c] = make_float2(0.f, 0.f);
+            if (c < C) {
+                ml[c] = recv_ml[c * Cg::kHeads + h];
+                v[c] = *reinterpret_cast<const float2*>(recv + ((c * G + h) << log_dc) + d0);
+            }
+        }
+        float M = ml[0].x;
+#pragma unroll
+        for (int c = 1; c < kClusterMaxCtas; ++c) M = fmaxf(M, ml[c].x);
+        float L = 0.f, x = 0.f, y = 0.f;
+#pragma unroll
+        for (int c = 0; c < kClusterMaxCtas; ++c) {
+            const float e = lse_weight(ml[c].x, M);
+            L = fmaf(e, ml[c].y, L);
+            x = fmaf(e, v[c].x, x);
+            y = fmaf(e, v[c].y, y);
+        }
+        const float inv = 1.f / L;
+        *reinterpret_cast<uint32_t*>(out + h * D + (rank << log_dc) + d0) = pack_bf16(x * inv, y * inv);
+    }
+}
+
+template <int D, bool GQA, bool FUSED>
+cudaError_t prepare_cluster()
+{
+    static cudaError_t status =
+        cudaFuncSetAttribute(cluster_kernel<D, GQA, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             ClusterGeo<D, GQA>::smem(kClusterMaxWarps, kClusterRingBytes / ClusterGeo<D, GQA>::kStage));
+    return status;
+}
+
+template <int D, bool GQA, bool FUSED>
+cudaError_t launch_variant(bool pdl, const ClusterShape& sh, int units, const CUtensorMap& tk, const CUtensorMap& tv,
+                           const DecodeParams& p, cudaStream_t st)
+{
+    if (cudaError_t e = prepare_cluster<D, GQA, FUSED>(); e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(units * sh.ctas));
+    cfg.blockDim = dim3((unsigned)(sh.warps * 32));
+    cfg.dynamicSmemBytes = (size_t)ClusterGeo<D, GQA>::smem(sh.warps, sh.ring);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)sh.ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, cluster_kernel<D, GQA, FUSED>, tk, tv, p);
+}
+
+template <int D, bool GQA>
+cudaError_t launch_shape(bool fused, bool pdl, const ClusterShape& sh, int units, const CUtensorMap& tk,
+                         const CUtensorMap& tv, const DecodeParams& p, cudaStream_t st)
+{
+    return fused ? launch_variant<D, GQA, true>(pdl, sh, units, tk, tv, p, st)
+                 : launch_variant<D, GQA, false>(pdl, sh, units, tk, tv, p, st);
+}
+
+}  // namespace
+
+template <int D, bool GQA>
+cudaError_t resident_shape(const ClusterShape& sh, int* clusters)
+{
+    if (cudaError_t e = prepare_cluster<D, GQA, true>(); e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)sh.ctas);
+    cfg.blockDim = dim3((unsigned)(sh.warps * 32));
+    cfg.dynamicSmemBytes = (size_t)ClusterGeo<D, GQA>::smem(sh.warps, sh.ring);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)sh.ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(clusters, cluster_kernel<D, GQA, true>, &cfg);
+}
+
+cudaError_t cluster_resident(int D, bool gqa, const ClusterShape& sh, int* clusters)
+{
+    if (D == 128) return gqa ? resident_shape<128, true>(sh, clusters) : resident_shape<128, false>(sh, clusters);
+    return gqa ? resident_shape<64, true>(sh, clusters) : resident_shape<64, false>(sh, clusters);
+}
+
+cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& sh, int units,
+                           const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t st)
+{
+    if (D == 128) return gqa ? launch_shape<128, true>(fused, pdl, sh, units, tk, tv, p, st)
+                             : launch_shape<128, false>(fused, pdl, sh, units, tk, tv, p, st);
+    if (D == 64) return gqa ? launch_shape<64, true>(fused, pdl, sh, units, tk, tv, p, st)
+                            : launch_shape<64, false>(fused, pdl, sh, units, tk, tv, p, st);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace kvd

@@ -131,37 +131,48 @@ struct MhaCompute {
         for (int k = 0; k < 4; ++k) o2[k] = 0ull;
     }
 
-    __device__ __forceinline__ void page(uint8_t* sK, uint8_t* sV, uint32_t, uint32_t, int valid,
-                                         float scale_log2, int lane)
+    // NP pages at once (their K tiles at sK[i], V tiles at sV[i], the first
+    // valid[i] of 16 tokens attended): the pages' dependent chains overlap.
+    template <int NP>
+    __device__ __forceinline__ void pages(uint8_t* const (&sK)[NP], uint8_t* const (&sV)[NP], const int (&valid)[NP],
+                                          float scale_log2)
     {
-        float part[IT];
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const uint4 kv = *reinterpret_cast<const uint4*>(sK + swz(i * TPI + tsub, c));
-            part[i] = dot8(kv, q2);
-        }
-        // Reduce-scatter over the CH lanes of a row: afterwards lane c holds
-        // token (c >> 1) * TPI + tsub, summed over all chunks.
-#pragma unroll
-        for (int lv = 0; lv < LOG_IT; ++lv) {
-            const int n = IT >> lv;
-            const int mask = CH >> (lv + 1);
-            const bool hi = (c & mask) != 0;
-#pragma unroll
-            for (int k = 0; k < n / 2; ++k) {
-                const float send = hi ? part[k] : part[k + n / 2];
-                const float keep = hi ? part[k + n / 2] : part[k];
-                part[k] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
-            }
-        }
-        float sc = part[0] + __shfl_xor_sync(0xffffffffu, part[0], 1);
         const int tok = (c >> 1) * TPI + tsub;
-        sc = (tok < valid) ? sc * scale_log2 : -INFINITY;
+        float sc[NP];
+        bool above = false;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            float part[IT];
+#pragma unroll
+            for (int i = 0; i < IT; ++i) {
+                const uint4 kv = *reinterpret_cast<const uint4*>(sK[q] + swz(i * TPI + tsub, c));
+                part[i] = dot8(kv, q2);
+            }
+            // Reduce-scatter over the CH lanes of a row: afterwards lane c holds
+            // token (c >> 1) * TPI + tsub, summed over all chunks.
+#pragma unroll
+            for (int lv = 0; lv < LOG_IT; ++lv) {
+                const int n = IT >> lv;
+                const int mask = CH >> (lv + 1);
+                const bool hi = (c & mask) != 0;
+#pragma unroll
+                for (int k = 0; k < n / 2; ++k) {
+                    const float send = hi ? part[k] : part[k + n / 2];
+                    const float keep = hi ? part[k + n / 2] : part[k];
+                    part[k] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+                }
+            }
+            const float x = part[0] + __shfl_xor_sync(0xffffffffu, part[0], 1);
+            sc[q] = (tok < valid[q]) ? x * scale_log2 : -INFINITY;
+            above |= sc[q] > m + 8.f;
+        }
         // The reference m moves only when a score exceeds it by more than 8
         // (log2 units; see GqaCompute::page), so most pages skip the max
         // reduction and the rescale.
-        if (__any_sync(0xffffffffu, sc > m + 8.f)) {
-            float pm = sc;
+        if (__any_sync(0xffffffffu, above)) {
+            float pm = sc[0];
+#pragma unroll
+            for (int q = 1; q < NP; ++q) pm = fmaxf(pm, sc[q]);
 #pragma unroll
             for (int mask = 2; mask < 32; mask <<= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, mask));
             const float mn = fmaxf(m, pm);
@@ -172,17 +183,29 @@ struct MhaCompute {
 #pragma unroll
             for (int k = 0; k < 4; ++k) o2[k] = f2_fma(o2[k], a2, 0ull);
         }
-        const float pe = ex2(sc - m);
-        l += (c & 1) ? 0.f : pe;
 #pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const float pt = __shfl_sync(0xffffffffu, pe, tsub * CH + 2 * i);
-            const int t = i * TPI + tsub;
-            if (t < valid) {   // rows past the end may hold anything
-                const uint4 vv = *reinterpret_cast<const uint4*>(sV + swz(t, c));
-                axpy8(o2, f2_pack(pt, pt), vv);
+        for (int q = 0; q < NP; ++q) {
+            const float pe = ex2(sc[q] - m);
+            l += (c & 1) ? 0.f : pe;
+#pragma unroll
+            for (int i = 0; i < IT; ++i) {
+                const float pt = __shfl_sync(0xffffffffu, pe, tsub * CH + 2 * i);
+                const int t = i * TPI + tsub;
+                if (t < valid[q]) {   // rows past the end may hold anything
+                    const uint4 vv = *reinterpret_cast<const uint4*>(sV[q] + swz(t, c));
+                    axpy8(o2, f2_pack(pt, pt), vv);
+                }
             }
         }
+    }
+
+    __device__ __forceinline__ void page(uint8_t* sK, uint8_t* sV, uint32_t, uint32_t, int valid,
+                                         float scale_log2, int)
+    {
+        uint8_t* const k[1] = {sK};
+        uint8_t* const v[1] = {sV};
+        const int n[1] = {valid};
+        pages<1>(k, v, n, scale_log2);
     }
 
     // Writes the output (a row of one item) or the item's partial (a split
@@ -234,14 +257,32 @@ struct GqaCompute {
     __device__ __forceinline__ void start(const DecodeParams& p, const PlanEntry& en, int g, int lane)
     {
         G = p.G;
-        const int n = lane >> 2;
-        const uint16_t* qrow = p.q + ((int64_t)en.b * p.H_q + g * G + (n < G ? n : 0)) * D;
+        // Lane (n, c) = (lane / 4, lane % 4) loads 16-byte chunks c, c + 4, ..
+        // of head n's row (4-byte loads in the fragment layout cost 8 L1
+        // wavefronts each); a 4 x 4 transpose of words over the lanes of a
+        // head then gives the B fragments (words c, c + 4, .. of the row).
+        const int n = lane >> 2, c = lane & 3;
+        const uint4* qrow = reinterpret_cast<const uint4*>(p.q + ((int64_t)en.b * p.H_q + g * G + (n < G ? n : 0)) * D) + c;
+        uint4 x[KS / 2];
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-            const uint32_t x0 = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * (lane & 3));
-            const uint32_t x1 = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * (lane & 3));
-            qb[ks][0] = (n < G) ? x0 : 0u;
-            qb[ks][1] = (n < G) ? x1 : 0u;
+        for (int j = 0; j < KS / 2; ++j) x[j] = qrow[4 * j];
+#pragma unroll
+        for (int j = 0; j < KS / 2; ++j) {
+            uint32_t w[4] = {x[j].x, x[j].y, x[j].z, x[j].w};
+#pragma unroll
+            for (int k = 0; k < 4; k += 2) {
+                const uint32_t t = __shfl_xor_sync(0xffffffffu, (c & 1) ? w[k] : w[k + 1], 1);
+                w[k] = (c & 1) ? t : w[k];
+                w[k + 1] = (c & 1) ? w[k + 1] : t;
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t t = __shfl_xor_sync(0xffffffffu, (c & 2) ? w[k] : w[k + 2], 2);
+                w[k] = (c & 2) ? t : w[k];
+                w[k + 2] = (c & 2) ? w[k + 2] : t;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) qb[2 * j + (k >> 1)][k & 1] = (n < G) ? w[k] : 0u;
         }
         m0 = m1 = -INFINITY;
         l0 = l1 = 0.f;

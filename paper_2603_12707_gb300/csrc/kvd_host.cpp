@@ -136,7 +136,13 @@ struct kv_cache {
     int32_t step_max_chunks = kMaxChunks;       // bound on the items of a row of the step
     int32_t step_batch = 0;
     int32_t step_entries = 0;
+    ClusterShape step_cluster{};                // the step's layers run as clusters (ctas > 0)
     int32_t split_override = 0;
+    int32_t dev_row_pages = 0;                  // longest row when device steps were enabled
+    int64_t dev_pages = 0;                      // pages held then (0: nothing known)
+    int32_t dev_seqs = 0;                       // sequences holding them
+    bool dev_split_override = false;
+    int cluster_resident[9][3][7];              // resident_clusters by [ctas][warps / 4][ring], -1: not asked yet
 
     int32_t* page_table() const { return meta; }
     int32_t* seq_len_dev() const { return meta + (int64_t)cfg.max_seqs * cfg.max_pages_per_seq; }
@@ -213,6 +219,62 @@ int32_t chunk_cap(const kv_cache* c, int64_t rows, int64_t max_pages, int32_t T)
     const bool few_units = rows * c->cfg.num_kv_heads * kChunkCap < warps;
     if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
     return c->group > 1 ? kChunkCapGqa : kChunkCap;
+}
+
+// Clusters of `shape` that the GPU holds at once (asked once per shape).
+int resident_clusters(kv_cache* c, const ClusterShape& sh)
+{
+    int& known = c->cluster_resident[sh.ctas][sh.warps / 4][sh.ring];
+    if (known < 0 && cluster_resident(c->cfg.head_dim, c->group > 1, sh, &known) != cudaSuccess) {
+        cudaGetLastError();
+        known = 0;
+    }
+    return known;
+}
+
+// Clusters for a step of `batch` rows that hold `pages` pages per KV head in
+// all and at most max_pages in one row, or ctas == 0: the split plan.
+//
+// The line between the two, measured as us per layer of graph-replayed steps
+// (split plan -> clusters).  Clusters save the merge pass and its dependency
+// hop (2.3 us), but cut the rows evenly, without the plan's balancing: they
+// win up to about 45 MB of K/V per layer (LLaVA heads, 800 tokens, B 1 / 2 / 3:
+// 6.5 -> 4.8, 9.2 -> 7.3, 11.2 -> 10.0; B 4, 52 MB: 13.5 -> 13.9; Qwen heads,
+// 1500 tokens, B 2 / 4 / 8: 5.3 -> 3.9, 7.0 -> 4.6, 9.3 -> 6.4; B 16, 46 MB:
+// 10.2 -> 10.4), unless one row is so long that its warps finish far behind
+// the others (Qwen heads, 8 rows of 300 to 3800 tokens, 8 pages per warp:
+// 9.8 -> 7.8; 1 row of 32000, 32 pages per warp: 19.5 -> 21.5).
+//
+// Of the shapes, the one with the most warps per unit whose units all find a
+// slot at once, with a tenth to spare for the next launch's (LLaVA heads,
+// B 3, 96 units: 4 x 4 warps with 2 stages, 110 slots, 10.0; with 3 stages,
+// 74 slots, 13.9), but no more than about a warp per page (8 x 8 against
+// 4 x 4 warps at 7 pages: 10.2 against 3.0).
+ClusterShape cluster_shape(kv_cache* c, int32_t batch, int64_t pages, int64_t max_pages)
+{
+    constexpr int64_t kMostBytes = 45000000;   // K and V of a layer
+    constexpr int kWarpsOf[][2] = {{8, 8}, {8, 4}, {4, 4}, {2, 4}, {1, 4}};
+    const int64_t units = (int64_t)batch * c->cfg.num_kv_heads;
+    const int64_t stage = 2 * (int64_t)kPageSize * c->cfg.head_dim * 2;
+    const int64_t bytes = pages * c->cfg.num_kv_heads * stage;
+    if (bytes > kMostBytes) return ClusterShape{};
+    for (const auto& cw : kWarpsOf) {
+        ClusterShape sh;
+        sh.ctas = cw[0];
+        sh.warps = cw[1];
+        const int64_t n = (int64_t)sh.ctas * sh.warps;
+        if (n > 4 && (n / 2 >= max_pages || (n == 64 && max_pages <= 128))) continue;
+        const int64_t per_warp = (max_pages + n - 1) / n;
+        const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
+        for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
+            if (10 * (int64_t)resident_clusters(c, sh) < 11 * units) continue;
+            // pages of the longest row's warps against the layer's share of HBM time
+            // the longest row's warps against what the layer's bytes take in
+            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB)
+            return per_warp * (c->cfg.head_dim == 128 ? 4000000 : 2800000) <= 20000000 + bytes ? sh : ClusterShape{};
+        }
+    }
+    return ClusterShape{};
 }
 
 int grow_scratch(kv_cache* c, int64_t entries, int64_t slots, int64_t page_ids, cudaStream_t st)
@@ -365,6 +427,7 @@ int kv_cache_create(const kvc_config* cfg, void* stream, kv_cache** out)
     if (k.flags & ~KVC_FLAG_HOST_ONLY) return fail(KVC_ERR_INVALID, "kv_cache_create: unknown flag");
 
     kv_cache* c = new kv_cache();
+    std::fill(&c->cluster_resident[0][0][0], &c->cluster_resident[0][0][0] + sizeof(c->cluster_resident) / sizeof(int), -1);
     c->cfg = k;
     c->host_only = (k.flags & KVC_FLAG_HOST_ONLY) != 0;
     c->group = k.num_q_heads / k.num_kv_heads;
@@ -794,19 +857,23 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         std::stable_sort(order.begin(), order.end(),
                          [&](int32_t x, int32_t y) { return np_after[x] > np_after[y]; });
     for (int32_t i = 0; i < batch; ++i) rank[order[i]] = i;
-    const int32_t cap = chunk_cap(c, batch, *std::max_element(np_after.begin(), np_after.end()), T);
+    const int32_t max_np = *std::max_element(np_after.begin(), np_after.end());
+    ClusterShape shape;
+    if (!c->split_override && !c->host_only)
+        shape = cluster_shape(c, batch, total_units / c->cfg.num_kv_heads, max_np);
+    const int32_t cap = chunk_cap(c, batch, max_np, T);
     int64_t entries = 0;
     int32_t stride = 1;
     bool split = false;
     int32_t max_chunks = 1;
-    for (int32_t b = 0; b < batch; ++b) {
+    for (int32_t b = 0; b < batch && !shape.ctas; ++b) {
         const int nch = row_chunks(np_after[b], row_item_pages(T, rank[b], batch), cap);
         entries += nch;
         split = split || nch > 1;
         max_chunks = std::max(max_chunks, nch);
         stride = std::max(stride, (np_after[b] + nch - 1) / nch);
     }
-    if (!c->host_only)
+    if (!c->host_only && !shape.ctas)
         if (int rc = grow_scratch(c, entries, entries * c->cfg.num_kv_heads, entries * stride,
                                   static_cast<cudaStream_t>(stream)))
             return rc;
@@ -841,6 +908,7 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         pa.err = c->err;
         pa.step_no = c->step_no;
         pa.queues = c->queue;
+        pa.no_plan = shape.ctas ? 1 : 0;
         // Longest rows first: their items start early and the tail is short.
         pa.use_order = use_order ? 1 : 0;
         if (use_order)
@@ -866,6 +934,7 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
     c->step_active = true;
     c->step_dev = false;
     c->step_split = split;
+    c->step_cluster = shape;
     c->step_max_chunks = max_chunks;
     c->page_stride = stride;
     c->step_batch = batch;
@@ -956,6 +1025,23 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     const int grid = (int)std::max<int64_t>(1, std::min(resident, want));
     p.kv_map = 1;
     const bool pdl = fused && c->chain_launches == c->launches && c->chain_stream == stream;
+    if (c->step_cluster.ctas) {
+        p.ring = c->step_cluster.ring;
+        p.early = pdl ? 1 : 0;
+        p.start_flags = nullptr;
+        p.step_no = nullptr;
+        p.tag = p.prev_tag = 0;
+        p.num_sms = c->num_sms;
+        c->last_stream = static_cast<cudaStream_t>(stream);
+        KVD_CUDA(launch_cluster(c->cfg.head_dim, c->group > 1, fused, pdl, c->step_cluster,
+                                batch * c->cfg.num_kv_heads, c->tmaps[layer], c->tmaps[layer], p,
+                                static_cast<cudaStream_t>(stream)));
+        ++c->launches;
+        c->prev_merge = false;
+        c->chain_launches = c->launches;
+        c->chain_stream = stream;
+        return KVC_OK;
+    }
     // The early L2 start waits for the previous launch's merge pass, so only
     // a launch chained after one that has a merge pass looks for it, and only
     // when both were issued the same way: eagerly, or into the same stream
@@ -1023,6 +1109,15 @@ int kv_cache_device_steps(kv_cache* c, int32_t max_batch, int32_t enable, void* 
     if (max_batch < 1 || max_batch > c->cfg.max_seqs)
         return fail(KVC_ERR_INVALID, "kv_cache_device_steps: max_batch outside 1 .. max_seqs");
     c->dev_mode = false;   // (re-)enabling may resize the buffers
+    c->dev_row_pages = 0;
+    c->dev_pages = c->pages_in_use;
+    c->dev_seqs = 0;
+    for (int32_t s = 0; s < c->cfg.max_seqs; ++s)
+        if (c->lens[s] > 0) {
+            c->dev_row_pages = std::max(c->dev_row_pages, (int32_t)c->pages[s].size());
+            ++c->dev_seqs;
+        }
+    c->dev_split_override = c->split_override != 0;
     // Work-item size from the pages now held (steps add a token per sequence).
     const int32_t T = c->split_override
                           ? c->split_override
@@ -1071,6 +1166,15 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     a.err = c->err;
     a.step_no = c->step_no;
     a.queues = c->queue;
+    // The rows' lengths are the device's: judge the step by the pages held
+    // when device steps were enabled, or by full rows if there were none.
+    ClusterShape shape;
+    if (!c->dev_split_override) {
+        const int64_t row = c->dev_seqs ? c->dev_row_pages + 1 : c->cfg.max_pages_per_seq;
+        const int64_t pages = c->dev_seqs ? (c->dev_pages * batch + c->dev_seqs - 1) / c->dev_seqs : row * batch;
+        shape = cluster_shape(c, batch, pages, row);
+    }
+    a.no_plan = shape.ctas ? 1 : 0;
     c->last_stream = st;
     KVD_CUDA(launch_step_device(a, st));
     ++c->launches;
@@ -1079,6 +1183,7 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     c->prev_merge = false;
     c->step_active = true;
     c->step_dev = true;
+    c->step_cluster = shape;
     c->step_split = true;   // the row split is only known on the device: always run the merge pass
     c->step_max_chunks =
         row_chunks(c->cfg.max_pages_per_seq, row_item_pages(c->dev_item_pages, batch, batch), c->dev_chunk_cap);

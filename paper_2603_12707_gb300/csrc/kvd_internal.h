@@ -71,7 +71,8 @@ struct StepPatch {
 };
 
 struct PlanArgs {
-    int32_t build;       // build the plan in this launch (last launch of a step)
+    int32_t build;       // 1: build the plan in this launch (last launch of a step)
+    int32_t no_plan;     // 1: the step runs without a plan (clusters): update lengths and pages only
     int32_t batch;
     int32_t item_pages;  // target pages per work item (T)
     int32_t max_pages;   // page-table row length
@@ -103,6 +104,7 @@ struct StepDevArgs {
     int32_t* step_seq;        // out: [batch] sequence of each row, -1 where the row's step failed
     int32_t* seq_len;
     int32_t* page_table;
+    int32_t no_plan;          // 1: the step runs without a plan (clusters)
     PlanEntry* plan;
     int2* rows;
     int32_t* n_entries;       // out: plan entries of the step
@@ -192,7 +194,7 @@ struct DecodeParams {
     const PlanEntry* plan;
     float* part_o;            // [slots][G][D]
     float2* part_ml;          // [slots][G]  (running max in log2 units, sum)
-    const int2* rows;         // [batch]: (first partial slot, items) per batch row
+    const int2* rows;         // [batch]: (first partial slot, items) per batch row; for clusters (sequence, tokens)
     const int32_t* item_pages;// [entries][page_stride]: page ids of each plan entry's pages
     int32_t page_stride;
     const int32_t* n_entries_dev; // device-built plan: entries live here (n_items is then a bound)
@@ -225,7 +227,17 @@ struct DecodeParams {
     const uint32_t* step_no;
     uint32_t tag, prev_tag;
     int32_t num_sms;
+    // cluster_kernel only: it reads lengths and page ids by batch row instead of a plan.
+    int32_t ring;             // shared-memory stages per warp
+    int32_t early;            // 1: the cache may be read before the dependency wait
 };
+
+// Clusters of a step with few (sequence, KV head) units: CTAs per unit, warps
+// per CTA, ring stages per warp.  ctas == 0: the step runs from a split plan.
+struct ClusterShape {
+    int ctas = 0, warps = 0, ring = 0;
+};
+constexpr int kClusterRingBytes = 24576;   // a warp's ring at most (3 stages at d = 128, as the split pass)
 
 // TMA view of a (page, head) tile: box {64 columns, 16 rows, D/64 column
 // halves} of a pool whose rows are D bf16 (row index (page*H_kv + head)*16 +
@@ -280,5 +292,10 @@ cudaError_t launch_merge(int D, bool pdl, int max_chunks, int num_sms, int split
 // reads q / k_new / v_new and writes anything only after it has).
 cudaError_t launch_decode(int D, bool gqa, bool fused, bool pdl, int grid, const CUtensorMap& tk, const CUtensorMap& tv,
                           const DecodeParams& p, cudaStream_t st);
+// Decode attention with one cluster per (row, KV head) unit, no second pass
+// (kvd_cluster.cu).  pdl: launched with programmatic dependent launch.
+cudaError_t cluster_resident(int D, bool gqa, const ClusterShape& shape, int* clusters);   // clusters the GPU holds
+cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& shape, int units,
+                           const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t st);
 
 }  // namespace kvd
