@@ -431,6 +431,9 @@ __global__ void __launch_bounds__(kVarlenThreads) varlen_write_kernel(const __gr
 // the chunk goes to slot (len-1) % P of page page_table[seq][(len-1) / P].
 __global__ void append_kernel(const AppendArgs a)
 {
+    // Every thread waits (and so completes after) the kernel before it.
+    griddep_launch_dependents();
+    griddep_wait();
     const int chunks = a.D / 8;
     const int total = a.batch * a.H_kv * chunks;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -552,12 +555,20 @@ cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t launch_append(const AppendArgs& a, cudaStream_t st)
+cudaError_t launch_append(const AppendArgs& a, bool pdl, cudaStream_t st)
 {
     const int total = a.batch * a.H_kv * (a.D / 8);
     if (total <= 0) return cudaSuccess;
-    append_kernel<<<(total + 255) / 256, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((total + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, append_kernel, a);
 }
 
 }  // namespace kvd

@@ -177,7 +177,10 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
         if (lane == 0) load(pid, s);
     };
     const int pre = min(n, R);
-    if (lane < pre) load(pid_cur, lane);   // lane i: page i into stage i
+    // lane i: page i into stage i (after a kv_append a row's last page only
+    // once that is complete)
+    const bool late_page = p.hold_last && has_last && n == pre;
+    if (lane < pre - (late_page ? 1 : 0)) load(pid_cur, lane);
     // The pages past the ring into L2: when a stage is free again its next
     // page is an L2 round trip away.
     if (p.kv_map) {
@@ -195,6 +198,8 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     hold(out);
     hold(G);
     if (!waited) griddep_wait();
+    if (late_page && lane == pre - 1) load(pid_cur, lane);
+    __syncwarp();
     using Comp = typename std::conditional<GQA, GqaCompute<D>, MhaCompute<D>>::type;
     Comp comp;
     comp.start(p, en, g, lane);

@@ -38,13 +38,7 @@ template <int D, bool GQA>
 cudaError_t launch_variant(bool fused, bool pdl, int grid, const CUtensorMap& tk, const CUtensorMap& tv,
                            const DecodeParams& p, cudaStream_t st)
 {
-    if (!fused) {
-        cudaError_t e = prepare_variant<D, GQA, false>();
-        if (e != cudaSuccess) return e;
-        decode_kernel<D, GQA, false><<<grid, kWarps * 32, Geo<D, GQA>::kSmem, st>>>(tk, tv, p);
-        return cudaGetLastError();
-    }
-    cudaError_t e = prepare_variant<D, GQA, true>();
+    cudaError_t e = fused ? prepare_variant<D, GQA, true>() : prepare_variant<D, GQA, false>();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -56,7 +50,8 @@ cudaError_t launch_variant(bool fused, bool pdl, int grid, const CUtensorMap& tk
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, true>, tk, tv, p);
+    return fused ? cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, true>, tk, tv, p)
+                 : cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, false>, tk, tv, p);
 }
 
 }  // namespace

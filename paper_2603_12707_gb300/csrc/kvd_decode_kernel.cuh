@@ -20,8 +20,8 @@
 // Q.K^T and P.V as m16n8k16 bf16 MMAs with the 16 tokens of a page as M and the
 // G heads (padded to 8) as N.
 //
-// Chained launches (programmatic dependent launch, decode_attention_append
-// after another attention launch): a warp issues its first item's ring loads
+// Chained launches (programmatic dependent launch, after another attention
+// launch or a kv_append): a warp issues its first item's ring loads
 // before the dependency wait; once the previous launch's merge pass announces
 // (start_flags) that its split pass is complete, the warp brings the item's
 // next kEarlyL2Pages pages into L2; and right after its wait it brings the
@@ -511,10 +511,11 @@ __global__ void __launch_bounds__(kWarps * 32)
 
     using Comp = typename std::conditional<GQA, GqaCompute<D>, MhaCompute<D>>::type;
     Comp comp;
-    // Fused launches depend programmatically on the previous kernel: until
+    // Chained launches depend programmatically on the previous kernel: until
     // griddep_wait() only the plan, page table and cache pages (none of which
-    // that kernel writes) are read; q, k_new, v_new and every write come after.
-    bool waited = !FUSED;
+    // that kernel writes, but for a kv_append each row's last page) are read;
+    // q, k_new, v_new and every write come after.
+    bool waited = false;
     bool first_item = true;
 
     // The first item of every warp is its global warp index; later ones come
@@ -558,9 +559,12 @@ __global__ void __launch_bounds__(kWarps * 32)
             }
         };
 
+        const bool last_chunk = en.chunk == en.n_chunks - 1;
         const int pre = np < R ? np : R;
+        // After a kv_append a row's last page is loaded only once that is complete.
+        const bool hold = !FUSED && !waited && p.hold_last && last_chunk && np == pre;
         __syncwarp();
-        for (int j = 0; j < pre; ++j) issue(j, j);
+        for (int j = 0; j < pre - (hold ? 1 : 0); ++j) issue(j, j);
         pending = (1u << pre) - 1u;
         int ramp0 = R;   // first page of the L2 ramp at the wait's return
         if (!waited && p.prev_tag && np > R && p.kv_map) {
@@ -588,6 +592,7 @@ __global__ void __launch_bounds__(kWarps * 32)
             griddep_wait();
             griddep_launch_dependents();
             waited = true;
+            if (hold) issue(pre - 1, pre - 1);
         }
         if (first_item && p.kv_map) {
             // The ring holds this item's first R pages (loaded before the
@@ -600,7 +605,6 @@ __global__ void __launch_bounds__(kWarps * 32)
         }
         first_item = false;
         comp.start(p, en, g, lane);
-        const bool last_chunk = en.chunk == en.n_chunks - 1;
         uint4 new_kv = make_uint4(0u, 0u, 0u, 0u);
         if constexpr (FUSED)
             if (last_chunk) new_kv = load_new_token<D>(p, en, g, lane);

@@ -230,6 +230,7 @@ struct DecodeParams {
     // cluster_kernel only: it reads lengths and page ids by batch row instead of a plan.
     int32_t ring;             // shared-memory stages per warp
     int32_t early;            // 1: the cache may be read before the dependency wait
+    int32_t hold_last;        // 1: but not each row's last page (a kv_append may be writing it)
 };
 
 // Clusters of a step with few (sequence, KV head) units: CTAs per unit, warps
@@ -263,7 +264,9 @@ cudaError_t launch_gather_pages(const PlanEntry* plan, int32_t entries, const in
                                 int num_sms, cudaStream_t st);
 cudaError_t launch_step_device(const StepDevArgs& a, cudaStream_t st);
 cudaError_t launch_seq_op(const SeqOpArgs& a, cudaStream_t st);
-cudaError_t launch_append(const AppendArgs& a, cudaStream_t st);
+// pdl: launched with programmatic dependent launch (it waits for the kernel
+// before it first, and lets the next one start at once).
+cudaError_t launch_append(const AppendArgs& a, bool pdl, cudaStream_t st);
 cudaError_t launch_wait_timeout_check(uint64_t limit_ns, int32_t* status, cudaStream_t st);
 
 // Decode attention: variant chosen by (D, G == 1).
@@ -287,9 +290,9 @@ cudaError_t decode_variant_info(int D, bool gqa, DecodeVariant* v);
 // each of an SM's four schedulers (0: nothing resident beside it).
 cudaError_t launch_merge(int D, bool pdl, int max_chunks, int num_sms, int split_regs_per_subpartition,
                          const DecodeParams& p, cudaStream_t st);
-// fused: the append + attention kernel, launched with programmatic dependent
-// launch (it streams its first pages before the previous kernel finishes and
-// reads q / k_new / v_new and writes anything only after it has).
+// fused: the append + attention kernel.  pdl: launched with programmatic
+// dependent launch (it streams its first pages before the previous kernel
+// finishes and reads q / k_new / v_new and writes anything only after it has).
 cudaError_t launch_decode(int D, bool gqa, bool fused, bool pdl, int grid, const CUtensorMap& tk, const CUtensorMap& tv,
                           const DecodeParams& p, cudaStream_t st);
 // Decode attention with one cluster per (row, KV head) unit, no second pass

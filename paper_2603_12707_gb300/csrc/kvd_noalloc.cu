@@ -270,6 +270,7 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     p.step_no = nullptr;
     p.tag = p.prev_tag = 0;
     p.num_sms = num_sms;
+    p.hold_last = 0;
     p.k_new = p.v_new = nullptr;
     p.pool_k = p.pool_v = nullptr;
     const int64_t resident = (int64_t)num_sms * std::max(1, var.ctas_per_sm);

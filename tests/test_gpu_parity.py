@@ -403,3 +403,37 @@ def test_graph_replayed_steps_match_oracle_full_size(name, layers, rows):
         ref, vmax = t.oracle(l, ins[l][0], rows=rows)
         assert_close(bf16_to_f64(outs[l])[rows], ref, vmax, gqa=cfg.group > 1, what=(name, l))
     t.close()
+
+
+@pytest.mark.parametrize("lens,split", [([3, 16, 40, 700], 0), ([3, 16, 31, 5000], 2), ([1500] * 24 + [15, 16, 0], 0)])
+@pytest.mark.parametrize("Hq,Hkv", [(8, 8), (28, 4)])
+def test_chained_append_then_attend_sees_the_new_token(kvlib, Hq, Hkv, lens, split):
+    """kv_append and decode_attention of consecutive layers are chained: a
+    layer's pages load while its append is still waiting, but for the row's
+    last page.  The slot the append fills holds a huge stale K before it, so
+    a page loaded too early would show (several layers, no host waits)."""
+    cfg = wl.custom("chain", 6, Hq, Hkv, 128, len(lens), lens=lens, seed=83, page_order="shuffled")
+    outs = []
+    for fused in (True, False):
+        t = Tracked(cfg, extra_tokens=8, split_pages=split, keep_host=False)
+        s = torch.cuda.Stream()
+        ins = [wl.step_inputs(cfg, 0, l, "cuda") for l in range(cfg.num_layers)]
+        stale = torch.full_like(ins[0][1], 30.0)
+        res = [torch.empty_like(i[0]) for i in ins]
+        torch.cuda.synchronize()
+        kd.kv_begin_step(t.sess.h, t.sess.seq_ids, s)
+        for l in range(cfg.num_layers):
+            kd.kv_append(t.sess.h, l, cfg.batch, stale, stale, s)
+        for rep in range(3):
+            for l, (q, kn, vn) in enumerate(ins):
+                if fused:
+                    kd.decode_attention_append(t.sess.h, l, cfg.batch, q, kn, vn, res[l], 0.0, s)
+                else:
+                    kd.kv_append(t.sess.h, l, cfg.batch, kn, vn, s)
+                    kd.decode_attention(t.sess.h, l, cfg.batch, q, res[l], 0.0, s)
+        s.synchronize()
+        outs.append(res)
+        t.sess.lens += 1
+        t.close()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
