@@ -251,6 +251,7 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     for (; ok && j < n; ++j) {
         ok = arrived(j, s);
         if (!ok) break;
+        if (GQA && j == 0) comp.ready(lane);
         const uint32_t sk = ring_s + s * STAGE;
         comp.page(ring + s * STAGE, ring + s * STAGE + TILE, sk, sk + TILE, tokens(j), scale_log2, lane);
         __syncwarp();

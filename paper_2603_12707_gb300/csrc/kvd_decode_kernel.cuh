@@ -131,6 +131,8 @@ struct MhaCompute {
         for (int k = 0; k < 4; ++k) o2[k] = 0ull;
     }
 
+    __device__ __forceinline__ void ready(int) {}
+
     // NP pages at once (their K tiles at sK[i], V tiles at sV[i], the first
     // valid[i] of 16 tokens attended): the pages' dependent chains overlap.
     template <int NP>
@@ -249,6 +251,8 @@ struct MhaCompute {
 template <int D>
 struct GqaCompute {
     static constexpr int KS = D / 16;
+    // The 4-byte loads take an L1 wavefront per head and instruction.
+    static constexpr int kNarrowQ = 4;
     int G;
     uint32_t qb[KS][2];
     float m0, m1, l0, l1;
@@ -257,32 +261,23 @@ struct GqaCompute {
     __device__ __forceinline__ void start(const DecodeParams& p, const PlanEntry& en, int g, int lane)
     {
         G = p.G;
-        // Lane (n, c) = (lane / 4, lane % 4) loads 16-byte chunks c, c + 4, ..
-        // of head n's row (4-byte loads in the fragment layout cost 8 L1
-        // wavefronts each); a 4 x 4 transpose of words over the lanes of a
-        // head then gives the B fragments (words c, c + 4, .. of the row).
+        // More than kNarrowQ heads: lane (n, c) = (lane / 4, lane % 4) loads
+        // 16-byte chunks c, c + 4, .. of head n's row, and ready() makes them
+        // the B fragments; fewer: 4-byte loads in the fragment layout.
         const int n = lane >> 2, c = lane & 3;
-        const uint4* qrow = reinterpret_cast<const uint4*>(p.q + ((int64_t)en.b * p.H_q + g * G + (n < G ? n : 0)) * D) + c;
-        uint4 x[KS / 2];
+        const uint16_t* row = p.q + ((int64_t)en.b * p.H_q + g * G + (n < G ? n : 0)) * D;
+        if (G > kNarrowQ) {
 #pragma unroll
-        for (int j = 0; j < KS / 2; ++j) x[j] = qrow[4 * j];
-#pragma unroll
-        for (int j = 0; j < KS / 2; ++j) {
-            uint32_t w[4] = {x[j].x, x[j].y, x[j].z, x[j].w};
-#pragma unroll
-            for (int k = 0; k < 4; k += 2) {
-                const uint32_t t = __shfl_xor_sync(0xffffffffu, (c & 1) ? w[k] : w[k + 1], 1);
-                w[k] = (c & 1) ? t : w[k];
-                w[k + 1] = (c & 1) ? w[k + 1] : t;
+            for (int j = 0; j < KS / 2; ++j) {
+                const uint4 x = reinterpret_cast<const uint4*>(row)[c + 4 * j];
+                qb[2 * j][0] = x.x;
+                qb[2 * j][1] = x.y;
+                qb[2 * j + 1][0] = x.z;
+                qb[2 * j + 1][1] = x.w;
             }
+        } else {
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const uint32_t t = __shfl_xor_sync(0xffffffffu, (c & 2) ? w[k] : w[k + 2], 2);
-                w[k] = (c & 2) ? t : w[k];
-                w[k + 2] = (c & 2) ? w[k + 2] : t;
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) qb[2 * j + (k >> 1)][k & 1] = (n < G) ? w[k] : 0u;
+            for (int i = 0; i < 2 * KS; ++i) qb[i >> 1][i & 1] = reinterpret_cast<const uint32_t*>(row)[4 * i + c];
         }
         m0 = m1 = -INFINITY;
         l0 = l1 = 0.f;
@@ -290,6 +285,38 @@ struct GqaCompute {
         for (int mt = 0; mt < KS; ++mt)
 #pragma unroll
             for (int k = 0; k < 4; ++k) oacc[mt][k] = 0.f;
+    }
+
+    // Once, before the first page and after everything that can overlap the
+    // loads of q (waiting for them in start() cost short items 2 %): a 4 x 4
+    // transpose of words over the lanes of a head (words c, c + 4, .. of the
+    // row).
+    __device__ __forceinline__ void ready(int lane)
+    {
+        const int n = lane >> 2, c = lane & 3;
+        if (G > kNarrowQ) {
+#pragma unroll
+            for (int j = 0; j < KS / 2; ++j) {
+                uint32_t w[4] = {qb[2 * j][0], qb[2 * j][1], qb[2 * j + 1][0], qb[2 * j + 1][1]};
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    const uint32_t t = __shfl_xor_sync(0xffffffffu, (c & 1) ? w[k] : w[k + 1], 1);
+                    w[k] = (c & 1) ? t : w[k];
+                    w[k + 1] = (c & 1) ? w[k + 1] : t;
+                }
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const uint32_t t = __shfl_xor_sync(0xffffffffu, (c & 2) ? w[k] : w[k + 2], 2);
+                    w[k] = (c & 2) ? t : w[k];
+                    w[k + 2] = (c & 2) ? w[k + 2] : t;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) qb[2 * j + (k >> 1)][k & 1] = w[k];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * KS; ++i)
+            if (n >= G) qb[i >> 1][i & 1] = 0u;
     }
 
     __device__ __forceinline__ void page(uint8_t*, uint8_t*, uint32_t sK, uint32_t sV, int valid,
@@ -618,6 +645,7 @@ __global__ void __launch_bounds__(kWarps * 32)
             }
             phase ^= 1u << s;
             pending &= ~(1u << s);
+            if (GQA && j == 0) comp.ready(lane);
             const int valid = min(kPageSize, en.len - (en.first_page + j) * kPageSize);
             uint8_t* sK = ring + s * STAGE;
             // Generic-proxy writes into the stage (the new token's row) must be
