@@ -14,6 +14,7 @@
 // pass pay two dependency hops (~1 us each) and two L2 round trips for the
 // partials; this kernel pays one hop and a cluster barrier.
 #include <algorithm>
+#include <atomic>
 
 #include "kvd_decode_kernel.cuh"
 
@@ -100,10 +101,10 @@ template <class T>
 __device__ __forceinline__ void hold(T*& v) { asm volatile("" : "+l"(v)); }
 __device__ __forceinline__ void hold(int& v) { asm volatile("" : "+r"(v)); }
 
-template <int D, bool GQA, bool FUSED>
+template <int D, bool GQA, bool FUSED, class Rows>
 __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     cluster_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv,
-                   const DecodeParams p)
+                   const DecodeParams p, const __grid_constant__ Rows rt)
 {
     using Cg = ClusterGeo<D, GQA>;
     constexpr int STAGE = Cg::kStage;
@@ -131,7 +132,9 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     if (waited) griddep_wait();
     const int unit = (int)blockIdx.x / C;
     const int b = unit / p.H_kv, g = unit - b * p.H_kv;
-    const int2 row = p.rows[b];   // (sequence, tokens attended), by the step kernel; no tokens: the row's step failed
+    int2 row;   // (page-table row, tokens attended)
+    if constexpr (Rows::kTable) row = make_int2(b, rt.len[b]);
+    else row = p.rows[b];   // by the step kernel; no tokens: the row's step failed
     if (lane == 0) {
         for (int s = 0; s < R; ++s) mbar_init(smem_addr(&bars[s]), 1);
         if (warp == 0) mbar_init(smem_addr(recv_bar), 1);
@@ -207,6 +210,7 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     if constexpr (FUSED)
         if (has_last) new_kv = load_new_token<D>(p, en, g, lane);
 
+    const int k_off = Rows::kTable && p.kv_map == 2 ? TILE : 0, v_off = TILE - k_off;   // K and V within a stage
     uint32_t phase = 0, pending = (1u << pre) - 1u;
     bool ok = true;
     // Wait for page j in stage s and put the new token into it if it is the row's last.
@@ -218,7 +222,7 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
         if constexpr (FUSED) {
             if (has_last && j == n - 1) {   // the page-id window has not moved past this page
                 const int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
-                put_new_token<D>(p, en, g, pid, new_kv, ring + s * STAGE, ring + s * STAGE + TILE, lane);
+                put_new_token<D>(p, en, g, pid, new_kv, ring + s * STAGE + k_off, ring + s * STAGE + v_off, lane);
             }
         }
         return true;
@@ -238,8 +242,8 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
             const int s1 = after(s);
             ok = arrived(j, s) && arrived(j + 1, s1);
             if (!ok) break;
-            uint8_t* const k[2] = {ring + s * STAGE, ring + s1 * STAGE};
-            uint8_t* const v[2] = {k[0] + TILE, k[1] + TILE};
+            uint8_t* const k[2] = {ring + s * STAGE + k_off, ring + s1 * STAGE + k_off};
+            uint8_t* const v[2] = {ring + s * STAGE + v_off, ring + s1 * STAGE + v_off};
             const int valid[2] = {tokens(j), tokens(j + 1)};
             comp.template pages<2>(k, v, valid, scale_log2);
             __syncwarp();
@@ -252,8 +256,9 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
         ok = arrived(j, s);
         if (!ok) break;
         if (GQA && j == 0) comp.ready(lane);
-        const uint32_t sk = ring_s + s * STAGE;
-        comp.page(ring + s * STAGE, ring + s * STAGE + TILE, sk, sk + TILE, tokens(j), scale_log2, lane);
+        uint8_t* sk = ring + s * STAGE;
+        const uint32_t a = ring_s + s * STAGE;
+        comp.page(sk + k_off, sk + v_off, a + k_off, a + v_off, tokens(j), scale_log2, lane);
         __syncwarp();
         refill(j, s);
         s = after(s);
@@ -340,20 +345,20 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     }
 }
 
-template <int D, bool GQA, bool FUSED>
+template <int D, bool GQA, bool FUSED, class Rows = PlanRows>
 cudaError_t prepare_cluster()
 {
     static cudaError_t status =
-        cudaFuncSetAttribute(cluster_kernel<D, GQA, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(cluster_kernel<D, GQA, FUSED, Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              ClusterGeo<D, GQA>::smem(kClusterMaxWarps, kClusterRingBytes / ClusterGeo<D, GQA>::kStage));
     return status;
 }
 
-template <int D, bool GQA, bool FUSED>
+template <int D, bool GQA, bool FUSED, class Rows>
 cudaError_t launch_variant(bool pdl, const ClusterShape& sh, int units, const CUtensorMap& tk, const CUtensorMap& tv,
-                           const DecodeParams& p, cudaStream_t st)
+                           const DecodeParams& p, const Rows& rows, cudaStream_t st)
 {
-    if (cudaError_t e = prepare_cluster<D, GQA, FUSED>(); e != cudaSuccess) return e;
+    if (cudaError_t e = prepare_cluster<D, GQA, FUSED, Rows>(); e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(units * sh.ctas));
     cfg.blockDim = dim3((unsigned)(sh.warps * 32));
@@ -367,18 +372,17 @@ cudaError_t launch_variant(bool pdl, const ClusterShape& sh, int units, const CU
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, cluster_kernel<D, GQA, FUSED>, tk, tv, p);
+    return cudaLaunchKernelEx(&cfg, cluster_kernel<D, GQA, FUSED, Rows>, tk, tv, p, rows);
 }
 
 template <int D, bool GQA>
 cudaError_t launch_shape(bool fused, bool pdl, const ClusterShape& sh, int units, const CUtensorMap& tk,
-                         const CUtensorMap& tv, const DecodeParams& p, cudaStream_t st)
+                         const CUtensorMap& tv, const DecodeParams& p, const LensTable* lens, cudaStream_t st)
 {
-    return fused ? launch_variant<D, GQA, true>(pdl, sh, units, tk, tv, p, st)
-                 : launch_variant<D, GQA, false>(pdl, sh, units, tk, tv, p, st);
+    if (lens) return launch_variant<D, GQA, false>(pdl, sh, units, tk, tv, p, *lens, st);
+    return fused ? launch_variant<D, GQA, true>(pdl, sh, units, tk, tv, p, PlanRows{}, st)
+                 : launch_variant<D, GQA, false>(pdl, sh, units, tk, tv, p, PlanRows{}, st);
 }
-
-}  // namespace
 
 template <int D, bool GQA>
 cudaError_t resident_shape(const ClusterShape& sh, int* clusters)
@@ -394,23 +398,83 @@ cudaError_t resident_shape(const ClusterShape& sh, int* clusters)
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(clusters, cluster_kernel<D, GQA, true>, &cfg);
+    return cudaOccupancyMaxActiveClusters(clusters, cluster_kernel<D, GQA, true, PlanRows>, &cfg);
 }
 
-cudaError_t cluster_resident(int D, bool gqa, const ClusterShape& sh, int* clusters)
+// Clusters of a shape that the GPU holds at once, asked once per device and shape.
+int resident_clusters(int device, int D, bool gqa, const ClusterShape& sh)
 {
-    if (D == 128) return gqa ? resident_shape<128, true>(sh, clusters) : resident_shape<128, false>(sh, clusters);
-    return gqa ? resident_shape<64, true>(sh, clusters) : resident_shape<64, false>(sh, clusters);
+    static std::atomic<int> known[64][2][2][kClusterMaxCtas + 1][kClusterMaxWarps / 4 + 1][kClusterRingBytes / 4096 + 1];
+    if (device < 0 || device >= 64) return 0;
+    std::atomic<int>& at = known[device][D == 128][gqa][sh.ctas][sh.warps / 4][sh.ring];
+    int n = at.load(std::memory_order_relaxed) - 1;   // 0: not asked yet
+    if (n < 0) {
+        const cudaError_t e =
+            D == 128 ? (gqa ? resident_shape<128, true>(sh, &n) : resident_shape<128, false>(sh, &n))
+                     : (gqa ? resident_shape<64, true>(sh, &n) : resident_shape<64, false>(sh, &n));
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        at.store(n + 1, std::memory_order_relaxed);
+    }
+    return n;
 }
+
+}  // namespace
 
 cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& sh, int units,
-                           const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t st)
+                           const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p,
+                           const LensTable* lens, cudaStream_t st)
 {
-    if (D == 128) return gqa ? launch_shape<128, true>(fused, pdl, sh, units, tk, tv, p, st)
-                             : launch_shape<128, false>(fused, pdl, sh, units, tk, tv, p, st);
-    if (D == 64) return gqa ? launch_shape<64, true>(fused, pdl, sh, units, tk, tv, p, st)
-                            : launch_shape<64, false>(fused, pdl, sh, units, tk, tv, p, st);
+    if (D == 128) return gqa ? launch_shape<128, true>(fused, pdl, sh, units, tk, tv, p, lens, st)
+                             : launch_shape<128, false>(fused, pdl, sh, units, tk, tv, p, lens, st);
+    if (D == 64) return gqa ? launch_shape<64, true>(fused, pdl, sh, units, tk, tv, p, lens, st)
+                            : launch_shape<64, false>(fused, pdl, sh, units, tk, tv, p, lens, st);
     return cudaErrorInvalidValue;
+}
+
+// The line between the two, measured as us per layer of graph-replayed steps
+// (split plan -> clusters).  Clusters save the merge pass and its dependency
+// hop (2.3 us), but cut the rows evenly, without the plan's balancing: they
+// win up to about 45 MB of K/V per layer (LLaVA heads, 800 tokens, B 1 / 2 / 3:
+// 6.5 -> 4.8, 9.2 -> 7.3, 11.2 -> 10.0; B 4, 52 MB: 13.5 -> 13.9; Qwen heads,
+// 1500 tokens, B 2 / 4 / 8: 5.3 -> 3.9, 7.0 -> 4.6, 9.3 -> 6.4; B 16, 46 MB:
+// 10.2 -> 10.4), unless one row is so long that its warps finish far behind
+// the others (Qwen heads, 8 rows of 300 to 3800 tokens, 8 pages per warp:
+// 9.8 -> 7.8; 1 row of 32000, 32 pages per warp: 19.5 -> 21.5).
+//
+// Of the shapes, the one with the most warps per unit whose units all find a
+// slot at once, with a tenth to spare for the next launch's (LLaVA heads,
+// B 3, 96 units: 4 x 4 warps with 2 stages, 110 slots, 10.0; with 3 stages,
+// 74 slots, 13.9), but no more than about a warp per page (8 x 8 against
+// 4 x 4 warps at 7 pages: 10.2 against 3.0).
+ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
+                           int64_t max_pages)
+{
+    constexpr int64_t kMostBytes = 45000000;   // K and V of a layer
+    constexpr int kWarpsOf[][2] = {{8, 8}, {8, 4}, {4, 4}, {2, 4}, {1, 4}};
+    const int64_t units = batch * num_kv_heads;
+    const int64_t stage = 2 * (int64_t)kPageSize * D * 2;
+    const int64_t bytes = pages * num_kv_heads * stage;
+    if (bytes > kMostBytes) return ClusterShape{};
+    for (const auto& cw : kWarpsOf) {
+        ClusterShape sh;
+        sh.ctas = cw[0];
+        sh.warps = cw[1];
+        const int64_t n = (int64_t)sh.ctas * sh.warps;
+        if (n > 4 && (n / 2 >= max_pages || (n == 64 && max_pages <= 128))) continue;
+        const int64_t per_warp = (max_pages + n - 1) / n;
+        const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
+        for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
+            if (10 * (int64_t)resident_clusters(device, D, gqa, sh) < 11 * units) continue;
+            // pages of the longest row's warps against the layer's share of HBM time
+            // the longest row's warps against what the layer's bytes take in
+            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB)
+            return per_warp * (D == 128 ? 4000000 : 2800000) <= 20000000 + bytes ? sh : ClusterShape{};
+        }
+    }
+    return ClusterShape{};
 }
 
 }  // namespace kvd

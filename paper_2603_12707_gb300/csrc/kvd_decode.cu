@@ -9,10 +9,10 @@ namespace kvd {
 
 namespace {
 
-template <int D, bool GQA, bool FUSED>
+template <int D, bool GQA, bool FUSED, class Rows = PlanRows>
 cudaError_t prepare_variant()
 {
-    static cudaError_t status = cudaFuncSetAttribute(decode_kernel<D, GQA, FUSED>,
+    static cudaError_t status = cudaFuncSetAttribute(decode_kernel<D, GQA, FUSED, Rows>,
                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<D, GQA>::kSmem);
     return status;
 }
@@ -26,12 +26,12 @@ cudaError_t variant_info(DecodeVariant* v)
     v->warps = kWarps;
     v->smem_bytes = Geo<D, GQA>::kSmem;
     cudaFuncAttributes a0, a1;
-    e = cudaFuncGetAttributes(&a0, decode_kernel<D, GQA, false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a1, decode_kernel<D, GQA, true>);
+    e = cudaFuncGetAttributes(&a0, decode_kernel<D, GQA, false, PlanRows>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a1, decode_kernel<D, GQA, true, PlanRows>);
     if (e != cudaSuccess) return e;
     v->regs = std::max(a0.numRegs, a1.numRegs);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v->ctas_per_sm, decode_kernel<D, GQA, false>, kWarps * 32,
-                                                         Geo<D, GQA>::kSmem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v->ctas_per_sm, decode_kernel<D, GQA, false, PlanRows>,
+                                                         kWarps * 32, Geo<D, GQA>::kSmem);
 }
 
 template <int D, bool GQA>
@@ -50,11 +50,45 @@ cudaError_t launch_variant(bool fused, bool pdl, int grid, const CUtensorMap& tk
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    return fused ? cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, true>, tk, tv, p)
-                 : cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, false>, tk, tv, p);
+    return fused ? cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, true, PlanRows>, tk, tv, p, PlanRows{})
+                 : cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, false, PlanRows>, tk, tv, p, PlanRows{});
+}
+
+// Batches of up to 64 rows pass a table of 0.6 KB, larger ones 10 KB.
+template <int D, bool GQA, int N>
+cudaError_t launch_table(int grid, const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p,
+                         const RowTable<1024>& all, cudaStream_t st)
+{
+    using Rows = RowTable<N>;
+    if (cudaError_t e = prepare_variant<D, GQA, false, Rows>(); e != cudaSuccess) return e;
+    Rows rows;
+    rows.n = all.n;
+    std::copy_n(all.row, all.n, rows.row);
+    std::copy_n(all.len, all.n, rows.len);
+    std::copy_n(all.off, all.n + 1, rows.off);
+    decode_kernel<D, GQA, false, Rows><<<grid, kWarps * 32, Geo<D, GQA>::kSmem, st>>>(tk, tv, p, rows);
+    return cudaGetLastError();
+}
+
+template <int D, bool GQA>
+cudaError_t launch_table_size(int grid, const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p,
+                              const RowTable<1024>& rows, cudaStream_t st)
+{
+    return rows.n <= kTableRows[0] ? launch_table<D, GQA, kTableRows[0]>(grid, tk, tv, p, rows, st)
+                                   : launch_table<D, GQA, kTableRows[1]>(grid, tk, tv, p, rows, st);
 }
 
 }  // namespace
+
+cudaError_t launch_decode_table(int D, bool gqa, int grid, const CUtensorMap& tk, const CUtensorMap& tv,
+                                const DecodeParams& p, const RowTable<1024>& rows, cudaStream_t st)
+{
+    if (D == 128) return gqa ? launch_table_size<128, true>(grid, tk, tv, p, rows, st)
+                             : launch_table_size<128, false>(grid, tk, tv, p, rows, st);
+    if (D == 64) return gqa ? launch_table_size<64, true>(grid, tk, tv, p, rows, st)
+                            : launch_table_size<64, false>(grid, tk, tv, p, rows, st);
+    return cudaErrorInvalidValue;
+}
 
 cudaError_t decode_variant_info(int D, bool gqa, DecodeVariant* v)
 {

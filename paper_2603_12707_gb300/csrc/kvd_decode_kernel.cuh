@@ -502,10 +502,31 @@ __device__ __forceinline__ void put_new_token(const DecodeParams& p, const PlanE
     __syncwarp();
 }
 
-template <int D, bool GQA, bool FUSED>
+// Entry e of the rows a launch has as parameters.
+template <int N>
+__device__ __forceinline__ PlanEntry find_item(const RowTable<N>& rt, int e)
+{
+    int lo = 0, hi = rt.n - 1;   // the last row with off <= e
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (rt.off[mid] <= e) lo = mid;
+        else hi = mid - 1;
+    }
+    PlanEntry en;
+    en.b = en.seq = rt.row[lo];
+    en.len = rt.len[lo];
+    en.chunk = e - rt.off[lo];
+    en.n_chunks = rt.off[lo + 1] - rt.off[lo];
+    en.slot_base = rt.off[lo];
+    chunk_range((en.len + kPageSize - 1) / kPageSize, en.n_chunks, en.chunk, &en.first_page, &en.n_pages);
+    return en;
+}
+__device__ __forceinline__ PlanEntry find_item(const PlanRows&, int) { return PlanEntry{}; }
+
+template <int D, bool GQA, bool FUSED, class Rows>
 __global__ void __launch_bounds__(kWarps * 32)
     decode_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv,
-                  const DecodeParams p)
+                  const DecodeParams p, const __grid_constant__ Rows rt)
 {
     using Gm = Geo<D, GQA>;
     constexpr int R = Gm::kRing;
@@ -545,6 +566,12 @@ __global__ void __launch_bounds__(kWarps * 32)
     bool waited = false;
     bool first_item = true;
 
+    if constexpr (Rows::kTable) {
+        if (blockIdx.x == 0)
+            for (int i = threadIdx.x; i < rt.n; i += blockDim.x)
+                p.rows_out[rt.row[i]] = make_int2(rt.off[i], rt.off[i + 1] - rt.off[i]);
+    }
+
     // The first item of every warp is its global warp index; later ones come
     // from the work counter, offset by the number of warps.
     const int n_warps = (int)gridDim.x * kWarps;
@@ -557,11 +584,15 @@ __global__ void __launch_bounds__(kWarps * 32)
         // The entry's page ids sit at a fixed stride, so they load alongside
         // the entry.  Windows of 32: lane i holds page w*32 + i of the current
         // window; the next window is fetched 24 pages ahead.
-        const int32_t* pt_row = p.item_pages + (int64_t)e * p.page_stride;
-        auto load_window = [&](int w0) { return (w0 + lane < p.page_stride) ? pt_row[w0 + lane] : 0; };
+        // (a row table: the item's row by binary search, its pages straight
+        // from the page table)
+        const PlanEntry found = find_item(rt, e);
+        const int32_t* pt_row = Rows::kTable ? p.page_table + (int64_t)found.b * p.max_pages + found.first_page
+                                             : p.item_pages + (int64_t)e * p.page_stride;
+        auto load_window = [&](int w0) { return (w0 + lane < (Rows::kTable ? found.n_pages : p.page_stride)) ? pt_row[w0 + lane] : 0; };
         int32_t pid_cur = load_window(0);
         int32_t pid_next = 0;
-        const PlanEntry en = p.plan[e];
+        const PlanEntry en = Rows::kTable ? found : p.plan[e];
         const int np = en.n_pages;
 
         auto issue = [&](int j, int s) {
@@ -647,7 +678,9 @@ __global__ void __launch_bounds__(kWarps * 32)
             pending &= ~(1u << s);
             if (GQA && j == 0) comp.ready(lane);
             const int valid = min(kPageSize, en.len - (en.first_page + j) * kPageSize);
-            uint8_t* sK = ring + s * STAGE;
+            const int k_off = Rows::kTable && p.kv_map == 2 ? TILE : 0;   // the stage's K tile, and V's from there
+            const int v_off = k_off ? -TILE : TILE;
+            uint8_t* sK = ring + s * STAGE + k_off;
             // Generic-proxy writes into the stage (the new token's row) must be
             // ordered before the next TMA write to it; plain reads need no
             // fence (their values are consumed first).
@@ -656,11 +689,12 @@ __global__ void __launch_bounds__(kWarps * 32)
                 // the issue side has not moved past this page's id window
                 if (last_chunk && j == np - 1) {
                     int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
-                    put_new_token<D>(p, en, g, pid, new_kv, sK, sK + TILE, lane);
+                    put_new_token<D>(p, en, g, pid, new_kv, sK, sK + v_off, lane);
                     wrote = true;
                 }
             }
-            comp.page(sK, sK + TILE, ring_s + s * STAGE, ring_s + s * STAGE + TILE, valid, p.scale_log2, lane);
+            const uint32_t sk = ring_s + s * STAGE + k_off;
+            comp.page(sK, sK + v_off, sk, sk + v_off, valid, p.scale_log2, lane);
             if (wrote) fence_proxy_async_smem();
             __syncwarp();
             if (j + R < np) {
@@ -670,6 +704,8 @@ __global__ void __launch_bounds__(kWarps * 32)
         }
         if (!ok) break;
         comp.finish(p, en, g, lane);
+        if constexpr (Rows::kTable)
+            if (n_items <= n_warps) break;   // every item was some warp's first
         if (lane == 0) item = n_warps + (int)atomicAdd(&p.queue[0], 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
     }

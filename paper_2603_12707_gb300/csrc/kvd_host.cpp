@@ -144,7 +144,6 @@ struct kv_cache {
     int64_t dev_pages = 0;                      // pages held then (0: nothing known)
     int32_t dev_seqs = 0;                       // sequences holding them
     bool dev_split_override = false;
-    int cluster_resident[9][3][7];              // resident_clusters by [ctas][warps / 4][ring], -1: not asked yet
 
     int32_t* page_table() const { return meta; }
     int32_t* seq_len_dev() const { return meta + (int64_t)cfg.max_seqs * cfg.max_pages_per_seq; }
@@ -221,62 +220,6 @@ int32_t chunk_cap(const kv_cache* c, int64_t rows, int64_t max_pages, int32_t T)
     const bool few_units = rows * c->cfg.num_kv_heads * kChunkCap < warps;
     if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
     return c->group > 1 ? kChunkCapGqa : kChunkCap;
-}
-
-// Clusters of `shape` that the GPU holds at once (asked once per shape).
-int resident_clusters(kv_cache* c, const ClusterShape& sh)
-{
-    int& known = c->cluster_resident[sh.ctas][sh.warps / 4][sh.ring];
-    if (known < 0 && cluster_resident(c->cfg.head_dim, c->group > 1, sh, &known) != cudaSuccess) {
-        cudaGetLastError();
-        known = 0;
-    }
-    return known;
-}
-
-// Clusters for a step of `batch` rows that hold `pages` pages per KV head in
-// all and at most max_pages in one row, or ctas == 0: the split plan.
-//
-// The line between the two, measured as us per layer of graph-replayed steps
-// (split plan -> clusters).  Clusters save the merge pass and its dependency
-// hop (2.3 us), but cut the rows evenly, without the plan's balancing: they
-// win up to about 45 MB of K/V per layer (LLaVA heads, 800 tokens, B 1 / 2 / 3:
-// 6.5 -> 4.8, 9.2 -> 7.3, 11.2 -> 10.0; B 4, 52 MB: 13.5 -> 13.9; Qwen heads,
-// 1500 tokens, B 2 / 4 / 8: 5.3 -> 3.9, 7.0 -> 4.6, 9.3 -> 6.4; B 16, 46 MB:
-// 10.2 -> 10.4), unless one row is so long that its warps finish far behind
-// the others (Qwen heads, 8 rows of 300 to 3800 tokens, 8 pages per warp:
-// 9.8 -> 7.8; 1 row of 32000, 32 pages per warp: 19.5 -> 21.5).
-//
-// Of the shapes, the one with the most warps per unit whose units all find a
-// slot at once, with a tenth to spare for the next launch's (LLaVA heads,
-// B 3, 96 units: 4 x 4 warps with 2 stages, 110 slots, 10.0; with 3 stages,
-// 74 slots, 13.9), but no more than about a warp per page (8 x 8 against
-// 4 x 4 warps at 7 pages: 10.2 against 3.0).
-ClusterShape cluster_shape(kv_cache* c, int32_t batch, int64_t pages, int64_t max_pages)
-{
-    constexpr int64_t kMostBytes = 45000000;   // K and V of a layer
-    constexpr int kWarpsOf[][2] = {{8, 8}, {8, 4}, {4, 4}, {2, 4}, {1, 4}};
-    const int64_t units = (int64_t)batch * c->cfg.num_kv_heads;
-    const int64_t stage = 2 * (int64_t)kPageSize * c->cfg.head_dim * 2;
-    const int64_t bytes = pages * c->cfg.num_kv_heads * stage;
-    if (bytes > kMostBytes) return ClusterShape{};
-    for (const auto& cw : kWarpsOf) {
-        ClusterShape sh;
-        sh.ctas = cw[0];
-        sh.warps = cw[1];
-        const int64_t n = (int64_t)sh.ctas * sh.warps;
-        if (n > 4 && (n / 2 >= max_pages || (n == 64 && max_pages <= 128))) continue;
-        const int64_t per_warp = (max_pages + n - 1) / n;
-        const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
-        for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
-            if (10 * (int64_t)resident_clusters(c, sh) < 11 * units) continue;
-            // pages of the longest row's warps against the layer's share of HBM time
-            // the longest row's warps against what the layer's bytes take in
-            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB)
-            return per_warp * (c->cfg.head_dim == 128 ? 4000000 : 2800000) <= 20000000 + bytes ? sh : ClusterShape{};
-        }
-    }
-    return ClusterShape{};
 }
 
 int grow_scratch(kv_cache* c, int64_t entries, int64_t slots, int64_t page_ids, cudaStream_t st)
@@ -429,7 +372,6 @@ int kv_cache_create(const kvc_config* cfg, void* stream, kv_cache** out)
     if (k.flags & ~KVC_FLAG_HOST_ONLY) return fail(KVC_ERR_INVALID, "kv_cache_create: unknown flag");
 
     kv_cache* c = new kv_cache();
-    std::fill(&c->cluster_resident[0][0][0], &c->cluster_resident[0][0][0] + sizeof(c->cluster_resident) / sizeof(int), -1);
     c->cfg = k;
     c->host_only = (k.flags & KVC_FLAG_HOST_ONLY) != 0;
     c->group = k.num_q_heads / k.num_kv_heads;
@@ -862,7 +804,8 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
     const int32_t max_np = *std::max_element(np_after.begin(), np_after.end());
     ClusterShape shape;
     if (!c->split_override && !c->host_only)
-        shape = cluster_shape(c, batch, total_units / c->cfg.num_kv_heads, max_np);
+        shape = cluster_shape(c->device, c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, batch,
+                              total_units / c->cfg.num_kv_heads, max_np);
     const int32_t cap = chunk_cap(c, batch, max_np, T);
     int64_t entries = 0;
     int32_t stride = 1;
@@ -1009,6 +952,8 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     p.part_o = c->part_o;
     p.part_ml = c->part_ml;
     p.rows = c->rows;
+    p.rows_out = nullptr;
+    p.rows_late = 0;
     p.item_pages = c->item_pages;
     p.page_stride = c->page_stride;
     p.n_entries_dev = c->step_dev ? c->d_small + 1 : nullptr;
@@ -1049,7 +994,7 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
         c->last_stream = static_cast<cudaStream_t>(stream);
         KVD_CUDA(launch_cluster(c->cfg.head_dim, c->group > 1, fused, pdl, c->step_cluster,
                                 batch * c->cfg.num_kv_heads, c->tmaps[layer], c->tmaps[layer], p,
-                                static_cast<cudaStream_t>(stream)));
+                                nullptr, static_cast<cudaStream_t>(stream)));
         ++c->launches;
         c->prev_merge = false;
         c->chain_launches = c->launches;
@@ -1185,7 +1130,7 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     if (!c->dev_split_override) {
         const int64_t row = c->dev_seqs ? c->dev_row_pages + 1 : c->cfg.max_pages_per_seq;
         const int64_t pages = c->dev_seqs ? (c->dev_pages * batch + c->dev_seqs - 1) / c->dev_seqs : row * batch;
-        shape = cluster_shape(c, batch, pages, row);
+        shape = cluster_shape(c->device, c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, batch, pages, row);
     }
     a.no_plan = shape.ctas ? 1 : 0;
     c->last_stream = st;

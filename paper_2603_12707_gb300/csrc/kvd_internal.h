@@ -43,6 +43,31 @@ __host__ __device__ inline int row_item_pages(int T, int i, int n)
     return T;
 }
 
+// The rows of a call as kernel parameters, for a caller whose lengths are on
+// the host: the split pass finds an item's row by a binary search instead of
+// reading a plan that a kernel before it wrote.  Rows stand in planning order
+// (longest first, so the rows of several items come before the others and
+// their entries number the partial slots too).
+template <int N>
+struct RowTable {
+    static constexpr bool kTable = true;
+    int32_t n;
+    uint16_t row[N];     // batch row
+    int32_t len[N];      // tokens attended
+    int32_t off[N + 1];  // first entry of the row; off[n] = entries
+};
+struct PlanRows {        // rows and items come from the step's plan
+    static constexpr bool kTable = false;
+};
+constexpr int kTableRows[2] = {64, 1024};
+
+// The same for clusters: the length of each batch row.
+constexpr int kLensRows = 320;
+struct LensTable {
+    static constexpr bool kTable = true;
+    int32_t len[kLensRows];
+};
+
 // Split policy shared by host and device.  A row of np pages is cut into
 // nch items of near-equal size: the target size T, raised for long rows so a
 // row never has more than `cap` items (which bounds the merge).
@@ -194,6 +219,8 @@ struct DecodeParams {
     const PlanEntry* plan;
     float* part_o;            // [slots][G][D]
     float2* part_ml;          // [slots][G]  (running max in log2 units, sum)
+    int2* rows_out;           // RowTable launches: the split pass writes `rows` for its merge pass
+    int32_t rows_late;        // 1: the merge pass may read `rows` only after its dependency wait
     const int2* rows;         // [batch]: (first partial slot, items) per batch row; for clusters (sequence, tokens)
     const int32_t* item_pages;// [entries][page_stride]: page ids of each plan entry's pages
     int32_t page_stride;
@@ -213,8 +240,8 @@ struct DecodeParams {
     const uint16_t* v_new;
     uint16_t* pool_k;         // this layer's pools [num_pages][H_kv][P][D]
     uint16_t* pool_v;
-    // 1: the first tensor map covers K and V (one 4-D load per page); 0: two
-    // 3-D maps, K and V.
+    // 1: the first tensor map covers K and V (one 4-D load per page), 2: V
+    // and K in that order; 0: two 3-D maps, K and V.
     int32_t kv_map;
     // Early start of a chained launch: the merge pass of each launch writes
     // step * 65536 + tag into every SM's word of start_flags (one word per
@@ -256,12 +283,6 @@ cudaError_t launch_scatter_i32(int32_t* base, const ScatterI32& s, cudaStream_t 
 cudaError_t launch_step(const StepPatch& patch, const PlanArgs& plan, cudaStream_t st);
 cudaError_t launch_token_copy(const TokenCopyArgs& a, cudaStream_t st);
 cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, cudaStream_t st);
-// Copy each plan entry's page ids from the page table into item_pages
-// ([entries][stride]), so the decode kernel reads them alongside the entry.
-// entries_dev (if non-null) holds the entry count; `entries` is then its bound.
-cudaError_t launch_gather_pages(const PlanEntry* plan, int32_t entries, const int32_t* entries_dev,
-                                const int32_t* page_table, int32_t max_pages, int32_t* item_pages, int32_t stride,
-                                int num_sms, cudaStream_t st);
 cudaError_t launch_step_device(const StepDevArgs& a, cudaStream_t st);
 cudaError_t launch_seq_op(const SeqOpArgs& a, cudaStream_t st);
 // pdl: launched with programmatic dependent launch (it waits for the kernel
@@ -297,8 +318,17 @@ cudaError_t launch_decode(int D, bool gqa, bool fused, bool pdl, int grid, const
                           const DecodeParams& p, cudaStream_t st);
 // Decode attention with one cluster per (row, KV head) unit, no second pass
 // (kvd_cluster.cu).  pdl: launched with programmatic dependent launch.
-cudaError_t cluster_resident(int D, bool gqa, const ClusterShape& shape, int* clusters);   // clusters the GPU holds
+// lens: the rows' lengths as parameters (batch <= kLensRows), or null: p.rows.
 cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& shape, int units,
-                           const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t st);
+                           const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p,
+                           const LensTable* lens, cudaStream_t st);
+// Clusters for `batch` rows of num_kv_heads that hold `pages` pages per KV
+// head in all and at most max_pages in one row, or ctas == 0: the split plan.
+ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
+                           int64_t max_pages);
+// The split pass over rows given as parameters (no append, an ordinary
+// launch): p.rows is written for the merge pass, p.item_pages is not used.
+cudaError_t launch_decode_table(int D, bool gqa, int grid, const CUtensorMap& tk, const CUtensorMap& tv,
+                                const DecodeParams& p, const RowTable<1024>& rows, cudaStream_t st);
 
 }  // namespace kvd

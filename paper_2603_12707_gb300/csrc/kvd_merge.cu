@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const DecodePar
     const int total = p.batch * p.H_q * kMergeSplit;
     int w = blockIdx.x * kMergeWarps + (threadIdx.x >> 5);
     int2 row = make_int2(0, 0);
-    if (w < total) row = p.rows[(w / kMergeSplit) / p.H_q];
+    if (w < total && !p.rows_late) row = p.rows[(w / kMergeSplit) / p.H_q];
     if (pdl) {
         griddep_launch_dependents();   // the next layer may start streaming now
         griddep_wait();                // the split pass of this layer is complete
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const DecodePar
         const int part = w % kMergeSplit;
         const int bh = w / kMergeSplit;
         const int b = bh / p.H_q, h = bh - b * p.H_q;
-        if (!first) row = p.rows[b];
+        if (!first || p.rows_late) row = p.rows[b];
         if (row.y <= 1) continue;
         const int g = h / p.G;
         merge_unit<D, BATCH>(p, row, b, g, h - g * p.G, part, lane);
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kWideWarps * 32) merge_wide_kernel(const Decod
     const int total = p.batch * p.H_q;
     int u = blockIdx.x;
     int2 row = make_int2(0, 0);
-    if (u < total) row = p.rows[u / p.H_q];
+    if (u < total && !p.rows_late) row = p.rows[u / p.H_q];
     if (pdl) {
         griddep_launch_dependents();   // the next layer may start streaming now
         griddep_wait();                // the split pass of this layer is complete
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kWideWarps * 32) merge_wide_kernel(const Decod
     }
     for (bool first = true; u < total; u += gridDim.x, first = false) {
         const int b = u / p.H_q, h = u - b * p.H_q;
-        if (!first) row = p.rows[b];
+        if (!first || p.rows_late) row = p.rows[b];
         if (row.y <= 1) continue;      // the same for every warp of the CTA
         const int g = h / p.G, hh = h - g * p.G;
         const int c0 = wid * kWideItems;

@@ -10,15 +10,26 @@
 // not take the allocator's locks.  Those callers own the K/V pools and page
 // table themselves and call this entry point instead.
 //
-// Scratch.  The split plan, the per-item partial results, the per-row merge
-// table and the work counters live in one file-scope __device__ array of
+// Launches.  Everything that a plan would say follows from the lengths, which
+// are on the host: they go to the kernels as parameters (RowTable, LensTable)
+// and the page ids come straight from the caller's table, so a call is the
+// split pass and its merge pass, or one cluster launch for a small batch.
+// (A plan kernel with 20 KB of parameters and a page-list kernel before the
+// split pass, two loads per page, the merge pass as an ordinary launch and
+// five device queries per call measured 41 us a call on the Qwen-shaped
+// batch, 34 us of it on the host.)  The first launch is an ordinary one: what
+// ran before the call may have written the pools and the page table.
+//
+// Scratch.  The per-item partial results, the per-row merge table and the
+// work counter live in one file-scope __device__ array of
 // kNoAllocScratchBytes (16 MiB) that every GPU loading this library holds
 // until the process exits.  Host code cannot use the array's name as a device
 // address; the first call on each device looks the address up with
 // cudaGetSymbolAddress (make that first call before any stream capture) and
 // later calls reuse it.  Every call shares the array and leaves its contents
-// behind, so each call clears the counters it needs before use, and calls
-// that overlap on the GPU (different streams, no ordering) race on it.
+// behind, but for the work counter, which is zero before and after each call
+// (the merge pass, or a memset where there is none, puts it back); calls that
+// overlap on the GPU (different streams, no ordering) race on the array.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -37,40 +48,6 @@ constexpr int kNoAllocMaxBatch = 1024;
 
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocScratchBytes];
 
-struct NoAllocPlanArgs {
-    int32_t batch;
-    PlanEntry* plan;
-    int2* rows;            // [batch]: (first partial slot, items)
-    uint32_t* queue;
-    int32_t* err;
-    int32_t clear_err;
-    // rows in planning order (longest first)
-    int32_t row[kNoAllocMaxBatch];   // batch row
-    int32_t len[kNoAllocMaxBatch];   // tokens attended
-    int32_t off[kNoAllocMaxBatch];   // first plan entry of the row
-    int32_t nch[kNoAllocMaxBatch];   // items of the row
-    int32_t slot[kNoAllocMaxBatch];  // first partial slot (rows with one item use none)
-};
-
-// One block: clear the work counters, then write each row's items
-// (near-equal page ranges) at the offsets the host computed.
-__global__ void __launch_bounds__(1024) noalloc_plan_kernel(const __grid_constant__ NoAllocPlanArgs a)
-{
-    if (threadIdx.x == 0) {
-        a.queue[0] = 0;
-        if (a.clear_err) *a.err = 0;
-    }
-    for (int i = threadIdx.x; i < a.batch; i += blockDim.x) {
-        const int np = (a.len[i] + kPageSize - 1) / kPageSize;
-        for (int c = 0; c < a.nch[i]; ++c) {
-            int first, n;
-            chunk_range(np, a.nch[i], c, &first, &n);
-            a.plan[a.off[i] + c] = PlanEntry{a.row[i], a.row[i], a.len[i], first, n, c, a.nch[i], a.slot[i]};
-        }
-        a.rows[a.row[i]] = make_int2(a.slot[i], a.nch[i]);
-    }
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 encoder()
 {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -86,29 +63,38 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder()
     return fn;
 }
 
-// Device address of the scratch array on the current device, looked up once.
-int scratch_address(uint8_t** out)
+// What a call needs to know of the current device, asked once per device:
+// the address of the scratch array and the split pass's variants.
+struct DeviceInfo {
+    uint8_t* scratch = nullptr;
+    int num_sms = 0;
+    DecodeVariant var[2][2];   // [D == 128][GQA]
+};
+
+int device_info(int* device, const DeviceInfo** out)
 {
     static std::mutex mu;
-    static uint8_t* addr[64] = {};
+    static DeviceInfo info[64];
+    auto err = [](const char* what, cudaError_t e) {
+        set_last_error((std::string("decode_attention_noalloc: ") + what + ": " + cudaGetErrorString(e)).c_str());
+        return KVC_ERR_CUDA;
+    };
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || dev < 0 || dev >= 64) {
-        set_last_error((std::string("decode_attention_noalloc: cudaGetDevice: ") + cudaGetErrorString(e)).c_str());
-        return KVC_ERR_CUDA;
-    }
+    if (e != cudaSuccess || dev < 0 || dev >= 64) return err("cudaGetDevice", e);
     std::lock_guard<std::mutex> lock(mu);
-    if (!addr[dev]) {
+    DeviceInfo& d = info[dev];
+    if (!d.scratch) {
+        e = cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev);
+        for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = decode_variant_info(i & 2 ? 128 : 64, i & 1, &d.var[i >> 1][i & 1]);
+        if (e != cudaSuccess) return err("cannot query the current device", e);
         void* p = nullptr;
         e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-        if (e != cudaSuccess || !p) {
-            set_last_error(
-                (std::string("decode_attention_noalloc: cudaGetSymbolAddress: ") + cudaGetErrorString(e)).c_str());
-            return KVC_ERR_CUDA;
-        }
-        addr[dev] = static_cast<uint8_t*>(p);
+        if (e != cudaSuccess || !p) return err("cudaGetSymbolAddress", e);
+        d.scratch = static_cast<uint8_t*>(p);
     }
-    *out = addr[dev];
+    *device = dev;
+    *out = &d;
     return KVC_OK;
 }
 
@@ -155,131 +141,150 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
     int dev = 0;
-    DecodeVariant var{};
-    int num_sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess)
-        return fail(KVC_ERR_CUDA, "cannot query the current device");
-    if (cudaError_t e = decode_variant_info(head_dim, G > 1, &var); e != cudaSuccess)
-        return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
-    uint8_t* scratch = nullptr;
-    if (int rc = scratch_address(&scratch)) return rc;
+    const DeviceInfo* info = nullptr;
+    if (int rc = device_info(&dev, &info)) return rc;
+    const DecodeVariant& var = info->var[head_dim == 128][G > 1];
+    const int num_sms = info->num_sms;
+    uint8_t* const scratch = info->scratch;
 
     // Items: the library's usual target (about three per resident warp),
-    // enlarged until the plan and the partials fit the static scratch.
+    // enlarged until a plan (an entry and its page ids per item) and the
+    // partials fit the static scratch: the documented limit.
     const int64_t warps = (int64_t)num_sms * std::max(1, var.ctas_per_sm) * std::max(1, var.warps);
-    int64_t T = std::min<int64_t>(128, std::max<int64_t>(2, (total_pages * num_kv_heads + 3 * warps - 1) / (3 * warps)));
-    int64_t entries = 0;
-    bool split_rows = false;
-    int stride = 1;
-    size_t off_pages = 0, off_o = 0, off_ml = 0, off_rows = 0, off_q = 0, off_err = 0, need = 0;
+    const int64_t units = total_pages * num_kv_heads;
+    auto target = [&](int64_t per_warp) {
+        return std::min<int64_t>(128, std::max<int64_t>(2, (units + per_warp * warps - 1) / (per_warp * warps)));
+    };
+    const size_t partial = (size_t)num_kv_heads * G * (head_dim * sizeof(float) + sizeof(float2));   // per entry
+    int64_t T = target(3);
+    size_t need = 0;
+    int max_np = 0;
     // T doubles, clamped to kMaxItemPages; the attempt at kMaxItemPages is the last.
     for (;; T = std::min<int64_t>(2 * T, kMaxItemPages)) {
-        entries = 0;
-        int64_t split_items = 0;   // only rows cut into several items keep partials
-        for (int b = 0; b < batch; ++b) {
-            const int64_t nch = row_chunks((lens[b] + kPageSize - 1) / kPageSize, (int)T);
-            entries += nch;
-            if (nch > 1) split_items += nch;
-        }
-        split_rows = split_items > 0;
-        const int64_t slots = split_items * num_kv_heads;
-        stride = 1;
+        int64_t entries = 0, split_items = 0;   // only rows cut into several items keep partials
+        int stride = 1;
         for (int b = 0; b < batch; ++b) {
             const int np = (lens[b] + kPageSize - 1) / kPageSize;
             const int nch = row_chunks(np, (int)T);
+            entries += nch;
+            if (nch > 1) split_items += nch;
             stride = std::max(stride, (np + nch - 1) / nch);
+            max_np = std::max(max_np, np);
         }
-        off_pages = round256((size_t)entries * sizeof(PlanEntry));
-        off_o = round256(off_pages + (size_t)entries * stride * sizeof(int32_t));
-        off_ml = round256(off_o + (size_t)slots * G * head_dim * sizeof(float));
-        off_rows = round256(off_ml + (size_t)slots * G * sizeof(float2));
-        off_q = round256(off_rows + (size_t)batch * sizeof(int2));
-        off_err = off_q + 2 * sizeof(uint32_t);
-        need = round256(off_err + sizeof(int32_t));
+        const size_t off_pages = round256((size_t)entries * sizeof(PlanEntry));
+        const size_t off_o = round256(off_pages + (size_t)entries * stride * sizeof(int32_t));
+        const size_t slots = (size_t)split_items * num_kv_heads;
+        const size_t off_ml = round256(off_o + slots * G * head_dim * sizeof(float));
+        const size_t off_rows = round256(off_ml + slots * G * sizeof(float2));
+        need = round256(round256(off_rows + (size_t)batch * sizeof(int2)) + 3 * sizeof(uint32_t));
         if (need <= kNoAllocScratchBytes || T >= kMaxItemPages) break;
     }
     if (need > kNoAllocScratchBytes)
         return fail(KVC_ERR_UNSUPPORTED, ("the batch needs " + std::to_string(need) +
                                           " bytes of scratch; the static limit is 16 MiB").c_str());
 
+    // One tensor map over both pools (one load per page), the lower one first,
+    // where their distance is a whole number of 128-byte lines; else a map for
+    // each.
     auto encode = encoder();
     if (!encode) return fail(KVC_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
     CUtensorMap maps[2];
-    for (int kv = 0; kv < 2; ++kv) {
+    const int64_t rows = num_pages * num_kv_heads * kPageSize;
+    const int64_t apart = static_cast<const char*>(v_pool) - static_cast<const char*>(k_pool);
+    int kv_map = 0;
+    if (apart != 0 && apart % 128 == 0 && std::abs(apart) < (int64_t)1 << 40 &&
+        encode_tile_map(reinterpret_cast<void*>(encode), &maps[0], const_cast<void*>(apart > 0 ? k_pool : v_pool), rows,
+                        head_dim, std::abs(apart)) == CUDA_SUCCESS) {
+        kv_map = apart > 0 ? 1 : 2;
+        maps[1] = maps[0];
+    }
+    for (int kv = 0; kv < 2 && !kv_map; ++kv) {
         CUresult r = encode_tile_map(reinterpret_cast<void*>(encode), &maps[kv], const_cast<void*>(kv ? v_pool : k_pool),
-                                     num_pages * num_kv_heads * kPageSize, head_dim, 0);
+                                     rows, head_dim, 0);
         if (r != CUDA_SUCCESS) return fail(KVC_ERR_INVALID, "cuTensorMapEncodeTiled rejected the pools");
     }
 
-    NoAllocPlanArgs pa;
-    pa.batch = batch;
-    pa.plan = reinterpret_cast<PlanEntry*>(scratch);
-    pa.rows = reinterpret_cast<int2*>(scratch + off_rows);
-    pa.queue = reinterpret_cast<uint32_t*>(scratch + off_q);
-    pa.err = device_error ? device_error : reinterpret_cast<int32_t*>(scratch + off_err);
-    pa.clear_err = device_error ? 0 : 1;
-    {
-        for (int b = 0; b < batch; ++b) pa.row[b] = b;
-        std::stable_sort(pa.row, pa.row + batch, [&](int32_t x, int32_t y) { return lens[x] > lens[y]; });
-        int32_t off = 0, slot = 0;
-        for (int i = 0; i < batch; ++i) {
-            const int32_t b = pa.row[i];
-            const int32_t nch = row_chunks((lens[b] + kPageSize - 1) / kPageSize, (int)T);
-            pa.len[i] = lens[b];
-            pa.off[i] = off;
-            pa.nch[i] = nch;
-            pa.slot[i] = slot;
-            off += nch;
-            if (nch > 1) slot += nch;
-        }
-    }
-    noalloc_plan_kernel<<<1, 1024, 0, st>>>(pa);
-    if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
-    int32_t* item_pages = reinterpret_cast<int32_t*>(scratch + off_pages);
-    if (cudaError_t e = launch_gather_pages(pa.plan, (int32_t)entries, nullptr, page_table, max_pages, item_pages, stride,
-                                            num_sms, st);
-        e != cudaSuccess)
-        return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
-
     const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt((float)head_dim);
-    DecodeParams p;
+    // The scratch: [work counter, error word], the merge table, the partials.
+    const size_t off_rows = 256, off_part = round256(off_rows + (size_t)batch * sizeof(int2));
+    DecodeParams p{};
     p.q = static_cast<const uint16_t*>(q);
     p.out = static_cast<uint16_t*>(out);
     p.page_table = page_table;
-    p.plan = pa.plan;
-    p.part_o = reinterpret_cast<float*>(scratch + off_o);
-    p.part_ml = reinterpret_cast<float2*>(scratch + off_ml);
-    p.rows = pa.rows;
-    p.item_pages = item_pages;
-    p.page_stride = stride;
-    p.n_entries_dev = nullptr;
+    p.rows_out = reinterpret_cast<int2*>(scratch + off_rows);
+    p.rows = p.rows_out;
+    p.rows_late = 1;
     p.batch = batch;
-    p.queue = pa.queue;
-    p.queue_next = nullptr;
-    p.err = pa.err;
+    p.queue = reinterpret_cast<uint32_t*>(scratch);
+    p.err = device_error ? device_error : reinterpret_cast<int32_t*>(scratch) + 1;
     p.num_pages = num_pages;
-    p.n_items = (int32_t)(entries * num_kv_heads);
     p.H_kv = num_kv_heads;
     p.H_q = num_q_heads;
     p.G = G;
     p.max_pages = max_pages;
     p.scale_log2 = scale * 1.4426950408889634f;
-    p.kv_map = 0;
-    p.start_flags = nullptr;
-    p.step_no = nullptr;
-    p.tag = p.prev_tag = 0;
+    p.kv_map = kv_map;
     p.num_sms = num_sms;
-    p.hold_last = 0;
-    p.k_new = p.v_new = nullptr;
-    p.pool_k = p.pool_v = nullptr;
-    const int64_t resident = (int64_t)num_sms * std::max(1, var.ctas_per_sm);
-    const int64_t want = (p.n_items + var.warps - 1) / var.warps;
-    const int grid = (int)std::max<int64_t>(1, std::min(resident, want));
-    if (cudaError_t e = launch_decode(head_dim, G > 1, false, false, grid, maps[0], maps[1], p, st); e != cudaSuccess)
-        return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
-    if (split_rows)
-        if (cudaError_t e = launch_merge(head_dim, false, kChunkCap, num_sms, 0, p, st); e != cudaSuccess)
+
+    const ClusterShape shape = cluster_shape(dev, head_dim, G > 1, num_kv_heads, batch, total_pages, max_np);
+    if (shape.ctas && batch <= kLensRows) {
+        LensTable lt;
+        std::copy_n(lens, batch, lt.len);
+        p.ring = shape.ring;
+        if (cudaError_t e = launch_cluster(head_dim, G > 1, false, false, shape, batch * num_kv_heads, maps[0], maps[1], p,
+                                           &lt, st);
+            e != cudaSuccess)
             return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
+        return KVC_OK;
+    }
+
+    // Rows in planning order, longest first.
+    RowTable<kNoAllocMaxBatch> rt;
+    rt.n = batch;
+    for (int b = 0; b < batch; ++b) rt.row[b] = (uint16_t)b;
+    std::stable_sort(rt.row, rt.row + batch, [&](uint16_t x, uint16_t y) { return lens[x] > lens[y]; });
+    for (int i = 0; i < batch; ++i) rt.len[i] = lens[rt.row[i]];
+    // The plan of a step of the cache (items per resident warp, graduated
+    // sizes, items per row) where its partials fit, else the one sized above
+    // (whose rows of one item come last and keep no partial).
+    int max_chunks = 1;
+    int64_t split_end = 0;   // entries up to the last row of several items: those with partial slots
+    auto cut = [&](int64_t size, int cap, bool graduated) {
+        int32_t off = 0;
+        split_end = 0;
+        max_chunks = 1;
+        for (int i = 0; i < batch; ++i) {
+            const int np = (rt.len[i] + kPageSize - 1) / kPageSize;
+            const int nch = row_chunks(np, graduated ? row_item_pages((int)size, i, batch) : (int)size, cap);
+            rt.off[i] = off;
+            off += nch;
+            if (nch > 1) split_end = off;
+            max_chunks = std::max(max_chunks, nch);
+        }
+        rt.off[batch] = off;
+        return off_part + (size_t)split_end * partial + 512 <= kNoAllocScratchBytes;
+    };
+    const int64_t T_step = std::max(T, target(G > 1 ? 2 : 3));
+    if (!cut(T_step, G > 1 ? kChunkCapGqa : kChunkCap, true) && !cut(T, kChunkCap, false))
+        return fail(KVC_ERR_UNSUPPORTED, "the batch does not fit the static scratch");
+    const int32_t entries = rt.off[batch];
+    p.part_o = reinterpret_cast<float*>(scratch + off_part);
+    p.part_ml = reinterpret_cast<float2*>(
+        scratch + round256(off_part + (size_t)split_end * num_kv_heads * G * head_dim * sizeof(float)));
+    p.n_items = entries * num_kv_heads;
+    const int64_t resident = (int64_t)num_sms * std::max(1, var.ctas_per_sm);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(resident, p.n_items));
+    if (cudaError_t e = launch_decode_table(head_dim, G > 1, grid, maps[0], maps[1], p, rt, st); e != cudaSuccess)
+        return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
+    cudaError_t e = cudaSuccess;
+    if (max_chunks > 1) {
+        const int split_regs = ((var.ctas_per_sm * var.warps + 3) / 4) * warp_register_allocation(var.regs);
+        e = launch_merge(head_dim, true, max_chunks, num_sms, split_regs, p, st);
+    }
+    if ((max_chunks == 1 && p.n_items > grid) || e != cudaSuccess) {
+        const cudaError_t m = cudaMemsetAsync(p.queue, 0, sizeof(uint32_t), st);   // (a memset: it allocates nothing)
+        if (e == cudaSuccess) e = m;
+    }
+    if (e != cudaSuccess) return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
     return KVC_OK;
 }

@@ -201,3 +201,50 @@ def test_noalloc_rejects_what_does_not_fit(kvlib):
         kd.decode_attention_noalloc(kp, vp, sess.num_pages, 32, 32, 128, pt, sess.max_pages, [4, 4], q[:1], out)
     t.close()
 
+
+
+@pytest.mark.parametrize("layout", ["k_first", "v_first", "apart_by_16_bytes"])
+@pytest.mark.parametrize("Hq,Hkv,d,B,longest", [
+    (14, 2, 64, 5, 300),      # clusters
+    (6, 6, 128, 3, 500),
+    (12, 12, 128, 30, 700),   # split pass and merge pass, rows in the small table
+    (28, 4, 128, 70, 900),    # the large table
+    (8, 8, 64, 200, 32),      # more items than warps, no row split: no merge pass
+])
+def test_noalloc_pool_layouts_and_row_tables(kvlib, Hq, Hkv, d, B, longest, layout):
+    """K and V pools in either order (one tensor map over both) and at a
+    distance that is no multiple of 128 bytes (a map for each); batches that
+    run as clusters, with and without a merge pass, in both table sizes;
+    three calls in a row, so each leaves the work counter as it found it."""
+    rng = np.random.default_rng(Hq + B)
+    lens = [int(n) for n in rng.integers(1, longest + 1, size=B)]
+    lens[0], lens[-1] = longest, 1
+    need = [(n + 15) // 16 for n in lens]
+    pages, width = sum(need) + 3, max(need) + 1
+    table = np.full((B, width), -1, np.int32)
+    order = rng.permutation(pages)
+    at = 0
+    for b, n in enumerate(need):
+        table[b, :n] = order[at:at + n]
+        at += n
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    n = pages * Hkv * 16 * d
+    buf = torch.randn(2 * n + 64, generator=gen, device="cuda").bfloat16()
+    lo, hi = buf[:n], buf[n + (8 if layout == "apart_by_16_bytes" else 0):][:n]
+    k, v = (hi, lo) if layout == "v_first" else (lo, hi)
+    q = torch.randn((B, Hq, d), generator=gen, device="cuda").bfloat16()
+    pt = torch.from_numpy(table).cuda()
+    outs = []
+    for _ in range(3):
+        out = torch.empty_like(q)
+        kd.decode_attention_noalloc(k, v, pages, Hq, Hkv, d, pt, width, lens, q, out)
+        outs.append(out)
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    kh, vh = (u16(x).reshape(pages, Hkv, 16, d).transpose(0, 2, 1, 3) for x in (k, v))
+    rows = sorted({0, 1, B // 2, B - 1})
+    kk = [kh[table[b, :need[b]]].reshape(-1, Hkv, d)[:lens[b]] for b in rows]
+    vv = [vh[table[b, :need[b]]].reshape(-1, Hkv, d)[:lens[b]] for b in rows]
+    ref = oracle.decode_attention(u16(q)[rows], [lens[b] for b in rows], np.concatenate(kk), np.concatenate(vv))
+    vmax = np.array([np.abs(oracle.bf16_to_f64(x)).max() for x in vv])
+    assert_close(bf16_to_f64(outs[0])[rows], ref, vmax, gqa=Hq > Hkv)
