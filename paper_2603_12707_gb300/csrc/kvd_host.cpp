@@ -5,7 +5,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <cstring>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -106,6 +105,8 @@ struct kv_cache {
     // writer.
     int64_t chain_launches = -1;                // `launches` right after the last of them
     void* chain_stream = nullptr;
+    int64_t seq_launches = -1;                  // the same for reservations and releases
+    cudaStream_t seq_stream = nullptr;
     bool chain_append = false;                  // a kv_append since the last attention launch
     int32_t* err = nullptr;
     PlanEntry* plan = nullptr;
@@ -175,20 +176,24 @@ int check_device(const kv_cache* c, const char* what)
     return KVC_OK;
 }
 
+// Reservations and releases that follow one another on a stream are chained.
+bool seq_chained(const kv_cache* c, cudaStream_t st)
+{
+    return c->seq_launches == c->launches && c->seq_stream == st;
+}
+
 // Enqueue int32 updates of the page table / lengths.
 int push_updates(kv_cache* c, const std::vector<int32_t>& idx, const std::vector<int32_t>& val,
                  cudaStream_t st)
 {
     if (c->host_only || idx.empty()) return KVC_OK;
     c->last_stream = st;
-    ScatterI32 s;
     for (size_t off = 0; off < idx.size(); off += kScatterMax) {
         const size_t n = std::min<size_t>(kScatterMax, idx.size() - off);
-        s.n = (int32_t)n;
-        std::memcpy(s.idx, idx.data() + off, n * sizeof(int32_t));
-        std::memcpy(s.val, val.data() + off, n * sizeof(int32_t));
-        KVD_CUDA(launch_scatter_i32(c->meta, s, st));
+        KVD_CUDA(launch_scatter_i32(c->meta, idx.data() + off, val.data() + off, (int)n, seq_chained(c, st), st));
         ++c->launches;
+        c->seq_launches = c->launches;
+        c->seq_stream = st;
     }
     return KVC_OK;
 }
@@ -547,8 +552,10 @@ static int seq_op_device(kv_cache* c, int32_t seq, int32_t n, bool free_seq, voi
     a.page_table = c->page_table();
     a.err = c->err;
     c->last_stream = static_cast<cudaStream_t>(stream);
-    KVD_CUDA(launch_seq_op(a, c->last_stream));
+    KVD_CUDA(launch_seq_op(a, seq_chained(c, c->last_stream), c->last_stream));
     ++c->launches;
+    c->seq_launches = c->launches;
+    c->seq_stream = c->last_stream;
     c->dev_dirty = true;
     return KVC_OK;
 }

@@ -16,6 +16,7 @@ constexpr int kChunkCapGqa = 16;       // GQA: the merge variant for 16 items fi
 constexpr int kMaxItemPages = 1024;    // largest target item size a caller may request
 constexpr int kPatchMax = 1024;        // step entries carried in one launch's parameters
 constexpr int kScatterMax = 2048;      // int32 updates carried in one launch's parameters
+constexpr int kScatterSmall = 120;     // the same for most calls (a row of up to 1900 tokens): 1 KB instead of 16
 constexpr int kVarlenMax = 512;        // token blocks carried in one bulk-write launch's parameters
 
 // One work item of a step's split plan: consecutive pages [first_page,
@@ -141,10 +142,11 @@ struct StepDevArgs {
     uint32_t* queues;         // the two work counters of the attention launches, zeroed
 };
 
+template <int N>
 struct ScatterI32 {
     int32_t n;
-    int32_t idx[kScatterMax];
-    int32_t val[kScatterMax];
+    int32_t idx[N];
+    int32_t val[N];
 };
 
 // Sequence reservation or release on the device free stack (device-side
@@ -279,14 +281,14 @@ CUresult encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_
 void set_last_error(const char* msg);
 
 // ---- launchers (return cudaGetLastError() of the launch) -----------------
-cudaError_t launch_scatter_i32(int32_t* base, const ScatterI32& s, cudaStream_t st);
+// pdl: launched with programmatic dependent launch; the kernel waits for the
+// one before it first and lets the next one start at once.
+cudaError_t launch_scatter_i32(int32_t* base, const int32_t* idx, const int32_t* val, int n, bool pdl, cudaStream_t st);
 cudaError_t launch_step(const StepPatch& patch, const PlanArgs& plan, cudaStream_t st);
 cudaError_t launch_token_copy(const TokenCopyArgs& a, cudaStream_t st);
 cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, cudaStream_t st);
 cudaError_t launch_step_device(const StepDevArgs& a, cudaStream_t st);
-cudaError_t launch_seq_op(const SeqOpArgs& a, cudaStream_t st);
-// pdl: launched with programmatic dependent launch (it waits for the kernel
-// before it first, and lets the next one start at once).
+cudaError_t launch_seq_op(const SeqOpArgs& a, bool pdl, cudaStream_t st);   // pdl as above
 cudaError_t launch_append(const AppendArgs& a, bool pdl, cudaStream_t st);
 cudaError_t launch_wait_timeout_check(uint64_t limit_ns, int32_t* status, cudaStream_t st);
 

@@ -198,3 +198,36 @@ def test_device_path_failures_are_reported_and_change_nothing(kvlib):
     assert kd.kv_seq_info(h3, s3)[0] == 8 * P
     for x in (h, h2, h3):
         kd.kv_cache_destroy(x)
+
+
+@pytest.mark.parametrize("pages", [1, 118, 119, 120, 2046, 2047, 2048])
+def test_host_reservations_around_one_launchs_updates(kvlib, pages):
+    """A reservation updates a page-table entry per page and the length, 120
+    or 2048 at a time; releases and reservations in a row are chained.  The
+    device's table is right if every token reads back from where it was
+    written."""
+    cfg = kd.make_config(1, 2, 2, 64, 2 * pages + 3, 3, pages + 1)
+    h = kd.kv_cache_create(cfg)
+    perm = np.random.default_rng(pages).permutation(2 * pages + 3)
+    kd.kv_cache_set_page_order(h, perm)
+    for _ in range(3):
+        a = kd.kv_seq_create(h)
+        kd.kv_seq_reserve(h, a, pages * P)
+        b = kd.kv_seq_create(h)
+        kd.kv_seq_reserve(h, b, pages * P - 3)
+        kd.kv_seq_free(h, a)
+        a = kd.kv_seq_create(h)
+        kd.kv_seq_reserve(h, a, 5)
+        kd.kv_seq_reserve(h, a, pages * P - 5)
+        toks = {s: torch.randn((n, 2, 64), device="cuda").bfloat16() for s, n in ((a, pages * P), (b, pages * P - 3))}
+        for s, x in toks.items():
+            kd.kv_write_tokens(h, 0, s, 0, x.shape[0], x, -x)
+        for s, x in toks.items():
+            k, v = torch.empty_like(x), torch.empty_like(x)
+            kd.kv_read_tokens(h, 0, s, 0, x.shape[0], k, v)
+            torch.cuda.synchronize()
+            assert torch.equal(k, x) and torch.equal(v, -x)
+        kd.kv_seq_free(h, a)
+        kd.kv_seq_free(h, b)
+    assert kd.kv_cache_query(h).free_pages == 2 * pages + 3
+    kd.kv_cache_destroy(h)
