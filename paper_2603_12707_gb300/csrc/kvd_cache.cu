@@ -332,35 +332,63 @@ __global__ void __launch_bounds__(256) seq_op_kernel(const SeqOpArgs a)
     }
 }
 
-// One thread per 16-byte chunk of a [n][H_kv][D] token block.
-__global__ void token_copy_kernel(const TokenCopyArgs a)
+// Tokens of one sequence and layer to or from its pages.  CTA (x, y) takes
+// the x-th page touched and the y-th 1024 of its 16-byte chunks, in the
+// page's order ([H_kv][slot][D]); the page id is read once and a thread's
+// four chunks of K and V are in flight together.  (A grid-stride loop of one
+// chunk with 64-bit divisions, for 900 LLaVA tokens of a layer,
+// 14.7 MB read and written, 4.4 us at the copy rate: 10.2 us in
+// a row, now 6.4 with the launches chained; 16 tokens 4.2, now 2.6.)
+constexpr int kCopyThreads = 256;
+constexpr int kCopyUnroll = 4;
+
+template <bool TO_POOL>
+__global__ void __launch_bounds__(kCopyThreads) token_copy_kernel(const TokenCopyArgs a)
 {
+    griddep_launch_dependents();
+    griddep_wait();
     if (a.len && a.first_pos + a.n > *a.len) {   // positions past the sequence's length
-        if (blockIdx.x == 0 && threadIdx.x == 0) flag_error(a.err, 4);
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) flag_error(a.err, 4);
         return;
     }
-    const int chunks = a.D / 8;
-    const int64_t total = (int64_t)a.n * a.H_kv * chunks;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % chunks);
-        const int64_t tg = i / chunks;
-        const int g = (int)(tg % a.H_kv);
-        const int t = (int)(tg / a.H_kv);
-        const int pos = a.first_pos + t;
-        const int32_t page = a.pt_row[pos / kPageSize];
-        if (page < 0 || page >= a.num_pages) {
-            flag_error(a.err, 1);
-            continue;
+    const int page_idx = a.first_pos / kPageSize + (int)blockIdx.x;
+    const int p0 = max(a.first_pos, page_idx * kPageSize);
+    const int nt = min(a.first_pos + a.n, (page_idx + 1) * kPageSize) - p0;
+    const int32_t pid = a.pt_row[page_idx];
+    if (pid < 0 || pid >= a.num_pages) {
+        if (threadIdx.x == 0) flag_error(a.err, 1);
+        return;
+    }
+    const int cpr = a.D / 8;   // 16-byte chunks per (token, head) row
+    const int total = a.H_kv * nt * cpr;
+    const int slot0 = p0 - page_idx * kPageSize;
+    const int64_t page = (int64_t)pid * a.H_kv * kPageSize * cpr;
+    const int64_t tok0 = (int64_t)(p0 - a.first_pos) * a.H_kv * cpr;
+    uint4* pk = reinterpret_cast<uint4*>(a.pool_k) + page;
+    uint4* pv = reinterpret_cast<uint4*>(a.pool_v) + page;
+    uint4* tk = reinterpret_cast<uint4*>(a.tok_k) + tok0;
+    uint4* tv = reinterpret_cast<uint4*>(a.tok_v) + tok0;
+    uint4 rk[kCopyUnroll], rv[kCopyUnroll];
+    int from[kCopyUnroll], to[kCopyUnroll];
+    const int base = (int)blockIdx.y * kCopyThreads * kCopyUnroll + threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u) {
+        const int idx = base + u * kCopyThreads;
+        if (idx < total) {
+            const int r = idx / cpr, c = idx - r * cpr;
+            const int h = r / nt, t = r - h * nt;
+            const int in_page = (h * kPageSize + slot0 + t) * cpr + c, in_tok = (t * a.H_kv + h) * cpr + c;
+            from[u] = TO_POOL ? in_tok : in_page;
+            to[u] = TO_POOL ? in_page : in_tok;
+            rk[u] = (TO_POOL ? tk : pk)[from[u]];
+            rv[u] = (TO_POOL ? tv : pv)[from[u]];
         }
-        const int64_t poff = (((int64_t)page * a.H_kv + g) * kPageSize + pos % kPageSize) * a.D + c * 8;
-        const int64_t toff = i * 8;
-        if (a.to_pool) {
-            *reinterpret_cast<uint4*>(a.pool_k + poff) = *reinterpret_cast<const uint4*>(a.tok_k + toff);
-            *reinterpret_cast<uint4*>(a.pool_v + poff) = *reinterpret_cast<const uint4*>(a.tok_v + toff);
-        } else {
-            *reinterpret_cast<uint4*>(a.tok_k + toff) = *reinterpret_cast<const uint4*>(a.pool_k + poff);
-            *reinterpret_cast<uint4*>(a.tok_v + toff) = *reinterpret_cast<const uint4*>(a.pool_v + poff);
+    }
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u) {
+        if (base + u * kCopyThreads < total) {
+            (TO_POOL ? pk : tk)[to[u]] = rk[u];
+            (TO_POOL ? pv : tv)[to[u]] = rv[u];
         }
     }
 }
@@ -375,6 +403,8 @@ constexpr int kVarlenUnroll = 4;
 
 __global__ void __launch_bounds__(kVarlenThreads) varlen_write_kernel(const __grid_constant__ VarlenWriteArgs a)
 {
+    griddep_launch_dependents();
+    griddep_wait();
     const int tile = blockIdx.x;
     int lo = 0, hi = a.n_blocks - 1;   // the last block with tile_start <= tile
     while (lo < hi) {
@@ -489,10 +519,10 @@ __global__ void wait_timeout_kernel(uint64_t limit_ns, int32_t* status)
 // A launch that may start before the one before it has completed, if pdl (the
 // kernel waits before it reads or writes anything).
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kernel)(P...), int grid, int block, bool pdl, cudaStream_t st, const A&... args)
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, bool pdl, cudaStream_t st, const A&... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -545,21 +575,21 @@ cudaError_t launch_step(const StepPatch& patch, const PlanArgs& plan, cudaStream
     return cudaGetLastError();
 }
 
-cudaError_t launch_token_copy(const TokenCopyArgs& a, cudaStream_t st)
+cudaError_t launch_token_copy(const TokenCopyArgs& a, bool pdl, cudaStream_t st)
 {
-    const int64_t total = (int64_t)a.n * a.H_kv * (a.D / 8);
-    if (total <= 0) return cudaSuccess;
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > 65535) blocks = 65535;
-    token_copy_kernel<<<(unsigned)blocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    if (a.n <= 0) return cudaSuccess;
+    const int pages = (a.first_pos + a.n - 1) / kPageSize - a.first_pos / kPageSize + 1;
+    const int per_cta = kCopyThreads * kCopyUnroll;
+    const int chunks = a.H_kv * std::min(a.n, kPageSize) * (a.D / 8);   // of a page at most
+    const dim3 grid((unsigned)pages, (unsigned)((chunks + per_cta - 1) / per_cta));
+    return a.to_pool ? launch_chained(token_copy_kernel<true>, grid, kCopyThreads, pdl, st, a)
+                     : launch_chained(token_copy_kernel<false>, grid, kCopyThreads, pdl, st, a);
 }
 
-cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, cudaStream_t st)
+cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, bool pdl, cudaStream_t st)
 {
     if (a.n_tiles <= 0 || n_layers <= 0) return cudaSuccess;
-    varlen_write_kernel<<<dim3((unsigned)a.n_tiles, (unsigned)n_layers), kVarlenThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(varlen_write_kernel, dim3((unsigned)a.n_tiles, (unsigned)n_layers), kVarlenThreads, pdl, st, a);
 }
 
 cudaError_t launch_append(const AppendArgs& a, bool pdl, cudaStream_t st)

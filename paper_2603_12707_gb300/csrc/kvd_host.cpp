@@ -105,7 +105,7 @@ struct kv_cache {
     // writer.
     int64_t chain_launches = -1;                // `launches` right after the last of them
     void* chain_stream = nullptr;
-    int64_t seq_launches = -1;                  // the same for reservations and releases
+    int64_t seq_launches = -1;                  // the same for reservations, releases and token copies
     cudaStream_t seq_stream = nullptr;
     bool chain_append = false;                  // a kv_append since the last attention launch
     int32_t* err = nullptr;
@@ -176,10 +176,17 @@ int check_device(const kv_cache* c, const char* what)
     return KVC_OK;
 }
 
-// Reservations and releases that follow one another on a stream are chained.
+// Reservations, releases and token copies that follow one another on a stream
+// are chained: each waits for the one before it before it reads anything.
 bool seq_chained(const kv_cache* c, cudaStream_t st)
 {
     return c->seq_launches == c->launches && c->seq_stream == st;
+}
+
+void seq_launched(kv_cache* c, cudaStream_t st)
+{
+    c->seq_launches = ++c->launches;
+    c->seq_stream = st;
 }
 
 // Enqueue int32 updates of the page table / lengths.
@@ -191,9 +198,7 @@ int push_updates(kv_cache* c, const std::vector<int32_t>& idx, const std::vector
     for (size_t off = 0; off < idx.size(); off += kScatterMax) {
         const size_t n = std::min<size_t>(kScatterMax, idx.size() - off);
         KVD_CUDA(launch_scatter_i32(c->meta, idx.data() + off, val.data() + off, (int)n, seq_chained(c, st), st));
-        ++c->launches;
-        c->seq_launches = c->launches;
-        c->seq_stream = st;
+        seq_launched(c, st);
     }
     return KVC_OK;
 }
@@ -553,9 +558,7 @@ static int seq_op_device(kv_cache* c, int32_t seq, int32_t n, bool free_seq, voi
     a.err = c->err;
     c->last_stream = static_cast<cudaStream_t>(stream);
     KVD_CUDA(launch_seq_op(a, seq_chained(c, c->last_stream), c->last_stream));
-    ++c->launches;
-    c->seq_launches = c->launches;
-    c->seq_stream = c->last_stream;
+    seq_launched(c, c->last_stream);
     c->dev_dirty = true;
     return KVC_OK;
 }
@@ -667,8 +670,8 @@ static int token_copy(kv_cache* c, const char* what, int32_t layer, int32_t seq,
     a.to_pool = to_pool;
     a.err = c->err;
     c->last_stream = static_cast<cudaStream_t>(stream);
-    KVD_CUDA(launch_token_copy(a, static_cast<cudaStream_t>(stream)));
-    ++c->launches;
+    KVD_CUDA(launch_token_copy(a, seq_chained(c, c->last_stream), c->last_stream));
+    seq_launched(c, c->last_stream);
     return KVC_OK;
 }
 
@@ -747,8 +750,8 @@ int kv_write_varlen(kv_cache* c, int32_t layer_first, int32_t n_layers, int32_t 
     auto flush = [&]() -> int {
         if (a.n_blocks == 0) return KVC_OK;
         a.n_tiles = a.tile_start[a.n_blocks];
-        KVD_CUDA(launch_varlen_write(a, n_layers, st));
-        ++c->launches;
+        KVD_CUDA(launch_varlen_write(a, n_layers, seq_chained(c, st), st));
+        seq_launched(c, st);
         a.n_blocks = 0;
         return KVC_OK;
     };

@@ -285,8 +285,8 @@ void set_last_error(const char* msg);
 // one before it first and lets the next one start at once.
 cudaError_t launch_scatter_i32(int32_t* base, const int32_t* idx, const int32_t* val, int n, bool pdl, cudaStream_t st);
 cudaError_t launch_step(const StepPatch& patch, const PlanArgs& plan, cudaStream_t st);
-cudaError_t launch_token_copy(const TokenCopyArgs& a, cudaStream_t st);
-cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, cudaStream_t st);
+cudaError_t launch_token_copy(const TokenCopyArgs& a, bool pdl, cudaStream_t st);                    // pdl as above
+cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, bool pdl, cudaStream_t st);   // pdl as above
 cudaError_t launch_step_device(const StepDevArgs& a, cudaStream_t st);
 cudaError_t launch_seq_op(const SeqOpArgs& a, bool pdl, cudaStream_t st);   // pdl as above
 cudaError_t launch_append(const AppendArgs& a, bool pdl, cudaStream_t st);

@@ -437,3 +437,29 @@ def test_chained_append_then_attend_sees_the_new_token(kvlib, Hq, Hkv, lens, spl
         t.close()
     for a, b in zip(*outs):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("first,n", [(0, 1), (15, 1), (15, 2), (16, 16), (3, 13), (7, 90), (1, 143)])
+@pytest.mark.parametrize("H,d", [(40, 128), (2, 64), (3, 128), (33, 64)])
+def test_token_copies_touch_exactly_their_positions(kvlib, H, d, first, n):
+    """kv_write_tokens and kv_read_tokens at the edges of pages and of the
+    1024 chunks a CTA copies; the other positions keep their contents."""
+    cfg = wl.custom("copies", 2, H, H, d, 1, lens=[150], seed=H + d, page_order="shuffled")
+    t = Tracked(cfg)
+    h, s = t.sess.h, t.sess.seq_ids[0]
+    x = torch.randn((n, H, d), generator=torch.Generator().manual_seed(n)).bfloat16().cuda()
+    kd.kv_write_tokens(h, 1, s, first, n, x, -x)
+    back = [[torch.empty((150, H, d), dtype=torch.bfloat16, device="cuda") for _ in range(2)] for _ in range(2)]
+    part = [torch.empty_like(x) for _ in range(2)]
+    for l in range(2):
+        kd.kv_read_tokens(h, l, s, 0, 150, back[l][0], back[l][1])
+    kd.kv_read_tokens(h, 1, s, first, n, part[0], part[1])
+    torch.cuda.synchronize()
+    for l in range(2):
+        for i, kind in enumerate("kv"):
+            want = wl.kv_block(cfg, l, 0, 150, kind, "cuda")
+            if l == 1:
+                want[first:first + n] = x if kind == "k" else -x
+            assert torch.equal(back[l][i], want)
+    assert torch.equal(part[0], x) and torch.equal(part[1], -x)
+    t.close()
