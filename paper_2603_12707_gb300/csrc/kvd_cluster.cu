@@ -126,10 +126,11 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     int G = GQA ? p.G : 1;
 
     // The next launch may start at once: it reads nothing this one writes
-    // before its own dependency wait (but for slots that it replaces).
-    griddep_launch_dependents();
+    // before its own dependency wait (but for slots that it replaces).  After
+    // a step kernel both wait for that first.
     bool waited = p.early == 0;
     if (waited) griddep_wait();
+    griddep_launch_dependents();
     const int unit = (int)blockIdx.x / C;
     const int b = unit / p.H_kv, g = unit - b * p.H_kv;
     int2 row;   // (page-table row, tokens attended)

@@ -577,6 +577,9 @@ __global__ void __launch_bounds__(kWarps * 32)
     const int n_warps = (int)gridDim.x * kWarps;
     int item = (int)blockIdx.x * kWarps + warp;
 
+    // The first launch after a step kernel: placed early, but the plan is not
+    // there before the wait.
+    if (!p.early) griddep_wait();
     const int n_items = p.n_entries_dev ? min(p.n_items, *p.n_entries_dev * p.H_kv) : p.n_items;
     while (item < n_items) {
         const int e = item / p.H_kv;

@@ -105,6 +105,8 @@ struct kv_cache {
     // writer.
     int64_t chain_launches = -1;                // `launches` right after the last of them
     void* chain_stream = nullptr;
+    int64_t step_launches = -1;                 // the same for the step kernels
+    void* step_stream = nullptr;
     int64_t seq_launches = -1;                  // the same for reservations, releases and token copies
     cudaStream_t seq_stream = nullptr;
     bool chain_append = false;                  // a kv_append since the last attention launch
@@ -879,7 +881,8 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
             }
             pa.build = (b0 + n == batch) ? 1 : 0;
             KVD_CUDA(launch_step(patch, pa, st));
-            ++c->launches;
+            c->step_launches = ++c->launches;
+            c->step_stream = st;
         }
     }
     if (!c->host_only)
@@ -992,17 +995,19 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     const int grid = (int)std::max<int64_t>(1, std::min(resident, want));
     p.kv_map = 1;
     const bool pdl = c->chain_launches == c->launches && c->chain_stream == stream;
+    // After the step kernel: placed while it runs, reads nothing before its end.
+    const bool after_step = !pdl && c->step_launches == c->launches && c->step_stream == stream;
+    p.early = after_step ? 0 : 1;
     p.hold_last = pdl && !fused && c->chain_append ? 1 : 0;
     c->chain_append = false;
     if (c->step_cluster.ctas) {
         p.ring = c->step_cluster.ring;
-        p.early = pdl ? 1 : 0;
         p.start_flags = nullptr;
         p.step_no = nullptr;
         p.tag = p.prev_tag = 0;
         p.num_sms = c->num_sms;
         c->last_stream = static_cast<cudaStream_t>(stream);
-        KVD_CUDA(launch_cluster(c->cfg.head_dim, c->group > 1, fused, pdl, c->step_cluster,
+        KVD_CUDA(launch_cluster(c->cfg.head_dim, c->group > 1, fused, pdl || after_step, c->step_cluster,
                                 batch * c->cfg.num_kv_heads, c->tmaps[layer], c->tmaps[layer], p,
                                 nullptr, static_cast<cudaStream_t>(stream)));
         ++c->launches;
@@ -1031,7 +1036,7 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     p.tag = ++c->attn_tag;
     p.num_sms = c->num_sms;
     c->last_stream = static_cast<cudaStream_t>(stream);
-    KVD_CUDA(launch_decode(c->cfg.head_dim, c->group > 1, fused, pdl, grid, c->tmaps[layer], c->tmaps[layer], p,
+    KVD_CUDA(launch_decode(c->cfg.head_dim, c->group > 1, fused, pdl || after_step, grid, c->tmaps[layer], c->tmaps[layer], p,
                            static_cast<cudaStream_t>(stream)));
     ++c->launches;
     ++c->attn_launches;   // the launch used one counter and resets the other, whatever follows
@@ -1145,7 +1150,8 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     a.no_plan = shape.ctas ? 1 : 0;
     c->last_stream = st;
     KVD_CUDA(launch_step_device(a, st));
-    ++c->launches;
+    c->step_launches = ++c->launches;
+    c->step_stream = st;
     c->dev_dirty = true;
     c->attn_tag = 0;
     c->prev_merge = false;

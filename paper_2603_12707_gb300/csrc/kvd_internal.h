@@ -258,7 +258,7 @@ struct DecodeParams {
     int32_t num_sms;
     // cluster_kernel only: it reads lengths and page ids by batch row instead of a plan.
     int32_t ring;             // shared-memory stages per warp
-    int32_t early;            // 1: the cache may be read before the dependency wait
+    int32_t early;            // 1: plan and cache may be read before the dependency wait (0: after a step kernel)
     int32_t hold_last;        // 1: but not each row's last page (a kv_append may be writing it)
 };
 

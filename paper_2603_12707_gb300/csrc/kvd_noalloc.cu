@@ -224,6 +224,7 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     p.max_pages = max_pages;
     p.scale_log2 = scale * 1.4426950408889634f;
     p.kv_map = kv_map;
+    p.early = 1;   // (an ordinary launch)
     p.num_sms = num_sms;
 
     const ClusterShape shape = cluster_shape(dev, head_dim, G > 1, num_kv_heads, batch, total_pages, max_np);

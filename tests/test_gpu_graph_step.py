@@ -378,3 +378,32 @@ def test_graph_of_one_layer_hands_out_every_item_on_every_replay(kvlib, Hq, Hkv,
         s.synchronize()
         assert torch.equal(got, ref), rep
     t.close()
+
+
+@pytest.mark.parametrize("batch,rows", [(2, 4000), (5, 700), (40, 300), (300, 90), (1025, 40)])
+def test_plans_built_by_one_and_by_eight_ctas(kvlib, batch, rows):
+    """Step kernels over up to 2048 page ids run as one CTA, else as a cluster
+    of eight; batches past 1024 rows plan in two rounds.  The split plan shows
+    in the result: device and host steps give the same bits, and sampled rows
+    match the oracle (the layer goes through the plan: the split size is set)."""
+    lens = [1 + (rows * (7 * b + 3)) // (7 * batch) for b in range(batch)]
+    lens[0] = rows
+    cfg = wl.custom("ctas", 1, 4, 4, 64, batch, lens=lens, seed=batch, page_order="shuffled")
+    keep = sorted({0, 1, batch // 2, batch - 1})
+    a = Tracked(cfg, extra_tokens=4, split_pages=SPLIT, keep_rows=keep)
+    b = Tracked(cfg, extra_tokens=4, split_pages=SPLIT, keep_host=False)
+    kd.kv_cache_device_steps(b.sess.h, batch)
+    ids = torch.tensor(b.sess.seq_ids, dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        a.begin_step()
+        kd.kv_begin_step_device(b.sess.h, batch, ids)
+        b.step += 1
+        b.sess.lens += 1
+        oa, q, _, _ = a.run_layer(0, fused=True)
+        ob, _, _, _ = b.run_layer(0, fused=True)
+        torch.cuda.synchronize()
+        assert torch.equal(oa, ob)
+        ref, vmax = a.oracle(0, q, rows=keep)
+        assert_close(bf16_to_f64(oa)[keep], ref, vmax, gqa=False)
+    a.close()
+    b.close()
