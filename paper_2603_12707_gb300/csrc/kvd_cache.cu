@@ -425,9 +425,17 @@ __global__ void __launch_bounds__(kCopyThreads) token_copy_kernel(const TokenCop
 
 // Bulk write of packed token blocks.  CTA x finds its block by a binary
 // search over tile_start, reads the tile's page id once, then its threads
-// stream the tile in the page's order ([H_kv][slot][D], 16-byte chunks, four
-// per thread in flight) with streaming loads and stores: the source is read
-// once and the pages are not read back soon.
+// stream (the z-th cta_chunks 16-byte chunks of) the tile in the page's order
+// ([H_kv][slot][D], four chunks per thread in flight) with streaming loads and
+// stores: the source is read once and the pages are not read back soon.
+//
+// A whole page of 32 or 40 heads is 160 KB for one CTA: a few hundred CTAs
+// leave the last ones running alone.  2048 chunks of K and V per CTA, 1024
+// where that gives fewer than 5000 CTAs, 512 where that gives fewer than one
+// per SM (us, one CTA per tile before / 2048 / 1024 / 512; 40 heads, 11 blocks
+// of 4-220 tokens, 4 layers: 17.0 / 9.3 / 8.3 / 8.8; 32 heads, 64 blocks of
+// 900, 8 layers: 2160 / 2153 / 2199 / 2276; 8 heads of 64, 4 blocks of 96:
+// 3.5 / 3.6 / 3.7 / 2.9).
 constexpr int kVarlenThreads = 256;
 constexpr int kVarlenUnroll = 4;
 
@@ -459,7 +467,7 @@ __global__ void __launch_bounds__(kVarlenThreads) varlen_write_kernel(const __gr
         return;
     }
     const int cpr = a.D / 8;   // 16-byte chunks per (token, head) row
-    const int total = a.H_kv * nt * cpr;
+    const int total = min(a.H_kv * nt * cpr, ((int)blockIdx.z + 1) * a.cta_chunks);
     const int64_t layer = blockIdx.y;
     const uint4* sk = reinterpret_cast<const uint4*>(a.k + layer * a.src_layer_stride);
     const uint4* sv = reinterpret_cast<const uint4*>(a.v + layer * a.src_layer_stride);
@@ -469,7 +477,7 @@ __global__ void __launch_bounds__(kVarlenThreads) varlen_write_kernel(const __gr
                 (int64_t)pid * a.H_kv * kPageSize * cpr;
     const int64_t tok0 = (int64_t)a.src_row[lo] + (p0 - first);
     const int slot0 = p0 - page_idx * kPageSize;
-    for (int base = threadIdx.x; base < total; base += kVarlenUnroll * kVarlenThreads) {
+    for (int base = (int)blockIdx.z * a.cta_chunks + threadIdx.x; base < total; base += kVarlenUnroll * kVarlenThreads) {
         uint4 rk[kVarlenUnroll], rv[kVarlenUnroll];
         int64_t doff[kVarlenUnroll];
 #pragma unroll
@@ -635,7 +643,13 @@ cudaError_t launch_token_copy(const TokenCopyArgs& a, bool pdl, cudaStream_t st)
 cudaError_t launch_varlen_write(const VarlenWriteArgs& a, int n_layers, bool pdl, cudaStream_t st)
 {
     if (a.n_tiles <= 0 || n_layers <= 0) return cudaSuccess;
-    return launch_chained(varlen_write_kernel, dim3((unsigned)a.n_tiles, (unsigned)n_layers), kVarlenThreads, pdl, st, a);
+    const int64_t chunks = a.H_kv * kPageSize * (a.D / 8);   // of a whole page's K
+    auto parts = [&](int per_cta) { return (chunks + per_cta - 1) / per_cta; };
+    const int64_t tiles = (int64_t)a.n_tiles * n_layers;
+    VarlenWriteArgs args = a;
+    args.cta_chunks = tiles * parts(2048) > 5000 ? 2048 : tiles * parts(1024) > 150 ? 1024 : 512;
+    return launch_chained(varlen_write_kernel, dim3((unsigned)a.n_tiles, (unsigned)n_layers, (unsigned)parts(args.cta_chunks)),
+                          kVarlenThreads, pdl, st, args);
 }
 
 cudaError_t launch_append(const AppendArgs& a, bool pdl, cudaStream_t st)

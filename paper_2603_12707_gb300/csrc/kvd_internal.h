@@ -193,6 +193,7 @@ struct VarlenWriteArgs {
     int32_t max_pages;
     int32_t H_kv, D;
     int32_t n_blocks, n_tiles;
+    int32_t cta_chunks;          // 16-byte chunks of a tile's K (and of its V) that one CTA copies (set by the launch)
     int32_t* err;
     int32_t tile_start[kVarlenMax + 1];  // first tile of block i; tile_start[n_blocks] = n_tiles
     int32_t seq[kVarlenMax];

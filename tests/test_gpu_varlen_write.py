@@ -159,3 +159,33 @@ def test_decode_after_varlen_prefix_matches_oracle(kvlib):
             assert_close(bf16_to_f64(out), ref, vmax, gqa=True, what=(step, l))
     assert sess.query().device_error == 0
     sess.close()
+
+
+@pytest.mark.parametrize("H,d,L,lens,first", [
+    (40, 128, 1, [3, 17, 220], [0, 5, 15]),          # 512 chunks a CTA
+    (33, 64, 2, [1, 16, 31, 100], [0, 1, 2, 3]),
+    (40, 128, 4, [220, 100, 90, 1], [7, 0, 16, 15]),   # 1024
+    (32, 128, 16, [1500, 3, 900], [9, 30, 0]),        # 2048
+])
+def test_varlen_tiles_shared_by_several_ctas(kvlib, H, d, L, lens, first):
+    """A tile's chunks are spread over CTAs by the size of the call; read back
+    per token, neighbours of the blocks untouched."""
+    room = [f + n + 20 for f, n in zip(first, lens)]
+    cfg = kd.make_config(L, H, H, d, sum((n + 15) // 16 for n in room) + 2, len(lens), max((n + 15) // 16 for n in room))
+    h = kd.kv_cache_create(cfg)
+    kd.kv_cache_set_page_order(h, np.random.default_rng(H).permutation(int(cfg.num_pages)))
+    seqs = [kd.kv_seq_create(h) for _ in lens]
+    for s, n in zip(seqs, room):
+        kd.kv_seq_reserve(h, s, n)
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    gen = torch.Generator(device="cuda").manual_seed(H + L)
+    k = torch.randn((L, cu[-1], H, d), generator=gen, device="cuda").bfloat16()
+    kd.kv_write_varlen(h, 0, L, seqs, cu, k, -k, first)
+    for b, s in enumerate(seqs):
+        for l in {0, L - 1}:
+            bk, bv = (torch.empty((room[b], H, d), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+            kd.kv_read_tokens(h, l, s, 0, room[b], bk, bv)
+            want = torch.zeros_like(bk)
+            want[first[b]:first[b] + lens[b]] = k[l, cu[b]:cu[b + 1]]
+            assert torch.equal(bk, want) and torch.equal(bv, -want)
+    kd.kv_cache_destroy(h)
