@@ -53,6 +53,28 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 void kvd::set_last_error(const char* msg) { g_last_error = msg; }
 
+int32_t kvd::auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages,
+                             int64_t max_pages, bool growing)
+{
+    const int64_t units = rows * num_kv_heads, total = pages * num_kv_heads;
+    const int64_t per_warp = gqa ? 2 : 3;
+    int64_t T = std::min<int64_t>(128, std::max<int64_t>(2, (total + per_warp * warps - 1) / (per_warp * warps)));
+    // Pages of 4 KB (d = 128) per warp.
+    const double share = (double)total / (double)warps * D / 128;
+    if (share > 30 || rows < 1) return (int32_t)T;
+    const double even = (double)max_pages * (double)rows / (double)std::max<int64_t>(1, pages);   // longest row / mean row
+    int64_t few = 0;
+    if (even <= (share < 15 ? 1.35 : 1.15)) {
+        const double want = (double)warps / (double)units * (share < 15 ? 1.06 : 1.3) + (share < 15 ? 0.0 : 0.5);
+        const int64_t items = std::max<int64_t>(1, (int64_t)want);
+        few = (max_pages + (growing ? max_pages / 8 : 0) + items - 1) / items;
+    } else if (max_pages <= 8 || (units >= warps && 10 * max_pages * warps <= 13 * total)) {
+        few = max_pages;
+    }
+    if (few >= max_pages) few = std::max<int64_t>(few, 16);
+    return (int32_t)std::max(T, std::min<int64_t>(128, few));
+}
+
 CUresult kvd::encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_t rows, int D,
                               int64_t v_stride_bytes)
 {
@@ -205,17 +227,9 @@ int push_updates(kv_cache* c, const std::vector<int32_t>& idx, const std::vector
     return KVC_OK;
 }
 
-int32_t auto_item_pages(const kv_cache* c, int64_t total_units)
+int64_t resident_warps(const kv_cache* c)
 {
-    // About three work items per resident warp keeps the tail of the
-    // persistent schedule short; a GQA item leaves a partial for each of its
-    // G query heads, so GQA aims at two.  Items stay within [2, 128] pages
-    // (long rows get larger items through the per-row cap on items).
-    const int64_t warps = (int64_t)std::max(1, c->num_sms) * std::max(1, c->variant.ctas_per_sm) *
-                          std::max(1, c->variant.warps);
-    const int64_t per_warp = c->group > 1 ? 2 : 3;
-    const int64_t T = (total_units + per_warp * warps - 1) / (per_warp * warps);
-    return (int32_t)std::min<int64_t>(128, std::max<int64_t>(2, T));
+    return (int64_t)std::max(1, c->num_sms) * std::max(1, c->variant.ctas_per_sm) * std::max(1, c->variant.warps);
 }
 
 // Items per row at most: twice the usual cap when rows x KV heads x the
@@ -227,9 +241,7 @@ int32_t auto_item_pages(const kv_cache* c, int64_t total_units)
 // 16, 0.756 at 24, 0.686 at 12).
 int32_t chunk_cap(const kv_cache* c, int64_t rows, int64_t max_pages, int32_t T)
 {
-    const int64_t warps = (int64_t)std::max(1, c->num_sms) * std::max(1, c->variant.ctas_per_sm) *
-                          std::max(1, c->variant.warps);
-    const bool few_units = rows * c->cfg.num_kv_heads * kChunkCap < warps;
+    const bool few_units = rows * c->cfg.num_kv_heads * kChunkCap < resident_warps(c);
     if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
     return c->group > 1 ? kChunkCapGqa : kChunkCap;
 }
@@ -804,7 +816,11 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         np_after[b] = (c->lens[seq_ids[b]] + 1 + kPageSize - 1) / kPageSize;
         total_units += (int64_t)np_after[b] * c->cfg.num_kv_heads;
     }
-    const int32_t T = c->split_override ? c->split_override : auto_item_pages(c, total_units);
+    const int32_t max_np = *std::max_element(np_after.begin(), np_after.end());
+    const int32_t T = c->split_override ? c->split_override
+                                        : auto_item_pages(c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads,
+                                                          resident_warps(c), batch, total_units / c->cfg.num_kv_heads,
+                                                          max_np, false);
     // Plan order: longest rows first (stable), when the batch fits one launch.
     const bool use_order = batch <= kPatchMax;
     std::vector<int32_t> order((size_t)batch), rank((size_t)batch);
@@ -813,7 +829,6 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         std::stable_sort(order.begin(), order.end(),
                          [&](int32_t x, int32_t y) { return np_after[x] > np_after[y]; });
     for (int32_t i = 0; i < batch; ++i) rank[order[i]] = i;
-    const int32_t max_np = *std::max_element(np_after.begin(), np_after.end());
     ClusterShape shape;
     if (!c->split_override && !c->host_only)
         shape = cluster_shape(c->device, c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, batch,
@@ -1094,7 +1109,8 @@ int kv_cache_device_steps(kv_cache* c, int32_t max_batch, int32_t enable, void* 
     // Work-item size from the pages now held (steps add a token per sequence).
     const int32_t T = c->split_override
                           ? c->split_override
-                          : auto_item_pages(c, c->pages_in_use * (int64_t)c->cfg.num_kv_heads);
+                          : auto_item_pages(c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, resident_warps(c),
+                                            c->dev_seqs, c->dev_pages, c->dev_row_pages, true);
     const int32_t cap = chunk_cap(c, max_batch, c->cfg.max_pages_per_seq, T);
     const int32_t entries = max_batch * cap;
     const int32_t stride = std::max(T, (c->cfg.max_pages_per_seq + cap - 1) / cap) + 1;

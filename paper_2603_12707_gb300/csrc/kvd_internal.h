@@ -278,6 +278,27 @@ constexpr int kClusterRingBytes = 24576;   // a warp's ring at most (3 stages at
 CUresult encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_t rows, int D,
                          int64_t v_stride_bytes);
 
+// Target pages per work item of a step of `rows` rows that hold `pages` pages
+// per KV head in all and at most max_pages in one row; growing: the rows will
+// outgrow these numbers by some tokens (device steps fix the target once).
+//
+// Items end at about the same time on all warps if there are some of them per
+// warp: three for MHA, two for GQA, whose items leave a partial per query
+// head.  But an item costs about 0.6 pages beside its own, and a row of several
+// a merge, so where a warp's share is short (up to 30 pages of d = 128),
+//  - rows of nearly equal length are cut into one item per resident warp, or
+//    up to 1.3 for shares past 15 pages (us per layer, before -> now; 32 heads
+//    of 900 tokens, B 5 / 8 / 12: 17.0 -> 14.3, 22.8 -> 20.1, 30.4 -> 29.1;
+//    16/8 heads of 500, B 32: 14.9 -> 12.6; 14/2 heads at d = 64 of 1000, B
+//    128: 17.2 -> 15.2; 8/8 at d = 64 of 700, B 64: 22.1 -> 18.6);
+//  - rows of up to 8 pages, or unequal ones of which none is much longer than
+//    a warp's share, stay whole (56/8 heads, 106 rows of up to 105 tokens:
+//    13.0 -> 9.9; 32 heads, 57 rows of up to 263: 26.1 -> 23.1).
+// Longer shares gain nothing (32 heads of 900, B 24 / 32: best target within
+// 2 % of a third of the share).
+int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages, int64_t max_pages,
+                        bool growing);
+
 // Message returned by kv_last_error() on the calling thread.
 void set_last_error(const char* msg);
 

@@ -152,11 +152,8 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     // partials fit the static scratch: the documented limit.
     const int64_t warps = (int64_t)num_sms * std::max(1, var.ctas_per_sm) * std::max(1, var.warps);
     const int64_t units = total_pages * num_kv_heads;
-    auto target = [&](int64_t per_warp) {
-        return std::min<int64_t>(128, std::max<int64_t>(2, (units + per_warp * warps - 1) / (per_warp * warps)));
-    };
     const size_t partial = (size_t)num_kv_heads * G * (head_dim * sizeof(float) + sizeof(float2));   // per entry
-    int64_t T = target(3);
+    int64_t T = std::min<int64_t>(128, std::max<int64_t>(2, (units + 3 * warps - 1) / (3 * warps)));
     size_t need = 0;
     int max_np = 0;
     // T doubles, clamped to kMaxItemPages; the attempt at kMaxItemPages is the last.
@@ -265,7 +262,8 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
         rt.off[batch] = off;
         return off_part + (size_t)split_end * partial + 512 <= kNoAllocScratchBytes;
     };
-    const int64_t T_step = std::max(T, target(G > 1 ? 2 : 3));
+    const int64_t T_step =
+        std::max<int64_t>(T, auto_item_pages(head_dim, G > 1, num_kv_heads, warps, batch, total_pages, max_np, false));
     if (!cut(T_step, G > 1 ? kChunkCapGqa : kChunkCap, true) && !cut(T, kChunkCap, false))
         return fail(KVC_ERR_UNSUPPORTED, "the batch does not fit the static scratch");
     const int32_t entries = rt.off[batch];

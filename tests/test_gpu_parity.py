@@ -463,3 +463,24 @@ def test_token_copies_touch_exactly_their_positions(kvlib, H, d, first, n):
             assert torch.equal(back[l][i], want)
     assert torch.equal(part[0], x) and torch.equal(part[1], -x)
     t.close()
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,lens", [
+    (32, 32, 128, [900 + b for b in range(5)]),              # even rows, one item per warp
+    (32, 32, 128, [640, 650, 655] * 7),                      # up to 1.3 (a share past 15 pages)
+    (8, 8, 64, [700 - b % 40 for b in range(64)]),
+    (56, 8, 128, [22 + (b * 17) % 84 for b in range(106)]),  # short rows, whole
+    (32, 32, 128, [14 + (b * 31) % 240 for b in range(57)]),
+    (28, 4, 128, [127, 128] * 60),                           # 8 pages, then 9 for half of them
+])
+def test_even_and_short_rows_pick_their_item_size(kvlib, Hq, Hkv, d, lens):
+    cfg = wl.custom("even", 1, Hq, Hkv, d, len(lens), lens=lens, seed=53 + Hq, page_order="shuffled")
+    rows = sorted({0, 1, len(lens) // 2, len(lens) - 1})
+    t = Tracked(cfg, extra_tokens=8, keep_rows=rows)
+    for _ in range(2):
+        t.begin_step()
+        out, q, _, _ = t.run_layer(0, fused=True)
+        torch.cuda.synchronize()
+        ref, vmax = t.oracle(0, q, rows=rows)
+        assert_close(bf16_to_f64(out)[rows], ref, vmax, gqa=Hq > Hkv)
+    t.close()
