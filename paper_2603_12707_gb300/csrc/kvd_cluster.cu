@@ -236,24 +236,7 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     };
     auto after = [&](int s) { return s + 1 == R ? 0 : s + 1; };
     auto tokens = [&](int j) { return min(kPageSize, len - (first + j) * kPageSize); };
-    int j = 0, s = 0;
-    if constexpr (!GQA) {
-        // two pages at a time: MHA's page is a dependent chain of ~440 cycles
-        for (; ok && j + 1 < n && R > 1; j += 2) {
-            const int s1 = after(s);
-            ok = arrived(j, s) && arrived(j + 1, s1);
-            if (!ok) break;
-            uint8_t* const k[2] = {ring + s * STAGE + k_off, ring + s1 * STAGE + k_off};
-            uint8_t* const v[2] = {ring + s * STAGE + v_off, ring + s1 * STAGE + v_off};
-            const int valid[2] = {tokens(j), tokens(j + 1)};
-            comp.template pages<2>(k, v, valid, scale_log2);
-            __syncwarp();
-            refill(j, s);
-            refill(j + 1, s1);
-            s = after(s1);
-        }
-    }
-    for (; ok && j < n; ++j) {
+    for (int j = 0, s = 0; ok && j < n; ++j) {
         ok = arrived(j, s);
         if (!ok) break;
         if (GQA && j == 0) comp.ready(lane);

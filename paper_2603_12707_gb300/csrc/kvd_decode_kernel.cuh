@@ -133,48 +133,37 @@ struct MhaCompute {
 
     __device__ __forceinline__ void ready(int) {}
 
-    // NP pages at once (their K tiles at sK[i], V tiles at sV[i], the first
-    // valid[i] of 16 tokens attended): the pages' dependent chains overlap.
-    template <int NP>
-    __device__ __forceinline__ void pages(uint8_t* const (&sK)[NP], uint8_t* const (&sV)[NP], const int (&valid)[NP],
-                                          float scale_log2)
+    __device__ __forceinline__ void page(uint8_t* sK, uint8_t* sV, uint32_t, uint32_t, int valid,
+                                         float scale_log2, int lane)
     {
-        const int tok = (c >> 1) * TPI + tsub;
-        float sc[NP];
-        bool above = false;
+        float part[IT];
 #pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            float part[IT];
-#pragma unroll
-            for (int i = 0; i < IT; ++i) {
-                const uint4 kv = *reinterpret_cast<const uint4*>(sK[q] + swz(i * TPI + tsub, c));
-                part[i] = dot8(kv, q2);
-            }
-            // Reduce-scatter over the CH lanes of a row: afterwards lane c holds
-            // token (c >> 1) * TPI + tsub, summed over all chunks.
-#pragma unroll
-            for (int lv = 0; lv < LOG_IT; ++lv) {
-                const int n = IT >> lv;
-                const int mask = CH >> (lv + 1);
-                const bool hi = (c & mask) != 0;
-#pragma unroll
-                for (int k = 0; k < n / 2; ++k) {
-                    const float send = hi ? part[k] : part[k + n / 2];
-                    const float keep = hi ? part[k + n / 2] : part[k];
-                    part[k] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
-                }
-            }
-            const float x = part[0] + __shfl_xor_sync(0xffffffffu, part[0], 1);
-            sc[q] = (tok < valid[q]) ? x * scale_log2 : -INFINITY;
-            above |= sc[q] > m + 8.f;
+        for (int i = 0; i < IT; ++i) {
+            const uint4 kv = *reinterpret_cast<const uint4*>(sK + swz(i * TPI + tsub, c));
+            part[i] = dot8(kv, q2);
         }
+        // Reduce-scatter over the CH lanes of a row: afterwards lane c holds
+        // token (c >> 1) * TPI + tsub, summed over all chunks.
+#pragma unroll
+        for (int lv = 0; lv < LOG_IT; ++lv) {
+            const int n = IT >> lv;
+            const int mask = CH >> (lv + 1);
+            const bool hi = (c & mask) != 0;
+#pragma unroll
+            for (int k = 0; k < n / 2; ++k) {
+                const float send = hi ? part[k] : part[k + n / 2];
+                const float keep = hi ? part[k + n / 2] : part[k];
+                part[k] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+            }
+        }
+        float sc = part[0] + __shfl_xor_sync(0xffffffffu, part[0], 1);
+        const int tok = (c >> 1) * TPI + tsub;
+        sc = (tok < valid) ? sc * scale_log2 : -INFINITY;
         // The reference m moves only when a score exceeds it by more than 8
         // (log2 units; see GqaCompute::page), so most pages skip the max
         // reduction and the rescale.
-        if (__any_sync(0xffffffffu, above)) {
-            float pm = sc[0];
-#pragma unroll
-            for (int q = 1; q < NP; ++q) pm = fmaxf(pm, sc[q]);
+        if (__any_sync(0xffffffffu, sc > m + 8.f)) {
+            float pm = sc;
 #pragma unroll
             for (int mask = 2; mask < 32; mask <<= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, mask));
             const float mn = fmaxf(m, pm);
@@ -185,29 +174,17 @@ struct MhaCompute {
 #pragma unroll
             for (int k = 0; k < 4; ++k) o2[k] = f2_fma(o2[k], a2, 0ull);
         }
+        const float pe = ex2(sc - m);
+        l += (c & 1) ? 0.f : pe;
 #pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            const float pe = ex2(sc[q] - m);
-            l += (c & 1) ? 0.f : pe;
-#pragma unroll
-            for (int i = 0; i < IT; ++i) {
-                const float pt = __shfl_sync(0xffffffffu, pe, tsub * CH + 2 * i);
-                const int t = i * TPI + tsub;
-                if (t < valid[q]) {   // rows past the end may hold anything
-                    const uint4 vv = *reinterpret_cast<const uint4*>(sV[q] + swz(t, c));
-                    axpy8(o2, f2_pack(pt, pt), vv);
-                }
+        for (int i = 0; i < IT; ++i) {
+            const float pt = __shfl_sync(0xffffffffu, pe, tsub * CH + 2 * i);
+            const int t = i * TPI + tsub;
+            if (t < valid) {   // rows past the end may hold anything
+                const uint4 vv = *reinterpret_cast<const uint4*>(sV + swz(t, c));
+                axpy8(o2, f2_pack(pt, pt), vv);
             }
         }
-    }
-
-    __device__ __forceinline__ void page(uint8_t* sK, uint8_t* sV, uint32_t, uint32_t, int valid,
-                                         float scale_log2, int)
-    {
-        uint8_t* const k[1] = {sK};
-        uint8_t* const v[1] = {sV};
-        const int n[1] = {valid};
-        pages<1>(k, v, n, scale_log2);
     }
 
     // Writes the output (a row of one item) or the item's partial (a split
