@@ -422,11 +422,12 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
 // (split plan -> clusters).  Clusters save the merge pass and its dependency
 // hop (2.3 us), but cut the rows evenly, without the plan's balancing: they
 // win up to about 45 MB of K/V per layer (LLaVA heads, 800 tokens, B 1 / 2 / 3:
-// 6.5 -> 4.8, 9.2 -> 7.3, 11.2 -> 10.0; B 4, 52 MB: 13.5 -> 13.9; Qwen heads,
-// 1500 tokens, B 2 / 4 / 8: 5.3 -> 3.9, 7.0 -> 4.6, 9.3 -> 6.4; B 16, 46 MB:
-// 10.2 -> 10.4), unless one row is so long that its warps finish far behind
-// the others (Qwen heads, 8 rows of 300 to 3800 tokens, 8 pages per warp:
-// 9.8 -> 7.8; 1 row of 32000, 32 pages per warp: 19.5 -> 21.5).
+// 6.5 -> 4.3, 8.0 -> 7.1, 10.2 -> 9.7; B 4, 52 MB: 12.0 -> 13.9; Qwen heads,
+// 1500 tokens, B 4 / 8: 7.0 -> 4.3, 8.4 -> 6.3; 16/8 heads of 500, B 20: 9.1 ->
+// 8.7; B 16 of 1400, 46 MB: 10.2 -> 10.4), unless one row is so long that its
+// warps finish far behind the others (Qwen heads, 8 rows of 300 to 3800
+// tokens, 8 pages per warp: 9.8 -> 7.8; 8/8 heads, 20 rows of 50 to 1500, 12
+// pages per warp: 12.1 -> 14.2; 1 row of 32000, 32 pages: 19.5 -> 21.5).
 //
 // Of the shapes, the one with the most warps per unit whose units all find a
 // slot at once, with a tenth to spare for the next launch's (LLaVA heads,
@@ -454,8 +455,9 @@ ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_
             if (10 * (int64_t)resident_clusters(device, D, gqa, sh) < 11 * units) continue;
             // pages of the longest row's warps against the layer's share of HBM time
             // the longest row's warps against what the layer's bytes take in
-            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB)
-            return per_warp * (D == 128 ? 4000000 : 2800000) <= 20000000 + bytes ? sh : ClusterShape{};
+            // any case: 3.5 pages of 4 MB (d = 64: 7 of 2 MB) and 1 more per
+            // 5.3 MB (2.7 MB) that the layer holds
+            return per_warp * (D == 128 ? 4000000 : 2000000) <= 14000000 + bytes * 3 / 4 ? sh : ClusterShape{};
         }
     }
     return ClusterShape{};
