@@ -75,6 +75,13 @@ int32_t kvd::auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, i
     return (int32_t)std::max(T, std::min<int64_t>(128, few));
 }
 
+int32_t kvd::chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T)
+{
+    const bool few_units = units * kChunkCap < warps;
+    if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
+    return gqa ? kChunkCapGqa : kChunkCap;
+}
+
 CUresult kvd::encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_t rows, int D,
                               int64_t v_stride_bytes)
 {
@@ -230,20 +237,6 @@ int push_updates(kv_cache* c, const std::vector<int32_t>& idx, const std::vector
 int64_t resident_warps(const kv_cache* c)
 {
     return (int64_t)std::max(1, c->num_sms) * std::max(1, c->variant.ctas_per_sm) * std::max(1, c->variant.warps);
-}
-
-// Items per row at most: twice the usual cap when rows x KV heads x the
-// usual cap would leave resident warps without an item and some row (of up
-// to max_pages pages) is long enough to use more items of T pages.
-// Otherwise 32 for MHA and 16 for GQA: a GQA row of at most 16 items merges
-// in one round trip with the 16-item variant, the largest whose registers
-// fit beside the resident GQA split pass (Qwen shape: 0.742 at 32, 0.769 at
-// 16, 0.756 at 24, 0.686 at 12).
-int32_t chunk_cap(const kv_cache* c, int64_t rows, int64_t max_pages, int32_t T)
-{
-    const bool few_units = rows * c->cfg.num_kv_heads * kChunkCap < resident_warps(c);
-    if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
-    return c->group > 1 ? kChunkCapGqa : kChunkCap;
 }
 
 int grow_scratch(kv_cache* c, int64_t entries, int64_t slots, int64_t page_ids, cudaStream_t st)
@@ -833,7 +826,7 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
     if (!c->split_override && !c->host_only)
         shape = cluster_shape(c->device, c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, batch,
                               total_units / c->cfg.num_kv_heads, max_np);
-    const int32_t cap = chunk_cap(c, batch, max_np, T);
+    const int32_t cap = chunk_cap(c->group > 1, (int64_t)batch * c->cfg.num_kv_heads, resident_warps(c), max_np, T);
     int64_t entries = 0;
     int32_t stride = 1;
     bool split = false;
@@ -1111,7 +1104,8 @@ int kv_cache_device_steps(kv_cache* c, int32_t max_batch, int32_t enable, void* 
                           ? c->split_override
                           : auto_item_pages(c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, resident_warps(c),
                                             c->dev_seqs, c->dev_pages, c->dev_row_pages, true);
-    const int32_t cap = chunk_cap(c, max_batch, c->cfg.max_pages_per_seq, T);
+    const int32_t cap = chunk_cap(c->group > 1, (int64_t)max_batch * c->cfg.num_kv_heads, resident_warps(c),
+                                  c->cfg.max_pages_per_seq, T);
     const int32_t entries = max_batch * cap;
     const int32_t stride = std::max(T, (c->cfg.max_pages_per_seq + cap - 1) / cap) + 1;
     if (int rc = grow_scratch(c, entries, (int64_t)entries * c->cfg.num_kv_heads, (int64_t)entries * stride, st))

@@ -299,6 +299,15 @@ CUresult encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_
 int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages, int64_t max_pages,
                         bool growing);
 
+// Items per row at most: twice the usual cap when units (rows x KV heads) x the
+// usual cap would leave resident warps without an item and some row (of up
+// to max_pages pages) is long enough to use more items of T pages.
+// Otherwise 32 for MHA and 16 for GQA: a GQA row of at most 16 items merges
+// in one round trip with the 16-item variant, the largest whose registers
+// fit beside the resident GQA split pass (Qwen shape: 0.742 at 32, 0.769 at
+// 16, 0.756 at 24, 0.686 at 12).
+int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T);
+
 // Message returned by kv_last_error() on the calling thread.
 void set_last_error(const char* msg);
 

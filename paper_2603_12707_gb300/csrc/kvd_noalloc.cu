@@ -264,7 +264,8 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     };
     const int64_t T_step =
         std::max<int64_t>(T, auto_item_pages(head_dim, G > 1, num_kv_heads, warps, batch, total_pages, max_np, false));
-    if (!cut(T_step, G > 1 ? kChunkCapGqa : kChunkCap, true) && !cut(T, kChunkCap, false))
+    const int cap = chunk_cap(G > 1, (int64_t)batch * num_kv_heads, warps, max_np, (int32_t)T_step);
+    if (!cut(T_step, cap, true) && !cut(T, kChunkCap, false))
         return fail(KVC_ERR_UNSUPPORTED, "the batch does not fit the static scratch");
     const int32_t entries = rt.off[batch];
     p.part_o = reinterpret_cast<float*>(scratch + off_part);

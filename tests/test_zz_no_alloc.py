@@ -210,6 +210,7 @@ def test_noalloc_rejects_what_does_not_fit(kvlib):
     (12, 12, 128, 30, 700),   # split pass and merge pass, rows in the small table
     (28, 4, 128, 70, 900),    # the large table
     (8, 8, 64, 200, 32),      # more items than warps, no row split: no merge pass
+    (16, 8, 128, 2, 7000),    # few units: rows of up to 64 items, the four-warp merge
 ])
 def test_noalloc_pool_layouts_and_row_tables(kvlib, Hq, Hkv, d, B, longest, layout):
     """K and V pools in either order (one tensor map over both) and at a
