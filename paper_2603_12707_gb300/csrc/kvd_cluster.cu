@@ -115,7 +115,9 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int W = blockDim.x >> 5, R = p.ring;
     const int C = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
-    const int log_dc = 31 - __clz(D / C);                                       // C is a power of two
+    // CTAs and warps of a unit are powers of two: shifts in place of divisions,
+    // which cost the entry of a kernel this short.
+    const int log_dc = 31 - __clz(D / C), log_cw = 31 - __clz(C * W);
     uint8_t* ring = smem + warp * R * STAGE;
     float* recv = reinterpret_cast<float*>(smem + W * R * STAGE);               // [C][G][D / C]
     float2* recv_ml = reinterpret_cast<float2*>(reinterpret_cast<uint8_t*>(recv) + Cg::kRecv);   // [C][heads]
@@ -131,12 +133,12 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     bool waited = p.early == 0;
     if (waited) griddep_wait();
     griddep_launch_dependents();
-    const int unit = (int)blockIdx.x / C;
-    const int b = unit / p.H_kv, g = unit - b * p.H_kv;
+    const int b = blockIdx.y, g = (int)blockIdx.x >> (31 - __clz(C));
     int2 row;   // (page-table row, tokens attended)
     if constexpr (Rows::kTable) row = make_int2(b, rt.len[b]);
     else row = p.rows[b];   // by the step kernel; no tokens: the row's step failed
     if (lane == 0) {
+#pragma unroll 1
         for (int s = 0; s < R; ++s) mbar_init(smem_addr(&bars[s]), 1);
         if (warp == 0) mbar_init(smem_addr(recv_bar), 1);
         fence_mbar_init();
@@ -150,8 +152,8 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     cluster_arrive();   // "ready to receive": waited for before the first write to another CTA
     const int len = row.y;
     const int np = (len + kPageSize - 1) / kPageSize;
-    int first, n;
-    chunk_range(np, C * W, rank * W + warp, &first, &n);
+    const int at = rank * W + warp, each = np >> log_cw, more = np & ((1 << log_cw) - 1);   // chunk_range
+    const int first = at * each + min(at, more), n = each + (at < more ? 1 : 0);
     const bool has_last = n > 0 && first + n == np;
     const int32_t* pt_row = p.page_table + (int64_t)row.x * p.max_pages + first;
     auto load_window = [&](int w0) { return (w0 + lane < n) ? pt_row[w0 + lane] : 0; };
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
         const uint32_t dst = ring_s + s * STAGE;
         const int32_t y = (pid * p.H_kv + g) * kPageSize;
         mbar_arrive_expect_tx(bar, STAGE);
-        if (p.kv_map) {
+        if (!Rows::kTable || p.kv_map) {
             tma_load_4d(dst, &tmk, 0, y, 0, 0, bar, policy);
         } else {
             tma_load_3d(dst, &tmk, 0, y, 0, bar, policy);
@@ -183,11 +185,11 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     const int pre = min(n, R);
     // lane i: page i into stage i (after a kv_append a row's last page only
     // once that is complete)
-    const bool late_page = p.hold_last && has_last && n == pre;
+    const bool late_page = !FUSED && p.hold_last && has_last && n == pre;
     if (lane < pre - (late_page ? 1 : 0)) load(pid_cur, lane);
     // The pages past the ring into L2: when a stage is free again its next
     // page is an L2 round trip away.
-    if (p.kv_map) {
+    if (!Rows::kTable || p.kv_map) {
         const int end = min(min(n, 32), R + kClusterL2Pages);
         if (lane >= R && lane < end && pid_cur >= 0 && pid_cur < p.num_pages)
             tma_prefetch_l2_4d(&tmk, 0, (pid_cur * p.H_kv + g) * kPageSize, 0, 0);
@@ -216,7 +218,8 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     bool ok = true;
     // Wait for page j in stage s and put the new token into it if it is the row's last.
     auto arrived = [&](int j, int s) {
-        const bool w = mbar_wait_bounded(smem_addr(&bars[s]), (phase >> s) & 1u, kWaitLimitNs);
+        const uint32_t bar = smem_addr(&bars[s]), parity = (phase >> s) & 1u;
+        const bool w = mbar_try_wait_cluster(bar, parity) || mbar_wait_bounded_cluster(bar, parity, kWaitLimitNs);
         if (!__all_sync(0xffffffffu, w)) return false;
         phase ^= 1u << s;
         pending &= ~(1u << s);
@@ -236,6 +239,7 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     };
     auto after = [&](int s) { return s + 1 == R ? 0 : s + 1; };
     auto tokens = [&](int j) { return min(kPageSize, len - (first + j) * kPageSize); };
+#pragma unroll 1
     for (int j = 0, s = 0; ok && j < n; ++j) {
         ok = arrived(j, s);
         if (!ok) break;
@@ -249,8 +253,9 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     }
     if (!ok) {   // let the loads in flight land: their stages are about to be reused
         if (lane == 0) atomicOr(p.err, 2);
+#pragma unroll 1
         for (int i = 0; i < R; ++i)
-            if (pending & (1u << i)) mbar_wait_bounded(smem_addr(&bars[i]), (phase >> i) & 1u, kWaitLimitNs);
+            if (pending & (1u << i)) mbar_wait_bounded_cluster(smem_addr(&bars[i]), (phase >> i) & 1u, kWaitLimitNs);
     }
     __syncwarp();
 
@@ -260,6 +265,7 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     __syncthreads();
     cluster_wait();
     const uint32_t bar_s = smem_addr(recv_bar);
+#pragma unroll 1
     for (int i = threadIdx.x; i < G * (D / 4); i += blockDim.x) {
         const int h = i / (D / 4), d0 = (i % (D / 4)) * 4;
         // (fixed bounds, so that every load goes out before the first use)
@@ -295,12 +301,13 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
         // every CTA gets (M, L) of each head, from the thread of its first dims
         if (dd == 0) cluster_store_async2(cluster_map(smem_addr(recv_ml + rank * Cg::kHeads + h), dst), M, L, bar);
     }
-    if (!mbar_wait_bounded_cluster(bar_s, 0, kWaitLimitNs)) {
+    if (!mbar_try_wait_cluster(bar_s, 0) && !mbar_wait_bounded_cluster(bar_s, 0, kWaitLimitNs)) {
         atomicOr(p.err, 2);
         return;
     }
     // Hop 2: this CTA's dims over the cluster, two at a time.
     if (np == 0) return;   // a row whose step failed: its output is left alone
+#pragma unroll 1
     for (int i = threadIdx.x; i < G << (log_dc - 1); i += blockDim.x) {
         const int h = i >> (log_dc - 1), d0 = (i & ((1 << (log_dc - 1)) - 1)) * 2;
         float2 ml[kClusterMaxCtas], v[kClusterMaxCtas];
@@ -339,12 +346,12 @@ cudaError_t prepare_cluster()
 }
 
 template <int D, bool GQA, bool FUSED, class Rows>
-cudaError_t launch_variant(bool pdl, const ClusterShape& sh, int units, const CUtensorMap& tk, const CUtensorMap& tv,
+cudaError_t launch_variant(bool pdl, const ClusterShape& sh, const CUtensorMap& tk, const CUtensorMap& tv,
                            const DecodeParams& p, const Rows& rows, cudaStream_t st)
 {
     if (cudaError_t e = prepare_cluster<D, GQA, FUSED, Rows>(); e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(units * sh.ctas));
+    cfg.gridDim = dim3((unsigned)(p.H_kv * sh.ctas), (unsigned)p.batch);
     cfg.blockDim = dim3((unsigned)(sh.warps * 32));
     cfg.dynamicSmemBytes = (size_t)ClusterGeo<D, GQA>::smem(sh.warps, sh.ring);
     cfg.stream = st;
@@ -360,12 +367,12 @@ cudaError_t launch_variant(bool pdl, const ClusterShape& sh, int units, const CU
 }
 
 template <int D, bool GQA>
-cudaError_t launch_shape(bool fused, bool pdl, const ClusterShape& sh, int units, const CUtensorMap& tk,
+cudaError_t launch_shape(bool fused, bool pdl, const ClusterShape& sh, const CUtensorMap& tk,
                          const CUtensorMap& tv, const DecodeParams& p, const LensTable* lens, cudaStream_t st)
 {
-    if (lens) return launch_variant<D, GQA, false>(pdl, sh, units, tk, tv, p, *lens, st);
-    return fused ? launch_variant<D, GQA, true>(pdl, sh, units, tk, tv, p, PlanRows{}, st)
-                 : launch_variant<D, GQA, false>(pdl, sh, units, tk, tv, p, PlanRows{}, st);
+    if (lens) return launch_variant<D, GQA, false>(pdl, sh, tk, tv, p, *lens, st);
+    return fused ? launch_variant<D, GQA, true>(pdl, sh, tk, tv, p, PlanRows{}, st)
+                 : launch_variant<D, GQA, false>(pdl, sh, tk, tv, p, PlanRows{}, st);
 }
 
 template <int D, bool GQA>
@@ -407,14 +414,14 @@ int resident_clusters(int device, int D, bool gqa, const ClusterShape& sh)
 
 }  // namespace
 
-cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& sh, int units,
+cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& sh,
                            const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p,
                            const LensTable* lens, cudaStream_t st)
 {
-    if (D == 128) return gqa ? launch_shape<128, true>(fused, pdl, sh, units, tk, tv, p, lens, st)
-                             : launch_shape<128, false>(fused, pdl, sh, units, tk, tv, p, lens, st);
-    if (D == 64) return gqa ? launch_shape<64, true>(fused, pdl, sh, units, tk, tv, p, lens, st)
-                            : launch_shape<64, false>(fused, pdl, sh, units, tk, tv, p, lens, st);
+    if (D == 128) return gqa ? launch_shape<128, true>(fused, pdl, sh, tk, tv, p, lens, st)
+                             : launch_shape<128, false>(fused, pdl, sh, tk, tv, p, lens, st);
+    if (D == 64) return gqa ? launch_shape<64, true>(fused, pdl, sh, tk, tv, p, lens, st)
+                            : launch_shape<64, false>(fused, pdl, sh, tk, tv, p, lens, st);
     return cudaErrorInvalidValue;
 }
 
@@ -426,7 +433,8 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
 // 1500 tokens, B 4 / 8: 7.0 -> 4.3, 8.4 -> 6.3; 16/8 heads of 500, B 20: 9.1 ->
 // 8.7; B 16 of 1400, 46 MB: 10.2 -> 10.4), unless one row is so long that its
 // warps finish far behind the others (Qwen heads, 8 rows of 300 to 3800
-// tokens, 8 pages per warp: 9.8 -> 7.8; 8/8 heads, 20 rows of 50 to 1500, 12
+// tokens, 8 pages per warp: 9.8 -> 7.8; 7 of 300 to 4300, 24 MB, 9 pages: 9.3 ->
+// 8.1; 8/8 heads, 20 rows of 50 to 1500, 12
 // pages per warp: 12.1 -> 14.2; 1 row of 32000, 32 pages: 19.5 -> 21.5).
 //
 // Of the shapes, the one with the most warps per unit whose units all find a
@@ -455,9 +463,10 @@ ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_
             if (10 * (int64_t)resident_clusters(device, D, gqa, sh) < 11 * units) continue;
             // pages of the longest row's warps against the layer's share of HBM time
             // the longest row's warps against what the layer's bytes take in
-            // any case: 3.5 pages of 4 MB (d = 64: 7 of 2 MB) and 1 more per
-            // 5.3 MB (2.7 MB) that the layer holds
-            return per_warp * (D == 128 ? 4000000 : 2000000) <= 14000000 + bytes * 3 / 4 ? sh : ClusterShape{};
+            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB) that
+            // the layer holds, up to 25 MB, which keep the HBM busy beside them
+            const int64_t beside = std::min<int64_t>(bytes, 25000000);
+            return per_warp * (D == 128 ? 4000000 : 2800000) <= 20000000 + beside ? sh : ClusterShape{};
         }
     }
     return ClusterShape{};

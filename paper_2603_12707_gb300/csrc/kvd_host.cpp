@@ -1016,7 +1016,7 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
         p.num_sms = c->num_sms;
         c->last_stream = static_cast<cudaStream_t>(stream);
         KVD_CUDA(launch_cluster(c->cfg.head_dim, c->group > 1, fused, pdl || after_step, c->step_cluster,
-                                batch * c->cfg.num_kv_heads, c->tmaps[layer], c->tmaps[layer], p,
+                                c->tmaps[layer], c->tmaps[layer], p,
                                 nullptr, static_cast<cudaStream_t>(stream)));
         ++c->launches;
         c->prev_merge = false;

@@ -352,7 +352,7 @@ cudaError_t launch_decode(int D, bool gqa, bool fused, bool pdl, int grid, const
 // Decode attention with one cluster per (row, KV head) unit, no second pass
 // (kvd_cluster.cu).  pdl: launched with programmatic dependent launch.
 // lens: the rows' lengths as parameters (batch <= kLensRows), or null: p.rows.
-cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& shape, int units,
+cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterShape& shape,
                            const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p,
                            const LensTable* lens, cudaStream_t st);
 // Clusters for `batch` rows of num_kv_heads that hold `pages` pages per KV

@@ -229,7 +229,7 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
         LensTable lt;
         std::copy_n(lens, batch, lt.len);
         p.ring = shape.ring;
-        if (cudaError_t e = launch_cluster(head_dim, G > 1, false, false, shape, batch * num_kv_heads, maps[0], maps[1], p,
+        if (cudaError_t e = launch_cluster(head_dim, G > 1, false, false, shape, maps[0], maps[1], p,
                                            &lt, st);
             e != cudaSuccess)
             return fail(KVC_ERR_CUDA, cudaGetErrorString(e));

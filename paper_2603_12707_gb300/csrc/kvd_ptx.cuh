@@ -184,20 +184,27 @@ __device__ __forceinline__ void cluster_store_async2(uint32_t addr, float a, flo
                  : "memory");
 }
 
-// mbar_wait_bounded with acquire semantics over the cluster.
-__device__ __forceinline__ bool mbar_wait_bounded_cluster(uint32_t bar, uint32_t parity, uint64_t limit_ns)
+// mbar_try_wait with acquire semantics over the cluster.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// mbar_wait_bounded with acquire semantics over the cluster, the loop out of
+// line: it serves every wait of a kernel whose size counts.
+static __device__ __noinline__ bool mbar_wait_bounded_cluster(uint32_t bar, uint32_t parity, uint64_t limit_ns)
 {
     const uint64_t t0 = global_timer_ns();
     while (true) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
+        if (mbar_try_wait_cluster(bar, parity)) return true;
         if (global_timer_ns() - t0 > limit_ns) return false;
     }
 }
