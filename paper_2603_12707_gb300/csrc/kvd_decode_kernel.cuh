@@ -575,34 +575,45 @@ __global__ void __launch_bounds__(kWarps * 32)
         const PlanEntry en = Rows::kTable ? found : p.plan[e];
         const int np = en.n_pages;
 
+        auto load = [&](int32_t pid, int s) {   // page pid into stage s, by one lane
+            if (pid < 0 || pid >= p.num_pages) {
+                atomicOr(p.err, 1);
+                pid = 0;
+            }
+            const uint32_t bar = smem_addr(&bars[s]);
+            const uint32_t dst = ring_s + s * STAGE;
+            const int32_t y = (pid * p.H_kv + g) * kPageSize;
+            mbar_arrive_expect_tx(bar, STAGE);
+            if (!Rows::kTable || p.kv_map) {
+                tma_load_4d(dst, &tmk, 0, y, 0, 0, bar, policy);
+            } else {
+                tma_load_3d(dst, &tmk, 0, y, 0, bar, policy);
+                tma_load_3d(dst + TILE, &tmv, 0, y, 0, bar, policy);
+            }
+        };
         auto issue = [&](int j, int s) {
             if ((j & 31) == 8 && j + 24 < np) pid_next = load_window(j + 24);
             if ((j & 31) == 0 && j > 0) pid_cur = pid_next;
-            int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
-            if (pid < 0 || pid >= p.num_pages) {
-                if (lane == 0) atomicOr(p.err, 1);
-                pid = 0;
-            }
-            if (lane == 0) {
-                const uint32_t bar = smem_addr(&bars[s]);
-                const uint32_t dst = ring_s + s * STAGE;
-                const int32_t y = (pid * p.H_kv + g) * kPageSize;
-                mbar_arrive_expect_tx(bar, STAGE);
-                if (p.kv_map) {
-                    tma_load_4d(dst, &tmk, 0, y, 0, 0, bar, policy);
-                } else {
-                    tma_load_3d(dst, &tmk, 0, y, 0, bar, policy);
-                    tma_load_3d(dst + TILE, &tmv, 0, y, 0, bar, policy);
-                }
-            }
+            const int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
+            if (lane == 0) load(pid, s);
         };
 
+        // Pages j0 .. j1-1 (of the first window) into L2, one per lane; a bad
+        // page id is recorded when its load is issued.
+        auto prefetch = [&](int j0, int j1) {
+            if (lane >= j0 && lane < min(np, j1))
+                tma_prefetch_l2_4d(&tmk, 0, ((pid_cur < 0 || pid_cur >= p.num_pages ? 0 : pid_cur) * p.H_kv + g) * kPageSize,
+                                   0, 0);
+            __syncwarp();
+        };
         const bool last_chunk = en.chunk == en.n_chunks - 1;
         const int pre = np < R ? np : R;
         // After a kv_append a row's last page is loaded only once that is complete.
         const bool hold = !FUSED && !waited && p.hold_last && last_chunk && np == pre;
         __syncwarp();
-        for (int j = 0; j < pre - (hold ? 1 : 0); ++j) issue(j, j);
+        // lane i: page i into stage i
+        if (lane < pre - (hold ? 1 : 0)) load(pid_cur, lane);
+        __syncwarp();
         pending = (1u << pre) - 1u;
         int ramp0 = R;   // first page of the L2 ramp at the wait's return
         if (!waited && p.prev_tag && np > R && p.kv_map) {
@@ -618,11 +629,7 @@ __global__ void __launch_bounds__(kWarps * 32)
                 __nanosleep(128);
             }
             if (seen) {
-                for (int j = R; j < np && j < R + kEarlyL2Pages; ++j) {
-                    int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
-                    if (pid < 0 || pid >= p.num_pages) pid = 0;   // recorded when its load is issued
-                    if (lane == 0) tma_prefetch_l2_4d(&tmk, 0, (pid * p.H_kv + g) * kPageSize, 0, 0);
-                }
+                prefetch(R, R + kEarlyL2Pages);
                 ramp0 = R + kEarlyL2Pages;
             }
         }
@@ -630,16 +637,13 @@ __global__ void __launch_bounds__(kWarps * 32)
             griddep_wait();
             griddep_launch_dependents();
             waited = true;
-            if (hold) issue(pre - 1, pre - 1);
+            if (hold && lane == pre - 1) load(pid_cur, lane);
+            __syncwarp();
         }
         if (first_item && p.kv_map) {
             // The ring holds this item's first R pages (loaded before the
             // wait when chained); the next ones go into L2 now.
-            for (int j = ramp0; j < np && j < ramp0 + kRampL2Pages; ++j) {
-                int32_t pid = __shfl_sync(0xffffffffu, pid_cur, j & 31);
-                if (pid < 0 || pid >= p.num_pages) pid = 0;   // recorded when its load is issued
-                if (lane == 0) tma_prefetch_l2_4d(&tmk, 0, (pid * p.H_kv + g) * kPageSize, 0, 0);
-            }
+            prefetch(ramp0, ramp0 + kRampL2Pages);
         }
         first_item = false;
         comp.start(p, en, g, lane);
