@@ -130,7 +130,8 @@ KVC_API int kv_cache_pool(kv_cache *cache, int32_t layer, void **k_pool, void **
  * used by later kv_begin_step calls; 0 restores the automatic choice.
  * Range 0 .. 1024.  A row of n pages is cut into ceil(n / T') items of
  * near-equal size, T' = max(T, ceil(n / 32)): never more than 32 items per
- * (sequence, KV head). */
+ * (sequence, KV head).  With an override every step runs from a split plan;
+ * the automatic choice runs small steps without one (decode_attention). */
 KVC_API int kv_cache_set_split_pages(kv_cache *cache, int32_t pages);
 
 /* -------------------------------------------------------- sequences ------ */
@@ -236,7 +237,11 @@ KVC_API int kv_append(kv_cache *cache, int32_t layer, int32_t batch, const void 
  * work items of consecutive pages; each item runs an online softmax in fp32
  * over its pages for all G query heads of the KV head, and a second kernel
  * merges the partial results of every (sequence, KV head) cut into several
- * items by log-sum-exp. */
+ * items by log-sum-exp.  A step with little to read (up to about 45 MB of K
+ * and V per layer; kv_begin_step decides by the step's lengths,
+ * kv_begin_step_device by those held when device steps were enabled) has no
+ * plan: one thread-block cluster per (sequence, KV head) does both in one
+ * launch. */
 KVC_API int decode_attention(kv_cache *cache, int32_t layer, int32_t batch, const void *q, void *out,
                      float softmax_scale, void *stream);
 
@@ -331,8 +336,8 @@ KVC_API int kv_cache_sync(kv_cache *cache);
  * still do not fit at 1024 pages.  The first call on
  * each device looks up the array's device address (cudaGetSymbolAddress);
  * make that first call before any stream capture.  Every call uses the same
- * array and clears the counters it needs at its start, so calls that overlap
- * on the GPU race: order them on one stream.  Same shape limits as
+ * array and leaves its work counter at zero, as it found it, so calls that
+ * overlap on the GPU race: order them on one stream.  Same shape limits as
  * kv_cache_create (head_dim 64 or 128, G <= 8, 16-token pages). */
 KVC_API int decode_attention_noalloc(const void *k_pool, const void *v_pool, int64_t num_pages,
                                      int32_t num_q_heads, int32_t num_kv_heads, int32_t head_dim,

@@ -12,7 +12,11 @@
 // What bounds it: such a layer holds a few MB, 1-2 us of HBM time, so the
 // chain of dependent latencies per layer decides.  The split pass and merge
 // pass pay two dependency hops (~1 us each) and two L2 round trips for the
-// partials; this kernel pays one hop and a cluster barrier.
+// partials; this kernel pays one hop and one exchange over the cluster (sent
+// with st.async, received on an mbarrier: 0.4 us less than a cluster
+// barrier).  us per chained layer, split plan -> this: LLaVA heads, one
+// request of 850 tokens (14 MB) 6.5 -> 4.3; Qwen heads, two of 2500 and 4400
+// (14 MB) 6.9 -> 5.0; 4 requests of 100 tokens, 8/8 heads, d = 64: 4.6 -> 2.5.
 #include <algorithm>
 #include <atomic>
 

@@ -3,10 +3,11 @@
 // Schedule.  A step's plan cuts every (sequence, KV head) into work items of
 // consecutive pages.  A persistent grid of warps pulls items from a global
 // counter; each warp runs its items independently:
-//   * one lane streams the (page, head) tiles of K and V into the warp's
-//     private ring of R shared-memory stages, one 4-D TMA tile load per page
-//     covering K and V (128-byte swizzle, L2 evict-first), completing on one
-//     mbarrier per stage;
+//   * the (page, head) tiles of K and V stream into the warp's private ring of
+//     R shared-memory stages, one 4-D TMA tile load per page covering K and V
+//     (128-byte swizzle, L2 evict-first), completing on one mbarrier per
+//     stage; lane i issues the item's page i < R, lane 0 the later ones (one
+//     lane for all took ~0.2 us a load: Qwen-shaped step 0.7 % longer);
 //   * the warp computes an online softmax over the item's tokens for the G
 //     query heads of the KV head (reference max m in log2 units, running sum
 //     l = sum 2^(s - m), unnormalised accumulator o, all fp32; m trails the
