@@ -9,6 +9,7 @@ fallback implementation.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 
@@ -106,6 +107,8 @@ def load():
 def _ptr(x):
     if x is None:
         return None
+    if isinstance(x, array.array):
+        return x.buffer_info()[0]
     if hasattr(x, "data_ptr"):
         return x.data_ptr()
     if isinstance(x, ctypes.Array):
@@ -127,8 +130,15 @@ def _check(rc: int, fn: str):
 
 
 def _i32_array(values):
-    vals = [int(v) for v in values]
-    return (ctypes.c_int32 * len(vals))(*vals)
+    """The values as C int32s (``_ptr`` takes the result).  Integers are
+    converted in one C call (32 of them: 0.6 us, 4.1 one by one); anything
+    else goes through int()."""
+    values = values if isinstance(values, (list, tuple)) else list(values)
+    try:
+        return array.array("i", values)
+    except (TypeError, OverflowError):
+        vals = [int(v) for v in values]
+        return (ctypes.c_int32 * len(vals))(*vals)
 
 
 # ---------------------------------------------------------------- C names
@@ -144,7 +154,7 @@ def kv_cache_destroy(h):
 
 def kv_cache_set_page_order(h, order):
     arr = _i32_array(order)
-    _check(load().kv_cache_set_page_order(h, ctypes.addressof(arr), len(arr)), "kv_cache_set_page_order")
+    _check(load().kv_cache_set_page_order(h, _ptr(arr), len(arr)), "kv_cache_set_page_order")
 
 
 def kv_cache_query(h, raise_on_device_error: bool = True) -> kvc_stats:
@@ -211,14 +221,12 @@ def kv_write_varlen(h, layer_first: int, n_layers: int, seq_ids, cu_seqlens, k, 
     fp = _i32_array(first_pos) if first_pos is not None else None
     if fp is not None and len(fp) != len(ids):
         raise ValueError("first_pos needs len(seq_ids) entries")
-    _check(load().kv_write_varlen(h, layer_first, n_layers, len(ids), ctypes.addressof(ids),
-                                  ctypes.addressof(fp) if fp is not None else None, ctypes.addressof(cu),
-                                  _ptr(k), _ptr(v), _stream(stream)), "kv_write_varlen")
+    _check(load().kv_write_varlen(h, layer_first, n_layers, len(ids), _ptr(ids), _ptr(fp), _ptr(cu), _ptr(k), _ptr(v), _stream(stream)), "kv_write_varlen")
 
 
 def kv_begin_step(h, seq_ids, stream=None):
     arr = _i32_array(seq_ids)
-    _check(load().kv_begin_step(h, len(arr), ctypes.addressof(arr), _stream(stream)), "kv_begin_step")
+    _check(load().kv_begin_step(h, len(arr), _ptr(arr), _stream(stream)), "kv_begin_step")
 
 
 def kv_append(h, layer: int, batch: int, k_new, v_new, stream=None):
@@ -236,6 +244,17 @@ def decode_attention_append(h, layer: int, batch: int, q, k_new, v_new, out, sof
                                           float(softmax_scale), _stream(stream)), "decode_attention_append")
 
 
+def _check_tensor(x, name, dtype, shape, min_numel):
+    if not hasattr(x, "data_ptr"):
+        return
+    if x.dtype is not dtype or not x.is_cuda or not x.is_contiguous():
+        raise ValueError(f"{name} must be a contiguous CUDA tensor of {dtype}")
+    if shape is not None and x.shape != shape:
+        raise ValueError(f"{name} must have shape {tuple(shape)}, not {tuple(x.shape)}")
+    if x.numel() < min_numel:
+        raise ValueError(f"{name} holds {x.numel()} elements, fewer than {min_numel}")
+
+
 def decode_attention_noalloc(k_pool, v_pool, num_pages: int, num_q_heads: int, num_kv_heads: int,
                              head_dim: int, page_table, max_pages: int, lens, q, out,
                              softmax_scale: float = 0.0, device_error=None, stream=None):
@@ -249,28 +268,19 @@ def decode_attention_noalloc(k_pool, v_pool, num_pages: int, num_q_heads: int, n
     num_pages * num_kv_heads * 16 * head_dim elements, device_error int32."""
     arr = _i32_array(lens)
     batch = len(arr)
-
-    def _tensor(x, name, dtype, shape=None, min_numel=None):
-        if not hasattr(x, "data_ptr"):
-            return
-        if x.dtype != dtype or not x.is_cuda or not x.is_contiguous():
-            raise ValueError(f"{name} must be a contiguous CUDA tensor of {dtype}")
-        if shape is not None and tuple(x.shape) != tuple(shape):
-            raise ValueError(f"{name} must have shape {tuple(shape)}, not {tuple(x.shape)}")
-        if min_numel is not None and x.numel() < min_numel:
-            raise ValueError(f"{name} holds {x.numel()} elements, fewer than {min_numel}")
-
     import torch
-    _tensor(page_table, "page_table", torch.int32, (batch, max_pages))
-    _tensor(q, "q", torch.bfloat16, (batch, num_q_heads, head_dim))
-    _tensor(out, "out", torch.bfloat16, (batch, num_q_heads, head_dim))
+    rows = (batch, num_q_heads, head_dim)
     pool_elems = int(num_pages) * int(num_kv_heads) * 16 * int(head_dim)
-    _tensor(k_pool, "k_pool", torch.bfloat16, min_numel=pool_elems)
-    _tensor(v_pool, "v_pool", torch.bfloat16, min_numel=pool_elems)
-    _tensor(device_error, "device_error", torch.int32, min_numel=1)
+    _check_tensor(page_table, "page_table", torch.int32, (batch, max_pages), 0)
+    _check_tensor(q, "q", torch.bfloat16, rows, 0)
+    _check_tensor(out, "out", torch.bfloat16, rows, 0)
+    _check_tensor(k_pool, "k_pool", torch.bfloat16, None, pool_elems)
+    _check_tensor(v_pool, "v_pool", torch.bfloat16, None, pool_elems)
+    if device_error is not None:
+        _check_tensor(device_error, "device_error", torch.int32, None, 1)
     _check(load().decode_attention_noalloc(_ptr(k_pool), _ptr(v_pool), num_pages, num_q_heads, num_kv_heads,
                                            head_dim, batch, _ptr(page_table), max_pages,
-                                           ctypes.addressof(arr), _ptr(q), _ptr(out), float(softmax_scale),
+                                           _ptr(arr), _ptr(q), _ptr(out), float(softmax_scale),
                                            _ptr(device_error), _stream(stream)),
            "decode_attention_noalloc")
 

@@ -256,3 +256,26 @@ def test_noalloc_object_references_no_allocator(kvlib):
     bad = [l for l in r.stdout.splitlines()
            if any(s in l for s in ("cudaMalloc", "cudaFree", "cuMemAlloc", "cuMemFree", "cuMemCreate"))]
     assert not bad, bad
+
+
+def test_integer_lists_reach_the_library_as_int32():
+    """The binding converts lists of integers in one call and anything else
+    through int(), as C int32s either way (wrapped like a C cast)."""
+    import ctypes
+
+    import numpy as np
+
+    def seen(values):
+        arr = kd._i32_array(values)
+        n = len(arr)
+        return list((ctypes.c_int32 * n).from_address(kd._ptr(arr))) if n else []
+
+    assert seen([1, -2, 2**31 - 1, -2**31]) == [1, -2, 2**31 - 1, -2**31]
+    assert seen((3, True)) == [3, 1]
+    assert seen(range(4)) == [0, 1, 2, 3]
+    assert seen(np.array([5, 6], np.int64)) == [5, 6]
+    assert seen([np.int32(7), np.uint16(8)]) == [7, 8]
+    assert seen(np.array([1.0, 2.9])) == [1, 2]
+    assert seen(iter([4, 5])) == [4, 5]
+    assert seen([2**32 + 9, 1]) == [9, 1]
+    assert seen([]) == []
