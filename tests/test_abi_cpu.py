@@ -263,7 +263,7 @@ def test_integer_lists_reach_the_library_as_int32():
     through int(), as C int32s either way (wrapped like a C cast)."""
     import ctypes
 
-    import numpy as np
+    from paper_2603_12707_gb300 import kvdecode as kd
 
     def seen(values):
         arr = kd._i32_array(values)
