@@ -252,16 +252,17 @@ KVC_API int decode_attention(kv_cache *cache, int32_t layer, int32_t batch, cons
  * result and cache contents as kv_append followed by decode_attention.
  * When the library's previous launch on `stream` was an attention launch
  * (decode_attention or decode_attention_append of this cache) or a
- * kv_append, the kernel is
- * launched with programmatic dependent launch: it may start, and stream this
- * layer's cached pages (positions < s_b), while that launch is finishing; it
- * reads q, k_new and v_new and writes anything only after the kernel before
- * it has completed.  After any other call of this library it is an ordinary
- * launch.  The same holds for decode_attention (which, after a kv_append,
- * reads each row's last page only once that has completed) and for kv_append
- * (which reads and writes nothing before the kernel before it has).  So a kernel the caller enqueues between two layers must not write
- * the cache's pages (a foreign kernel could only race with the early reads
- * if it signalled its dependents early). */
+ * kv_append, the kernel is launched with programmatic dependent launch: it
+ * may start, and stream this layer's cached pages (positions < s_b), while
+ * that launch is finishing; it reads q, k_new and v_new and writes anything
+ * only after the kernel before it has completed.  After any other call of
+ * this library it is an ordinary launch.  The same holds for decode_attention
+ * (which, where a launch chained before it appended tokens, reads each row's
+ * last page only once that has completed) and for kv_append (which reads and
+ * writes nothing before the kernel before it has).  So a kernel the caller
+ * enqueues between two layers must not write the cache's pages (a foreign
+ * kernel could only race with the early reads if it signalled its dependents
+ * early). */
 KVC_API int decode_attention_append(kv_cache *cache, int32_t layer, int32_t batch, const void *q,
                                     const void *k_new, const void *v_new, void *out,
                                     float softmax_scale, void *stream);

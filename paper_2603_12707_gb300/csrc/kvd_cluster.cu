@@ -131,8 +131,9 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     const uint32_t ring_s = smem_addr(ring);
     int G = GQA ? p.G : 1;
 
-    // The next launch may start at once: it reads nothing this one writes
-    // before its own dependency wait (but for slots that it replaces).  After
+    // The next launch may start at once, with this one still waiting: before
+    // its own dependency wait it reads nothing that this launch or the chain
+    // before it writes (but for slots that it replaces itself).  After
     // a step kernel both wait for that first.
     bool waited = p.early == 0;
     if (waited) griddep_wait();
@@ -187,8 +188,8 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
         if (lane == 0) load(pid, s);
     };
     const int pre = min(n, R);
-    // lane i: page i into stage i (after a kv_append a row's last page only
-    // once that is complete)
+    // lane i: page i into stage i (a row's last page only after the wait where
+    // an append of the chain may be under way)
     const bool late_page = !FUSED && p.hold_last && has_last && n == pre;
     if (lane < pre - (late_page ? 1 : 0)) load(pid_cur, lane);
     // The pages past the ring into L2: when a stage is free again its next

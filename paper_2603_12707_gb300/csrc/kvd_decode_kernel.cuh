@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(kWarps * 32)
     Comp comp;
     // Chained launches depend programmatically on the previous kernel: until
     // griddep_wait() only the plan, page table and cache pages (none of which
-    // that kernel writes, but for a kv_append each row's last page) are read;
+    // it or the chain before it writes, but for each row's last page) are read;
     // q, k_new, v_new and every write come after.
     bool waited = false;
     bool first_item = true;
@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(kWarps * 32)
         };
         const bool last_chunk = en.chunk == en.n_chunks - 1;
         const int pre = np < R ? np : R;
-        // After a kv_append a row's last page is loaded only once that is complete.
+        // Where an append may be under way a row's last page is loaded only once that is complete.
         const bool hold = !FUSED && !waited && p.hold_last && last_chunk && np == pre;
         __syncwarp();
         // lane i: page i into stage i

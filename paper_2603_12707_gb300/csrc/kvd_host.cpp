@@ -140,7 +140,7 @@ struct kv_cache {
     void* step_stream = nullptr;
     int64_t seq_launches = -1;                  // the same for reservations, releases and token copies
     cudaStream_t seq_stream = nullptr;
-    bool chain_append = false;                  // a kv_append since the last attention launch
+    bool chain_append = false;                  // this chain holds a launch that writes new tokens
     int32_t* err = nullptr;
     PlanEntry* plan = nullptr;
     int64_t plan_cap = 0;
@@ -1008,8 +1008,12 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     // After the step kernel: placed while it runs, reads nothing before its end.
     const bool after_step = !pdl && c->step_launches == c->launches && c->step_stream == stream;
     p.early = after_step ? 0 : 1;
+    // A launch that appends nothing itself loads each row's last page after its
+    // wait if any launch of the chain wrote new tokens, kv_append or fused and
+    // however far back: a cluster launch lets the next one start before its own
+    // wait, so that writer need not have completed.
     p.hold_last = pdl && !fused && c->chain_append ? 1 : 0;
-    c->chain_append = false;
+    c->chain_append = fused || (pdl && c->chain_append);
     if (c->step_cluster.ctas) {
         p.ring = c->step_cluster.ring;
         p.start_flags = nullptr;

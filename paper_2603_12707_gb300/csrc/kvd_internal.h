@@ -260,7 +260,7 @@ struct DecodeParams {
     // cluster_kernel only: it reads lengths and page ids by batch row instead of a plan.
     int32_t ring;             // shared-memory stages per warp
     int32_t early;            // 1: plan and cache may be read before the dependency wait (0: after a step kernel)
-    int32_t hold_last;        // 1: but not each row's last page (a kv_append may be writing it)
+    int32_t hold_last;        // 1: but not each row's last page (a launch of the chain may be writing it)
 };
 
 // Clusters of a step with few (sequence, KV head) units: CTAs per unit, warps

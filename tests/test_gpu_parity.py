@@ -439,6 +439,48 @@ def test_chained_append_then_attend_sees_the_new_token(kvlib, Hq, Hkv, lens, spl
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("lens,split", [([3, 16, 40, 700], 0), ([15, 0, 31, 47], 0), ([3, 16, 31, 5000], 2)])
+@pytest.mark.parametrize("Hq,Hkv", [(8, 8), (28, 4)])
+@pytest.mark.parametrize("writer", ["append", "fused"])
+def test_attention_far_behind_the_append_sees_the_new_token(kvlib, Hq, Hkv, lens, split, writer):
+    """decode_attention after launches that wrote its layer's new tokens
+    earlier in the same chain: all layers are written first (kv_append, or the
+    fused call), then all are attended, twice, with no host waits.  Slots
+    written before held a huge K.  The same as with a wait after every call."""
+    cfg = wl.custom("behind", 4, Hq, Hkv, 128, len(lens), lens=lens, seed=89, page_order="shuffled")
+    outs = []
+    for wait in (True, False):
+        t = Tracked(cfg, extra_tokens=8, split_pages=split, keep_host=False)
+        h, B, s = t.sess.h, cfg.batch, torch.cuda.Stream()
+        ins = [wl.step_inputs(cfg, 0, l, "cuda") for l in range(cfg.num_layers)]
+        stale = torch.full_like(ins[0][1], 30.0)
+        res = [torch.empty_like(i[0]) for i in ins + ins]
+        torch.cuda.synchronize()
+        kd.kv_begin_step(h, t.sess.seq_ids, s)
+
+        def call(f, *args):
+            f(h, *args, s)
+            if wait:
+                s.synchronize()
+
+        for l in range(cfg.num_layers):
+            call(kd.kv_append, l, B, stale, stale)
+        for l, (q, kn, vn) in enumerate(ins):
+            if writer == "fused":
+                call(kd.decode_attention_append, l, B, q, kn, vn, res[l], 0.0)
+            else:
+                call(kd.kv_append, l, B, kn, vn)
+        for i in range(2 * cfg.num_layers):
+            l = i % cfg.num_layers if writer == "append" else cfg.num_layers - 1 - i % cfg.num_layers
+            call(kd.decode_attention, l, B, ins[l][0], res[i], 0.0)
+        s.synchronize()
+        outs.append(res)
+        t.sess.lens += 1
+        t.close()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
+
+
 @pytest.mark.parametrize("first,n", [(0, 1), (15, 1), (15, 2), (16, 16), (3, 13), (7, 90), (1, 143)])
 @pytest.mark.parametrize("H,d", [(40, 128), (2, 64), (3, 128), (33, 64)])
 def test_token_copies_touch_exactly_their_positions(kvlib, H, d, first, n):
