@@ -135,10 +135,12 @@ def _i32_array(values):
     else goes through int()."""
     values = values if isinstance(values, (list, tuple)) else list(values)
     try:
-        return array.array("i", values)
+        if values:   # (an empty array has no address)
+            return array.array("i", values)
     except (TypeError, OverflowError):
-        vals = [int(v) for v in values]
-        return (ctypes.c_int32 * len(vals))(*vals)
+        pass
+    vals = [int(v) for v in values]
+    return (ctypes.c_int32 * len(vals))(*vals)
 
 
 # ---------------------------------------------------------------- C names
@@ -221,7 +223,8 @@ def kv_write_varlen(h, layer_first: int, n_layers: int, seq_ids, cu_seqlens, k, 
     fp = _i32_array(first_pos) if first_pos is not None else None
     if fp is not None and len(fp) != len(ids):
         raise ValueError("first_pos needs len(seq_ids) entries")
-    _check(load().kv_write_varlen(h, layer_first, n_layers, len(ids), _ptr(ids), _ptr(fp), _ptr(cu), _ptr(k), _ptr(v), _stream(stream)), "kv_write_varlen")
+    _check(load().kv_write_varlen(h, layer_first, n_layers, len(ids), _ptr(ids), _ptr(fp), _ptr(cu),
+                                  _ptr(k), _ptr(v), _stream(stream)), "kv_write_varlen")
 
 
 def kv_begin_step(h, seq_ids, stream=None):

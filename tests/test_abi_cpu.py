@@ -279,3 +279,4 @@ def test_integer_lists_reach_the_library_as_int32():
     assert seen(iter([4, 5])) == [4, 5]
     assert seen([2**32 + 9, 1]) == [9, 1]
     assert seen([]) == []
+    assert kd._ptr(kd._i32_array([]))   # an empty list is not a null argument
