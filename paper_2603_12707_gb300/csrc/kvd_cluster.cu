@@ -307,7 +307,10 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
         if (dd == 0) cluster_store_async2(cluster_map(smem_addr(recv_ml + rank * Cg::kHeads + h), dst), M, L, bar);
     }
     if (!mbar_try_wait_cluster(bar_s, 0) && !mbar_wait_bounded_cluster(bar_s, 0, kWaitLimitNs)) {
+        // What is still on its way needs this CTA's shared memory: leave with
+        // the last of the cluster (every wait in here is bounded).
         atomicOr(p.err, 2);
+        cluster_leave();
         return;
     }
     // Hop 2: this CTA's dims over the cluster, two at a time.
@@ -466,7 +469,6 @@ ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_
         const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
         for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
             if (10 * (int64_t)resident_clusters(device, D, gqa, sh) < 11 * units) continue;
-            // pages of the longest row's warps against the layer's share of HBM time
             // the longest row's warps against what the layer's bytes take in
             // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB) that
             // the layer holds, up to 25 MB, which keep the HBM busy beside them

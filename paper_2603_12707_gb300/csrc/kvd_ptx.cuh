@@ -152,6 +152,12 @@ __device__ __forceinline__ void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// Until every thread of the cluster is here or has exited; a warp's threads may come apart.
+__device__ __forceinline__ void cluster_leave()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
 __device__ __forceinline__ int32_t cluster_load(uint32_t addr)
 {
     int32_t v;
