@@ -135,9 +135,12 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     // its own dependency wait it reads nothing that this launch or the chain
     // before it writes (but for slots that it replaces itself).  After
     // a step kernel both wait for that first.
-    bool waited = p.early == 0;
-    if (waited) griddep_wait();
-    griddep_launch_dependents();
+    // A launch with the caller's tables waits before it reads those.
+    const bool waited = Rows::kTable || p.early == 0;
+    if constexpr (!Rows::kTable) {
+        if (waited) griddep_wait();
+        griddep_launch_dependents();
+    }
     const int b = blockIdx.y, g = (int)blockIdx.x >> (31 - __clz(C));
     int2 row;   // (page-table row, tokens attended)
     if constexpr (Rows::kTable) row = make_int2(b, rt.len[b]);
@@ -162,6 +165,10 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
     const bool has_last = n > 0 && first + n == np;
     const int32_t* pt_row = p.page_table + (int64_t)row.x * p.max_pages + first;
     auto load_window = [&](int w0) { return (w0 + lane < n) ? pt_row[w0 + lane] : 0; };
+    if constexpr (Rows::kTable) {
+        griddep_wait();
+        griddep_launch_dependents();
+    }
     int32_t pid_cur = load_window(0);
     int32_t pid_next = 0;
     const uint64_t policy = l2_policy_evict_first();
@@ -450,8 +457,16 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
 // B 3, 96 units: 4 x 4 warps with 2 stages, 110 slots, 10.0; with 3 stages,
 // 74 slots, 13.9), but no more than about a warp per page (8 x 8 against
 // 4 x 4 warps at 7 pages: 10.2 against 3.0).
+//
+// spread: for a launch that loads nothing before its dependency wait.  Placed
+// while the clusters before it leave, it would crowd on the SMs that empty
+// first; with as many stages as let all units stay resident an SM takes no
+// more than its share of CTAs (us per call in a row, fewest stages -> most:
+// LLaVA heads, 850 tokens 5.0 -> 4.3, 40/40 heads, 500 tokens 4.0 -> 3.6, Qwen
+// heads, 8 rows of 700 5.2 -> 4.3).  A launch that does load early is better
+// off with a slot for every CTA at once (LLaVA layer 4.8 -> 5.2).
 ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
-                           int64_t max_pages)
+                           int64_t max_pages, bool spread)
 {
     constexpr int64_t kMostBytes = 45000000;   // K and V of a layer
     constexpr int kWarpsOf[][2] = {{8, 8}, {8, 4}, {4, 4}, {2, 4}, {1, 4}};
@@ -473,7 +488,12 @@ ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_
             // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB) that
             // the layer holds, up to 25 MB, which keep the HBM busy beside them
             const int64_t beside = std::min<int64_t>(bytes, 25000000);
-            return per_warp * (D == 128 ? 4000000 : 2800000) <= 20000000 + beside ? sh : ClusterShape{};
+            if (per_warp * (D == 128 ? 4000000 : 2800000) > 20000000 + beside) return ClusterShape{};
+            for (ClusterShape more = sh; spread && ++more.ring <= kClusterRingBytes / stage;) {
+                if (resident_clusters(device, D, gqa, more) < units) break;
+                sh = more;
+            }
+            return sh;
         }
     }
     return ClusterShape{};

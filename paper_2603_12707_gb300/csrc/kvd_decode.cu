@@ -66,8 +66,17 @@ cudaError_t launch_table(int grid, const CUtensorMap& tk, const CUtensorMap& tv,
     std::copy_n(all.row, all.n, rows.row);
     std::copy_n(all.len, all.n, rows.len);
     std::copy_n(all.off, all.n + 1, rows.off);
-    decode_kernel<D, GQA, false, Rows><<<grid, kWarps * 32, Geo<D, GQA>::kSmem, st>>>(tk, tv, p, rows);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kWarps * 32);
+    cfg.dynamicSmemBytes = Geo<D, GQA>::kSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, decode_kernel<D, GQA, false, Rows>, tk, tv, p, rows);
 }
 
 template <int D, bool GQA>

@@ -544,12 +544,6 @@ __global__ void __launch_bounds__(kWarps * 32)
     bool waited = false;
     bool first_item = true;
 
-    if constexpr (Rows::kTable) {
-        if (blockIdx.x == 0)
-            for (int i = threadIdx.x; i < rt.n; i += blockDim.x)
-                p.rows_out[rt.row[i]] = make_int2(rt.off[i], rt.off[i + 1] - rt.off[i]);
-    }
-
     // The first item of every warp is its global warp index; later ones come
     // from the work counter, offset by the number of warps.
     const int n_warps = (int)gridDim.x * kWarps;
@@ -557,7 +551,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 
     // The first launch after a step kernel: placed early, but the plan is not
     // there before the wait.
-    if (!p.early) griddep_wait();
+    if (!Rows::kTable && !p.early) griddep_wait();
     const int n_items = p.n_entries_dev ? min(p.n_items, *p.n_entries_dev * p.H_kv) : p.n_items;
     while (item < n_items) {
         const int e = item / p.H_kv;
@@ -568,6 +562,16 @@ __global__ void __launch_bounds__(kWarps * 32)
         // (a row table: the item's row by binary search, its pages straight
         // from the page table)
         const PlanEntry found = find_item(rt, e);
+        if constexpr (Rows::kTable) {
+            // What the caller ran before may have written the page table and
+            // the pages: nothing is read until that is complete.
+            if (first_item) {
+                griddep_wait();
+                if (blockIdx.x == 0)
+                    for (int i = threadIdx.x; i < rt.n; i += blockDim.x)
+                        p.rows_out[rt.row[i]] = make_int2(rt.off[i], rt.off[i + 1] - rt.off[i]);
+            }
+        }
         const int32_t* pt_row = Rows::kTable ? p.page_table + (int64_t)found.b * p.max_pages + found.first_page
                                              : p.item_pages + (int64_t)e * p.page_stride;
         auto load_window = [&](int w0) { return (w0 + lane < (Rows::kTable ? found.n_pages : p.page_stride)) ? pt_row[w0 + lane] : 0; };

@@ -357,10 +357,12 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
                            const LensTable* lens, cudaStream_t st);
 // Clusters for `batch` rows of num_kv_heads that hold `pages` pages per KV
 // head in all and at most max_pages in one row, or ctas == 0: the split plan.
+// spread: for launches that load nothing before their dependency wait.
 ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
-                           int64_t max_pages);
-// The split pass over rows given as parameters (no append, an ordinary
-// launch): p.rows is written for the merge pass, p.item_pages is not used.
+                           int64_t max_pages, bool spread = false);
+// The split pass over rows given as parameters (no append; placed early, it
+// reads nothing before its dependency wait): p.rows is written for the merge
+// pass, p.item_pages is not used.
 cudaError_t launch_decode_table(int D, bool gqa, int grid, const CUtensorMap& tk, const CUtensorMap& tv,
                                 const DecodeParams& p, const RowTable<1024>& rows, cudaStream_t st);
 

@@ -17,8 +17,14 @@
 // (A plan kernel with 20 KB of parameters and a page-list kernel before the
 // split pass, two loads per page, the merge pass as an ordinary launch and
 // five device queries per call measured 41 us a call on the Qwen-shaped
-// batch, 34 us of it on the host.)  The first launch is an ordinary one: what
-// ran before the call may have written the pools and the page table.
+// batch, 34 us of it on the host.)  The first launch is placed while what ran
+// before it finishes (programmatic dependent launch): it sets up its barriers
+// and finds its first item, and waits before it reads any device memory, since
+// what ran before may have written the pools or the page table.  Calls in a
+// row, us per call, as ordinary launches and so: the Qwen-shaped batch from
+// Python 26.6 and 24.1; replayed from a graph 13.7 and 13.6 (78 MB, in L2),
+// 64 LLaVA rows of 900 tokens 132.7 and 132.0, 2 Qwen rows of 2500 and 4400
+// (clusters) 6.5 and 5.9, 4 rows of 100, 8/8 heads, d = 64 3.1 and 2.5.
 //
 // Scratch.  The per-item partial results, the per-row merge table and the
 // work counter live in one file-scope __device__ array of
@@ -221,15 +227,15 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     p.max_pages = max_pages;
     p.scale_log2 = scale * 1.4426950408889634f;
     p.kv_map = kv_map;
-    p.early = 1;   // (an ordinary launch)
+    p.early = 0;   // placed early, but what ran before may have written anything it reads
     p.num_sms = num_sms;
 
-    const ClusterShape shape = cluster_shape(dev, head_dim, G > 1, num_kv_heads, batch, total_pages, max_np);
+    const ClusterShape shape = cluster_shape(dev, head_dim, G > 1, num_kv_heads, batch, total_pages, max_np, true);
     if (shape.ctas && batch <= kLensRows) {
         LensTable lt;
         std::copy_n(lens, batch, lt.len);
         p.ring = shape.ring;
-        if (cudaError_t e = launch_cluster(head_dim, G > 1, false, false, shape, maps[0], maps[1], p,
+        if (cudaError_t e = launch_cluster(head_dim, G > 1, false, true, shape, maps[0], maps[1], p,
                                            &lt, st);
             e != cudaSuccess)
             return fail(KVC_ERR_CUDA, cudaGetErrorString(e));

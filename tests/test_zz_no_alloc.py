@@ -249,3 +249,40 @@ def test_noalloc_pool_layouts_and_row_tables(kvlib, Hq, Hkv, d, B, longest, layo
     ref = oracle.decode_attention(u16(q)[rows], [lens[b] for b in rows], np.concatenate(kk), np.concatenate(vv))
     vmax = np.array([np.abs(oracle.bf16_to_f64(x)).max() for x in vv])
     assert_close(bf16_to_f64(outs[0])[rows], ref, vmax, gqa=Hq > Hkv)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,lens", [
+    (8, 8, 128, [200, 40, 3]),                             # clusters
+    (28, 4, 128, [900 - 25 * b for b in range(32)]),       # split pass and merge pass
+    (8, 8, 64, [1 + b % 30 for b in range(200)]),          # no merge pass
+])
+def test_noalloc_calls_see_what_ran_before_them(kvlib, Hq, Hkv, d, lens):
+    """A call is placed while what precedes it on the stream still runs: each
+    reads the query that the call before wrote, pages and page ids that a
+    copy just before it changed, and writes an output that the next call's
+    copy reads.  The same as with a wait after every operation."""
+    B, width = len(lens), max((n + 15) // 16 for n in lens)
+    pages = B * width
+    gen = torch.Generator(device="cuda").manual_seed(Hq + d)
+    pools = torch.randn((2, 2, pages * Hkv * 16 * d), generator=gen, device="cuda").bfloat16()
+    tables = torch.stack([torch.randperm(pages, generator=gen, device="cuda").reshape(B, width) for _ in range(2)]).int()
+    q0 = torch.randn((B, Hq, d), generator=gen, device="cuda").bfloat16()
+    res = []
+    for wait in (True, False):
+        kv, pt = torch.full_like(pools[0], 50.0), torch.full_like(tables[0], pages - 1)
+        outs = [q0] + [torch.zeros_like(q0) for _ in range(6)]
+        torch.cuda.synchronize()
+        for i in range(6):
+            if i % 3 != 1:   # (calls 1 and 4 follow a call directly)
+                for op in (lambda: kv.copy_(pools[i % 2]), lambda: pt.copy_(tables[i % 2])):
+                    op()
+                    if wait:
+                        torch.cuda.synchronize()
+            kd.decode_attention_noalloc(kv[0], kv[1], pages, Hq, Hkv, d, pt, width, lens, outs[i], outs[i + 1])
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert all(bool(o.isfinite().all()) for o in outs)
+        res.append(outs)
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
