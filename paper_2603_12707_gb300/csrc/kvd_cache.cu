@@ -16,6 +16,18 @@ namespace {
 // else 8 (8 rows of 2049: 9.5 us, 10.3 with 4, 14.2 with 1).
 int step_ctas(int64_t ids) { return ids <= 2048 ? 1 : 8; }
 
+// Threads per CTA of a step kernel: enough warps to copy the page ids in one
+// go (a warp has 128 in flight), 8 to 16 of them, and a thread per row where a
+// block can have one (the rows' order depends on that).  Device step of 32 /
+// 64 / 8 / 96 rows of up to 2.4k / 0.9k / 33k / 2k tokens with 256, 512 and 1024
+// threads: 5.7 5.9 6.9 / 5.5 5.8 6.9 / 6.9 6.5 7.3 / 7.5 7.0 7.7 us; without a
+// plan 1.65, 1.67 and 1.9.
+int step_threads(int64_t batch, int64_t ids, int ctas)
+{
+    if (batch > 512) return 1024;
+    return batch > 256 || ids > (int64_t)ctas * 1024 ? 512 : 256;
+}
+
 __device__ __forceinline__ void flag_error(int32_t* err, int bit) { atomicOr(err, bit); }
 
 template <int N>
@@ -27,7 +39,7 @@ __global__ void scatter_i32_kernel(int32_t* base, const __grid_constant__ Scatte
         base[s.idx[i]] = s.val[i];
 }
 
-// Exclusive block-wide prefix sum of one int per thread (blockDim.x = 1024).
+// Exclusive block-wide prefix sum of one int per thread (whole warps).
 __device__ int block_exclusive_scan(int v, int* total)
 {
     __shared__ int warp_sums[32];
@@ -56,7 +68,7 @@ __device__ int block_exclusive_scan(int v, int* total)
     return before_warp + x - v;
 }
 
-// Split plan of a step, built by a cluster of 1024-thread CTAs: plan position
+// Split plan of a step, built by a cluster of CTAs: plan position
 // i takes batch row b, sequence seq, len tokens from row_at(i, &b, &seq,
 // &len); the row is cut into row_chunks() items of near-equal size, a row's
 // items adjacent, its target size graduated by position (row_item_pages).
@@ -113,12 +125,14 @@ __device__ int build_split_plan(int batch, int item_pages, int chunk_cap, int ma
         // (chunk_range inverted: the first np % nch items hold one page more).
         const int n_rows = min((int)blockDim.x, batch - base);
         const int per_row = n_rows >= n_warps ? 1 : n_warps / n_rows;
+        if (warp >= n_rows * per_row) cluster_arrive_release();
         for (int t = warp; t < n_rows * per_row; t += n_warps) {
             const int r = t / per_row, part = t - r * per_row;
             const int field = cluster_load(cluster_map(smem_addr(&s_row[min(lane, kFields - 1)][r]), 0));
             const int rseq = __shfl_sync(0xffffffffu, field, 0), rnp = __shfl_sync(0xffffffffu, field, 1);
             const int roff = __shfl_sync(0xffffffffu, field, 2), rnch = __shfl_sync(0xffffffffu, field, 3);
             const int rb = __shfl_sync(0xffffffffu, field, 4), rlen = __shfl_sync(0xffffffffu, field, 5);
+            if (t + n_warps >= n_rows * per_row) cluster_arrive_release();   // the warp has read its last row's
             if (rnch == 0) continue;
             const int small = rnp / rnch, extra = rnp % rnch, big_pages = extra * (small + 1);
             const int32_t* src = page_table + (int64_t)rseq * max_pages;
@@ -156,7 +170,7 @@ __device__ int build_split_plan(int batch, int item_pages, int chunk_cap, int ma
             }
         }
         __syncwarp();
-        cluster_sync();   // CTA 0's shared arrays are read: the next chunk of rows, or its exit
+        cluster_wait();   // CTA 0's shared arrays are read: the next chunk of rows, or its exit
     }
     return carry;
 }
@@ -182,9 +196,10 @@ __global__ void __launch_bounds__(1024)
     build_split_plan(
         a.batch, a.item_pages, a.chunk_cap, INT_MAX,
         [&](int i, int* b, int* seq, int* len) {
+            // (an ordered batch is one launch: its rows are in the patch)
             *b = a.use_order ? a.order[i] : i;
-            *seq = a.step_seq[*b];
-            *len = a.seq_len[*seq];
+            *seq = a.use_order ? patch.seq[*b] : a.step_seq[*b];
+            *len = a.use_order ? patch.new_len[*b] : a.seq_len[*seq];
             if (*len <= 0 || *len > a.max_pages * kPageSize) {
                 flag_error(a.err, 4);
                 *len = 1;
@@ -209,13 +224,16 @@ __global__ void __launch_bounds__(1024)
 // sequence and new length stay in shared memory for the ranking and the plan.
 __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
 {
-    __shared__ int s_top;
+    __shared__ int s_free[1024];
     __shared__ int s_seq[1024], s_len[1024];   // per batch row when the batch fits the block
     griddep_launch_dependents();   // the first layer may be placed; it waits before it reads anything
     const bool small = a.batch <= (int)blockDim.x;
     const bool lead = cluster_ctarank() == 0;   // the other CTAs only help to write the plan
-    if (threadIdx.x == 0) s_top = *a.free_top;
-    int top0 = 0;
+    // The stack's top pages, one per thread, load along with the rows' lengths
+    // (with the threads above and the early arrival in build_split_plan, the
+    // steps named there take 5.2 / 5.8 / 6.4 / 6.5 us; 6.9 / 7.8 / 7.7 / 7.8 before).
+    const int top0 = lead ? *a.free_top : 0;
+    if (lead && threadIdx.x < top0) s_free[threadIdx.x] = a.free_pages[top0 - 1 - threadIdx.x];
     int carry = 0;
     for (int base = 0; lead && base < a.batch; base += blockDim.x) {
         const int i = base + threadIdx.x;
@@ -231,8 +249,7 @@ __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
             need = (ok && len % kPageSize == 0) ? 1 : 0;
         }
         int total;
-        const int rank = carry + block_exclusive_scan(need, &total);   // also orders s_top's write
-        if (base == 0) top0 = s_top;
+        const int rank = carry + block_exclusive_scan(need, &total);   // also orders s_free's writes
         if (ok) {
             int32_t page = -1;
             if (need) {
@@ -241,7 +258,7 @@ __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
                     flag_error(a.err, 8);   // pool exhausted
                     ok = false;
                 } else {
-                    page = a.free_pages[idx];
+                    page = rank < (int)blockDim.x ? s_free[rank] : a.free_pages[idx];
                 }
             }
             if (ok) {
@@ -573,11 +590,11 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, bool pdl,
 
 // A step kernel as one cluster.
 template <class... P, class... A>
-cudaError_t launch_cluster_of(int ctas, void (*kernel)(P...), cudaStream_t st, const A&... args)
+cudaError_t launch_cluster_of(int ctas, int threads, void (*kernel)(P...), cudaStream_t st, const A&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas);
-    cfg.blockDim = dim3(1024);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -613,7 +630,9 @@ cudaError_t launch_seq_op(const SeqOpArgs& a, bool pdl, cudaStream_t st)
 
 cudaError_t launch_step_device(const StepDevArgs& a, cudaStream_t st)
 {
-    return launch_cluster_of(a.no_plan ? 1 : step_ctas((int64_t)a.batch * a.max_pages), step_device_kernel, st, a);
+    const int64_t ids = a.no_plan ? 0 : (int64_t)a.batch * a.max_pages;
+    const int ctas = step_ctas(ids);
+    return launch_cluster_of(ctas, step_threads(a.batch, ids, ctas), step_device_kernel, st, a);
 }
 
 cudaError_t launch_scatter_i32(int32_t* base, const int32_t* idx, const int32_t* val, int n, bool pdl, cudaStream_t st)
@@ -625,8 +644,9 @@ cudaError_t launch_scatter_i32(int32_t* base, const int32_t* idx, const int32_t*
 
 cudaError_t launch_step(const StepPatch& patch, const PlanArgs& plan, cudaStream_t st)
 {
-    const bool plans = plan.build && !plan.no_plan;
-    return launch_cluster_of(plans ? step_ctas((int64_t)plan.batch * plan.max_pages) : 1, step_kernel, st, patch, plan);
+    const int64_t ids = plan.build && !plan.no_plan ? (int64_t)plan.batch * plan.max_pages : 0;
+    const int ctas = step_ctas(ids);
+    return launch_cluster_of(ctas, step_threads(plan.batch, ids, ctas), step_kernel, st, patch, plan);
 }
 
 cudaError_t launch_token_copy(const TokenCopyArgs& a, bool pdl, cudaStream_t st)

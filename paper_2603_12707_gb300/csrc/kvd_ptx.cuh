@@ -146,6 +146,7 @@ __device__ __forceinline__ uint32_t cluster_nctarank()
 
 // (relaxed: what the other CTAs must see is ordered by fence_mbar_init)
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 // Everything every CTA of the cluster wrote before is visible to all after.
 __device__ __forceinline__ void cluster_sync()
 {

@@ -380,14 +380,18 @@ def test_graph_of_one_layer_hands_out_every_item_on_every_replay(kvlib, Hq, Hkv,
     t.close()
 
 
-@pytest.mark.parametrize("batch,rows", [(2, 4000), (5, 700), (40, 300), (300, 90), (1025, 40)])
+@pytest.mark.parametrize("batch,rows", [(2, 4000), (5, 700), (40, 300), (300, 90), (1025, 40), (2, 7000),
+                                        (12, 1300), (255, 60), (256, 60), (257, 60), (512, 16), (513, 16), (1040, 16)])
 def test_plans_built_by_one_and_by_eight_ctas(kvlib, batch, rows):
     """Step kernels over up to 2048 page ids run as one CTA, else as a cluster
-    of eight; batches past 1024 rows plan in two rounds.  The split plan shows
+    of eight, of 256, 512 or 1024 threads; batches past 1024 rows plan in two
+    rounds; rows of 16 tokens all take a page at once.  The split plan shows
     in the result: device and host steps give the same bits, and sampled rows
     match the oracle (the layer goes through the plan: the split size is set)."""
     lens = [1 + (rows * (7 * b + 3)) // (7 * batch) for b in range(batch)]
     lens[0] = rows
+    if rows == 16:
+        lens = [16] * batch
     cfg = wl.custom("ctas", 1, 4, 4, 64, batch, lens=lens, seed=batch, page_order="shuffled")
     keep = sorted({0, 1, batch // 2, batch - 1})
     a = Tracked(cfg, extra_tokens=4, split_pages=SPLIT, keep_rows=keep)
