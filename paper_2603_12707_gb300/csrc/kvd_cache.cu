@@ -181,6 +181,7 @@ __device__ int build_split_plan(int batch, int item_pages, int chunk_cap, int ma
 __global__ void __launch_bounds__(1024)
     step_kernel(const __grid_constant__ StepPatch patch, const __grid_constant__ PlanArgs a)
 {
+    griddep_wait();
     griddep_launch_dependents();   // the first layer may be placed; it waits before it reads anything
     const bool lead = cluster_ctarank() == 0;
     for (int i = threadIdx.x; lead && i < patch.n; i += blockDim.x) {
@@ -226,6 +227,7 @@ __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
 {
     __shared__ int s_free[1024];
     __shared__ int s_seq[1024], s_len[1024];   // per batch row when the batch fits the block
+    griddep_wait();
     griddep_launch_dependents();   // the first layer may be placed; it waits before it reads anything
     const bool small = a.batch <= (int)blockDim.x;
     const bool lead = cluster_ctarank() == 0;   // the other CTAs only help to write the plan
@@ -588,7 +590,9 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, bool pdl,
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// A step kernel as one cluster.
+// A step kernel as one cluster, placed while what ran before it finishes; it
+// waits for that at its top.  (13B heads, 12 requests, 4 steps of 8 layers:
+// 1974 us as an ordinary launch, 1965 so; 28/4 heads, 254 rows 4828 and 4820.)
 template <class... P, class... A>
 cudaError_t launch_cluster_of(int ctas, int threads, void (*kernel)(P...), cudaStream_t st, const A&... args)
 {
@@ -596,12 +600,14 @@ cudaError_t launch_cluster_of(int ctas, int threads, void (*kernel)(P...), cudaS
     cfg.gridDim = dim3((unsigned)ctas);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cfg.gridDim.x;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cfg.gridDim.x;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = ctas > 1 ? 1 : 0;
+    cfg.numAttrs = ctas > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

@@ -255,6 +255,48 @@ def test_host_step_cannot_move_buffers_under_device_steps(kvlib):
     kd.kv_cache_destroy(h)
 
 
+@pytest.mark.parametrize("device", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,lens,split", [(8, 8, [15, 700, 31], 0), (28, 4, [14, 1500, 31, 400], 2)])
+def test_steps_in_a_row_without_host_waits(kvlib, Hq, Hkv, lens, split, device):
+    """A step kernel is placed while the layers before it still run: steps in a
+    row with no host wait give what they give with a wait after every call,
+    over rows that open pages (clusters, and a split plan)."""
+    cfg = wl.custom("rowsteps", 2, Hq, Hkv, 128, len(lens), lens=lens, seed=29, page_order="shuffled")
+    runs = []
+    for wait in (True, False):
+        t = Tracked(cfg, extra_tokens=24, split_pages=split, keep_host=False)
+        h, B, s = t.sess.h, cfg.batch, torch.cuda.Stream()
+        ins = [[wl.step_inputs(cfg, i, l, "cuda") for l in range(2)] for i in range(20)]
+        outs = [[torch.empty_like(q) for q, _, _ in x] for x in ins]
+        ids = torch.tensor(t.sess.seq_ids, dtype=torch.int32, device="cuda")
+        if device:
+            kd.kv_cache_device_steps(h, B)
+        torch.cuda.synchronize()
+
+        def call(f, *args):
+            f(h, *args, s)
+            if wait:
+                s.synchronize()
+
+        for i in range(20):
+            if device:
+                call(kd.kv_begin_step_device, B, ids)
+            else:
+                call(kd.kv_begin_step, t.sess.seq_ids)
+            for l, (q, kn, vn) in enumerate(ins[i]):
+                if i % 2:
+                    call(kd.decode_attention_append, l, B, q, kn, vn, outs[i][l], 0.0)
+                else:
+                    call(kd.kv_append, l, B, kn, vn)
+                    call(kd.decode_attention, l, B, q, outs[i][l], 0.0)
+        s.synchronize()
+        runs.append([o for x in outs for o in x])
+        t.sess.lens += 20
+        t.close()
+    for a, b in zip(*runs):
+        assert torch.equal(a, b)
+
+
 def test_batch_beyond_one_block_device_and_host_steps(kvlib):
     """1100 rows: the step kernels plan and copy page lists in two chunks of
     1024 rows (the host step also takes two launches); device and host steps
