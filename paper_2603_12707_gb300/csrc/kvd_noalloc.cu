@@ -249,8 +249,9 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     std::stable_sort(rt.row, rt.row + batch, [&](uint16_t x, uint16_t y) { return lens[x] > lens[y]; });
     for (int i = 0; i < batch; ++i) rt.len[i] = lens[rt.row[i]];
     // The plan of a step of the cache (items per resident warp, graduated
-    // sizes, items per row) where its partials fit, else the one sized above
-    // (whose rows of one item come last and keep no partial).
+    // sizes, items per row) where its partials fit, also with larger items,
+    // else the one sized above (whose rows of one item come last and keep no
+    // partial).
     int max_chunks = 1;
     int64_t split_end = 0;   // entries up to the last row of several items: those with partial slots
     auto cut = [&](int64_t size, int cap, bool graduated) {
@@ -268,10 +269,11 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
         rt.off[batch] = off;
         return off_part + (size_t)split_end * partial + 512 <= kNoAllocScratchBytes;
     };
-    const int64_t T_step =
-        std::max<int64_t>(T, auto_item_pages(head_dim, G > 1, num_kv_heads, warps, batch, total_pages, max_np, false));
-    const int cap = chunk_cap(G > 1, (int64_t)batch * num_kv_heads, warps, max_np, (int32_t)T_step);
-    if (!cut(T_step, cap, true) && !cut(T, kChunkCap, false))
+    const int64_t T_step = auto_item_pages(head_dim, G > 1, num_kv_heads, warps, batch, total_pages, max_np, false);
+    auto cut_as_step = [&](int64_t size) {
+        return cut(size, chunk_cap(G > 1, (int64_t)batch * num_kv_heads, warps, max_np, (int32_t)size), true);
+    };
+    if (!cut_as_step(T_step) && !cut_as_step(std::max(T, T_step)) && !cut(T, kChunkCap, false))
         return fail(KVC_ERR_UNSUPPORTED, "the batch does not fit the static scratch");
     const int32_t entries = rt.off[batch];
     p.part_o = reinterpret_cast<float*>(scratch + off_part);

@@ -481,6 +481,29 @@ def test_attention_far_behind_the_append_sees_the_new_token(kvlib, Hq, Hkv, lens
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("Hq,Hkv,B", [(32, 32, 24), (16, 8, 64)])
+@pytest.mark.parametrize("device", [False, True])
+def test_large_shares_with_smaller_items(kvlib, Hq, Hkv, B, device):
+    """Batches whose warps' share calls for items past 47 pages run with items
+    of 40 (rows of 5 to 4000 tokens and one of 9000, host and device steps)."""
+    lens = [9000, 5] + [4000 - 7 * b for b in range(B - 2)]
+    cfg = wl.custom("share", 1, Hq, Hkv, 128, B, lens=lens, seed=B, page_order="shuffled")
+    keep = [0, 1, B - 1]
+    t = Tracked(cfg, extra_tokens=4, keep_rows=keep)
+    if device:
+        kd.kv_cache_device_steps(t.sess.h, B)
+        kd.kv_begin_step_device(t.sess.h, B, torch.tensor(t.sess.seq_ids, dtype=torch.int32, device="cuda"))
+        t.step += 1
+        t.sess.lens += 1
+    else:
+        t.begin_step()
+    out, q, _, _ = t.run_layer(0, fused=True)
+    torch.cuda.synchronize()
+    ref, vmax = t.oracle(0, q, rows=keep)
+    assert_close(bf16_to_f64(out)[keep], ref, vmax, gqa=Hq > Hkv)
+    t.close()
+
+
 @pytest.mark.parametrize("first,n", [(0, 1), (15, 1), (15, 2), (16, 16), (3, 13), (7, 90), (1, 143)])
 @pytest.mark.parametrize("H,d", [(40, 128), (2, 64), (3, 128), (33, 64)])
 def test_token_copies_touch_exactly_their_positions(kvlib, H, d, first, n):
