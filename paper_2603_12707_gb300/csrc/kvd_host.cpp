@@ -59,7 +59,7 @@ int32_t kvd::auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, i
     const int64_t units = rows * num_kv_heads, total = pages * num_kv_heads;
     const int64_t per_warp = gqa ? 2 : 3;
     int64_t T = std::max<int64_t>(2, (total + per_warp * warps - 1) / (per_warp * warps));
-    if (T > (D == 128 ? 47 : 64) && max_pages > 128) T = 40;
+    if (T > (D == 128 ? 47 : 64) && max_pages > 128) T = std::max<int64_t>(40, T / 3);
     T = std::min<int64_t>(128, T);
     // Pages of 4 KB (d = 128) per warp.
     const double share = (double)total / (double)warps * D / 128;

@@ -296,10 +296,10 @@ CUresult encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_
 //    13.0 -> 9.9; 32 heads, 57 rows of up to 263: 26.1 -> 23.1).
 // Longer shares gain nothing (32 heads of 900, B 24 / 32: best target within
 // 2 % of a third of the share), up to items so long that the last ones to end
-// leave the others idle: from 48 pages (d = 64: 65) of rows past 128, 40
-// pages, well inside the third or half of the share (whole batches, ms; 32
-// heads, 96 rows of 128-8192 tokens, 128 -> 40: 13.82 -> 13.50, 48 13.50, 64
-// 13.50, 96 13.55; 78 rows of up to 4581 7.97 -> 7.75, 48 7.79, 64 7.88; 16/8
+// leave the others idle: targets from 48 pages (d = 64: 65) for rows past 128
+// become a third of that, at least 40 and at most 128 (whole batches, ms; 32
+// heads, 96 rows of 128-8192 tokens, 128 -> 53: 13.82 -> 13.49, 40 13.50, 64
+// 13.50, 96 13.55; 256 such rows, a third of 424: 128 54.14 a step, 40 54.50; 78 rows of up to 4581 7.97 -> 7.75, 48 7.79, 64 7.88; 16/8
 // heads, 149 rows of up to 4606, 55 -> 40: 5.79 -> 5.60; 8/8 at d = 64, 37 rows
 // of up to 27861, 87 -> 40: 6.04 -> 5.97.  Not below: 56/8 heads, 117 rows of up
 // to 4592, 47 -> 40: 5.93 -> 5.97; d = 64, 202 rows, 51 -> 40: 8.05 -> 8.11; nor
