@@ -207,10 +207,7 @@ __global__ void __launch_bounds__(1024)
             }
         },
         a.plan, a.rows, a.page_table, a.max_pages, a.page_ids, a.page_stride, a.err);
-    if (lead && threadIdx.x == 0) {
-        *a.step_no += 1u;
-        a.queues[0] = a.queues[1] = 0u;
-    }
+    if (lead && threadIdx.x == 0) *a.step_no += 1u;
 }
 
 // The same step on the device (graph-replayable, no host input): rows in
@@ -317,7 +314,6 @@ __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
     if (lead && threadIdx.x == 0) {
         *a.n_entries = min(entries, a.max_entries);
         *a.step_no += 1u;
-        a.queues[0] = a.queues[1] = 0u;
     }
 }
 

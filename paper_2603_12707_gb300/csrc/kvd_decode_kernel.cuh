@@ -27,13 +27,16 @@
 // (start_flags) that its split pass is complete, the warp brings the item's
 // next kEarlyL2Pages pages into L2; and right after its wait it brings the
 // next kRampL2Pages, so the HBM keeps streaming while the merge runs and the
-// ring's pages are worked.  Consecutive launches use alternating work counters; each
-// launch resets the next one's after its wait, so no warp does an atomic on
-// its way out.
+// ring's pages are worked.
+//
+// The work counter is zero before and after every launch, whatever ran before
+// it (graph replays of any number of launches among them): an item is followed
+// by exactly one fetch, so a launch of n items fetches n times, and the counter
+// wraps to zero with the n-th.  No extra atomic, reset or second counter.
 //
 // Every mbarrier wait is bounded: after a second without progress the warp
-// records KVC_DEVERR_WAIT_TIMEOUT, waits (bounded) for its loads in flight and
-// leaves.  Page ids outside the pool are recorded and replaced by page 0.
+// records KVC_DEVERR_WAIT_TIMEOUT, waits (bounded) for its loads in flight,
+// takes what is left off the work counter and leaves.  Page ids outside the pool are recorded and replaced by page 0.
 // Device code only (included by kvd_decode.cu, which instantiates and
 // launches it).
 #pragma once
@@ -695,11 +698,16 @@ __global__ void __launch_bounds__(kWarps * 32)
         comp.finish(p, en, g, lane);
         if constexpr (Rows::kTable)
             if (n_items <= n_warps) break;   // every item was some warp's first
-        if (lane == 0) item = n_warps + (int)atomicAdd(&p.queue[0], 1u);
+        if (lane == 0) item = n_warps + (int)atomicInc(p.queue, (unsigned)n_items - 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
     }
 
-    if (!ok && lane == 0) atomicOr(p.err, 2);
+    if (!ok && lane == 0) {
+        atomicOr(p.err, 2);
+        // one fetch per item all the same: the counter ends at zero
+        if (!Rows::kTable || n_items > n_warps)
+            while (n_warps + (int)atomicInc(p.queue, (unsigned)n_items - 1u) < n_items) {}
+    }
     // Let every load this warp issued land before the warp leaves.
 #pragma unroll
     for (int s = 0; s < R; ++s)
@@ -707,12 +715,9 @@ __global__ void __launch_bounds__(kWarps * 32)
     __syncwarp();
 
     // Every warp completes only after the launch it depends on has (so a
-    // launch's completion always implies its predecessor's).  Then one thread
-    // resets the work counter of the next launch: the previous launch used it
-    // and has completed.  The next launch fetches from it only after its own
-    // dependency wait, i.e. after this launch has completed.
+    // launch's completion always implies its predecessor's, and the next one,
+    // which fetches items only after its own wait, finds the counter at zero).
     if (!waited) griddep_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 0 && p.queue_next) *p.queue_next = 0u;
 }
 
 }  // namespace

@@ -124,13 +124,12 @@ struct kv_cache {
     int32_t* meta = nullptr;                    // page table [max_seqs][max_pages], then seq_len [max_seqs]
     int32_t* step_seq = nullptr;
     int2* rows = nullptr;                       // per batch row: (first partial slot, items)
-    uint32_t* queue = nullptr;                  // two work counters, used by alternate attention launches
+    uint32_t* queue = nullptr;                  // the attention launches' work counter
     uint32_t* start_flags = nullptr;            // [num_sms][32]: merge passes announce their split pass's end
     uint32_t* step_no = nullptr;                // device step counter
     uint32_t attn_tag = 0;                      // tag of the step's latest attention launch (0: none yet)
     bool prev_merge = false;                    // that launch has a merge pass
     unsigned long long prev_capture = 0;        // its stream-capture sequence (0: not captured)
-    uint32_t attn_launches = 0;                 // attention launches so far (selects the counter)
     int64_t launches = 0;                       // kernels launched (reported by kv_cache_query)
     // An attention launch or a kv_append may depend programmatically on the
     // launch before it only if that was one of these on the same stream: the
@@ -431,7 +430,7 @@ int kv_cache_create(const kvc_config* cfg, void* stream, kv_cache** out)
         KVD_CUDA_C(cudaMalloc((void**)&c->meta, meta_elems * sizeof(int32_t)));
         KVD_CUDA_C(cudaMalloc((void**)&c->step_seq, (size_t)k.max_seqs * sizeof(int32_t)));
         KVD_CUDA_C(cudaMalloc((void**)&c->rows, (size_t)k.max_seqs * sizeof(int2)));
-        KVD_CUDA_C(cudaMalloc((void**)&c->queue, 4 * sizeof(uint32_t)));
+        KVD_CUDA_C(cudaMalloc((void**)&c->queue, sizeof(uint32_t)));
         KVD_CUDA_C(cudaMalloc((void**)&c->start_flags, (size_t)c->num_sms * 32 * sizeof(uint32_t)));
         KVD_CUDA_C(cudaMalloc((void**)&c->step_no, sizeof(uint32_t)));
         KVD_CUDA_C(cudaMemsetAsync(c->start_flags, 0, (size_t)c->num_sms * 32 * sizeof(uint32_t), st));
@@ -442,7 +441,7 @@ int kv_cache_create(const kvc_config* cfg, void* stream, kv_cache** out)
         KVD_CUDA_C(cudaMemsetAsync(c->seq_len_dev(), 0, (size_t)k.max_seqs * sizeof(int32_t), st));
         KVD_CUDA_C(cudaMemsetAsync(c->step_seq, 0, (size_t)k.max_seqs * sizeof(int32_t), st));
         KVD_CUDA_C(cudaMemsetAsync(c->rows, 0, (size_t)k.max_seqs * sizeof(int2), st));
-        KVD_CUDA_C(cudaMemsetAsync(c->queue, 0, 4 * sizeof(uint32_t), st));
+        KVD_CUDA_C(cudaMemsetAsync(c->queue, 0, sizeof(uint32_t), st));
         KVD_CUDA_C(cudaMemsetAsync(c->err, 0, sizeof(int32_t), st));
 #undef KVD_CUDA_C
 
@@ -876,7 +875,6 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         pa.page_stride = stride;
         pa.err = c->err;
         pa.step_no = c->step_no;
-        pa.queues = c->queue;
         pa.no_plan = shape.ctas ? 1 : 0;
         // Longest rows first: their items start early and the tail is short.
         pa.use_order = use_order ? 1 : 0;
@@ -983,13 +981,7 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     p.page_stride = c->page_stride;
     p.n_entries_dev = c->step_dev ? c->d_small + 1 : nullptr;
     p.batch = batch;
-    // Consecutive attention launches use different work counters: a chained
-    // launch may start while the previous one drains, and each launch resets
-    // the counter of the next one once the previous launch has completed.
-    // That order breaks where a graph replays an odd number of launches, so
-    // the step kernels zero both counters and a merge pass its launch's own.
-    p.queue = c->queue + (c->attn_launches & 1u);
-    p.queue_next = c->queue + ((c->attn_launches + 1u) & 1u);
+    p.queue = c->queue;
     p.err = c->err;
     p.num_pages = c->cfg.num_pages;
     p.n_items = c->step_entries * c->cfg.num_kv_heads;
@@ -1055,7 +1047,6 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     KVD_CUDA(launch_decode(c->cfg.head_dim, c->group > 1, fused, pdl || after_step, grid, c->tmaps[layer], c->tmaps[layer], p,
                            static_cast<cudaStream_t>(stream)));
     ++c->launches;
-    ++c->attn_launches;   // the launch used one counter and resets the other, whatever follows
     c->prev_merge = false;
     if (c->step_split) {
         // Launched early, the merge CTAs sit beside the resident split pass.
@@ -1156,7 +1147,6 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     a.page_stride = c->dev_stride;
     a.err = c->err;
     a.step_no = c->step_no;
-    a.queues = c->queue;
     // The rows' lengths are the device's: judge the step by the pages held
     // when device steps were enabled, or by full rows if there were none.
     ClusterShape shape;

@@ -114,7 +114,6 @@ struct PlanArgs {
     int32_t page_stride;
     int32_t* err;
     uint32_t* step_no;   // step counter, advanced by the launch that builds the plan
-    uint32_t* queues;    // the two work counters of the attention launches, zeroed by that launch
 };
 
 // kv_begin_step_device: the step's lazy allocation and plan, on the device.
@@ -139,7 +138,6 @@ struct StepDevArgs {
     int32_t page_stride;
     int32_t* err;
     uint32_t* step_no;        // step counter, advanced once per step
-    uint32_t* queues;         // the two work counters of the attention launches, zeroed
 };
 
 template <int N>
@@ -229,8 +227,7 @@ struct DecodeParams {
     int32_t page_stride;
     const int32_t* n_entries_dev; // device-built plan: entries live here (n_items is then a bound)
     int32_t batch;
-    uint32_t* queue;          // next item to hand out (zero at launch)
-    uint32_t* queue_next;     // the next launch's counter, reset by this one (null: none)
+    uint32_t* queue;          // next item to hand out (zero before and after each launch)
     int32_t* err;
     int64_t num_pages;
     int32_t n_items;

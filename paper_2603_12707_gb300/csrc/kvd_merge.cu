@@ -120,7 +120,6 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const DecodePar
     }
     // Announce that the split pass is complete to the next layer's warps,
     // which are resident already and warm L2 while this pass runs.
-    if (blockIdx.x == 0 && lane == 0) *p.queue = 0u;   // every item of this launch is done
     if (blockIdx.x == 0 && p.start_flags) {
         const uint32_t v = *p.step_no * 65536u + p.tag;
         for (int k = lane; k < p.num_sms; k += 32) p.start_flags[k * 32] = v;
@@ -162,7 +161,6 @@ __global__ void __launch_bounds__(kWideWarps * 32) merge_wide_kernel(const Decod
         griddep_launch_dependents();   // the next layer may start streaming now
         griddep_wait();                // the split pass of this layer is complete
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *p.queue = 0u;   // every item of this launch is done
     if (blockIdx.x == 0 && wid == 0 && p.start_flags) {
         const uint32_t v = *p.step_no * 65536u + p.tag;
         for (int k = lane; k < p.num_sms; k += 32) p.start_flags[k * 32] = v;

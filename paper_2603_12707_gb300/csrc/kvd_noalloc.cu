@@ -33,9 +33,9 @@
 // address; the first call on each device looks the address up with
 // cudaGetSymbolAddress (make that first call before any stream capture) and
 // later calls reuse it.  Every call shares the array and leaves its contents
-// behind, but for the work counter, which is zero before and after each call
-// (the merge pass, or a memset where there is none, puts it back); calls that
-// overlap on the GPU (different streams, no ordering) race on the array.
+// behind, but for the work counter, which is zero before and after each
+// launch; calls that overlap on the GPU (different streams, no ordering) race
+// on the array.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -284,15 +284,10 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(resident, p.n_items));
     if (cudaError_t e = launch_decode_table(head_dim, G > 1, grid, maps[0], maps[1], p, rt, st); e != cudaSuccess)
         return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
-    cudaError_t e = cudaSuccess;
     if (max_chunks > 1) {
         const int split_regs = ((var.ctas_per_sm * var.warps + 3) / 4) * warp_register_allocation(var.regs);
-        e = launch_merge(head_dim, true, max_chunks, num_sms, split_regs, p, st);
+        if (cudaError_t e = launch_merge(head_dim, true, max_chunks, num_sms, split_regs, p, st); e != cudaSuccess)
+            return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
     }
-    if ((max_chunks == 1 && p.n_items > grid) || e != cudaSuccess) {
-        const cudaError_t m = cudaMemsetAsync(p.queue, 0, sizeof(uint32_t), st);   // (a memset: it allocates nothing)
-        if (e == cudaSuccess) e = m;
-    }
-    if (e != cudaSuccess) return fail(KVC_ERR_CUDA, cudaGetErrorString(e));
     return KVC_OK;
 }

@@ -422,6 +422,47 @@ def test_graph_of_one_layer_hands_out_every_item_on_every_replay(kvlib, Hq, Hkv,
     t.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 3])
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 8, 64), (28, 4, 128)])
+def test_unsplit_plan_hands_out_every_item_on_every_replay(kvlib, Hq, Hkv, d, n):
+    """A host-planned step whose rows are all whole has no merge pass.  Graphs
+    of n of its layer calls, one captured and never replayed, single calls
+    between the replays: every launch hands out every item (1600 and more
+    items, so some are claimed from the counter)."""
+    B = 1600 // Hkv
+    cfg = wl.custom("whole", 1, Hq, Hkv, d, B, lens=[1 + b % 15 for b in range(B)], seed=73)
+    t = Tracked(cfg, extra_tokens=4, keep_host=False)
+    h = t.sess.h
+    q, _, _ = wl.step_inputs(cfg, 0, 0, "cuda")
+    out, ref = torch.empty_like(q), torch.empty_like(q)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    kd.kv_begin_step(h, t.sess.seq_ids, s)
+    n0 = t.sess.query().kernel_launches
+    kd.kv_append(h, 0, B, *wl.step_inputs(cfg, 0, 0, "cuda")[1:], s)
+    kd.decode_attention(h, 0, B, q, ref, 0.0, s)
+    s.synchronize()
+    assert t.sess.query().kernel_launches - n0 == 2   # no merge pass
+    graphs = [torch.cuda.CUDAGraph() for _ in range(2)]
+    for g in graphs:
+        with torch.cuda.graph(g, stream=s):
+            for _ in range(n):
+                kd.decode_attention(h, 0, B, q, out, 0.0, s)
+    with torch.cuda.stream(s):
+        for rep in range(4):
+            for replay in (True, False, True):
+                out.zero_()
+                if replay:
+                    graphs[0].replay()
+                else:
+                    kd.decode_attention(h, 0, B, q, out, 0.0, s)
+                got = out.clone()
+                s.synchronize()
+                assert torch.equal(got, ref), (rep, replay)
+    t.sess.lens += 1
+    t.close()
+
+
 @pytest.mark.parametrize("batch,rows", [(2, 4000), (5, 700), (40, 300), (300, 90), (1025, 40), (2, 7000),
                                         (12, 1300), (255, 60), (256, 60), (257, 60), (512, 16), (513, 16), (1040, 16)])
 def test_plans_built_by_one_and_by_eight_ctas(kvlib, batch, rows):
