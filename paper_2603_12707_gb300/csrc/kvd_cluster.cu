@@ -354,10 +354,10 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 1)
 template <int D, bool GQA, bool FUSED, class Rows = PlanRows>
 cudaError_t prepare_cluster()
 {
-    static cudaError_t status =
-        cudaFuncSetAttribute(cluster_kernel<D, GQA, FUSED, Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             ClusterGeo<D, GQA>::smem(kClusterMaxWarps, kClusterRingBytes / ClusterGeo<D, GQA>::kStage));
-    return status;
+    static OncePerDevice once;
+    return once.set_attribute(
+        cluster_kernel<D, GQA, FUSED, Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        ClusterGeo<D, GQA>::smem(kClusterMaxWarps, kClusterRingBytes / ClusterGeo<D, GQA>::kStage));
 }
 
 template <int D, bool GQA, bool FUSED, class Rows>
@@ -407,7 +407,10 @@ cudaError_t resident_shape(const ClusterShape& sh, int* clusters)
     return cudaOccupancyMaxActiveClusters(clusters, cluster_kernel<D, GQA, true, PlanRows>, &cfg);
 }
 
-// Clusters of a shape that the GPU holds at once, asked once per device and shape.
+// Clusters of a shape that the GPU holds at once, asked once per device and
+// shape, for the fused kernel: of a head shape's variants it takes the most
+// registers (108 / 126 / 132 / 164 for d = 64 MHA, GQA, d = 128 MHA, GQA; the
+// others 92 / 114 / 119 / 154), so the others fit as well.
 int resident_clusters(int device, int D, bool gqa, const ClusterShape& sh)
 {
     static std::atomic<int> known[64][2][2][kClusterMaxCtas + 1][kClusterMaxWarps / 4 + 1][kClusterRingBytes / 4096 + 1];

@@ -12,9 +12,9 @@ namespace {
 template <int D, bool GQA, bool FUSED, class Rows = PlanRows>
 cudaError_t prepare_variant()
 {
-    static cudaError_t status = cudaFuncSetAttribute(decode_kernel<D, GQA, FUSED, Rows>,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<D, GQA>::kSmem);
-    return status;
+    static OncePerDevice once;
+    return once.set_attribute(decode_kernel<D, GQA, FUSED, Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Geo<D, GQA>::kSmem);
 }
 
 template <int D, bool GQA>

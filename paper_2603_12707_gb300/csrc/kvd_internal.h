@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace kvd {
 
 constexpr int kPageSize = 16;          // tokens per page (the only supported P)
@@ -312,6 +314,31 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
 // fit beside the resident GQA split pass (Qwen shape: 0.742 at 32, 0.769 at
 // 16, 0.756 at 24, 0.686 at 12).
 int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T);
+
+// A setup that belongs to a device (a kernel's attributes do), done once on
+// each: `set` is called until it succeeds there.
+struct OncePerDevice {
+    static constexpr int kDevices = 64;
+    std::atomic<bool> done[kDevices] = {};
+
+    template <class F>
+    cudaError_t operator()(int device, F set)
+    {
+        const bool known = device >= 0 && device < kDevices;
+        if (known && done[device].load(std::memory_order_acquire)) return cudaSuccess;
+        const cudaError_t e = set();
+        if (known && e == cudaSuccess) done[device].store(true, std::memory_order_release);
+        return e;
+    }
+
+    template <class Kernel>
+    cudaError_t set_attribute(Kernel* kernel, cudaFuncAttribute attribute, int value)   // on the current device
+    {
+        int device = 0;
+        if (cudaError_t e = cudaGetDevice(&device); e != cudaSuccess) return e;
+        return (*this)(device, [&] { return cudaFuncSetAttribute(kernel, attribute, value); });
+    }
+};
 
 // Message returned by kv_last_error() on the calling thread.
 void set_last_error(const char* msg);

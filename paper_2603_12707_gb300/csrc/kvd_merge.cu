@@ -245,18 +245,20 @@ __global__ void __launch_bounds__(kWideWarps * 32) merge_wide_kernel(const Decod
 template <int D, int BATCH>
 cudaError_t launch_merge_variant(const cudaLaunchConfig_t& cfg, const DecodeParams& p, int flag)
 {
-    static cudaError_t status =
-        cudaFuncSetAttribute(merge_kernel<D, BATCH>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (status != cudaSuccess) return status;
+    static OncePerDevice once;
+    if (cudaError_t e = once.set_attribute(merge_kernel<D, BATCH>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        e != cudaSuccess)
+        return e;
     return cudaLaunchKernelEx(&cfg, merge_kernel<D, BATCH>, p, flag);
 }
 
 template <int D>
 cudaError_t launch_merge_wide(const cudaLaunchConfig_t& cfg, const DecodeParams& p, int flag)
 {
-    static cudaError_t status =
-        cudaFuncSetAttribute(merge_wide_kernel<D>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (status != cudaSuccess) return status;
+    static OncePerDevice once;
+    if (cudaError_t e = once.set_attribute(merge_wide_kernel<D>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        e != cudaSuccess)
+        return e;
     return cudaLaunchKernelEx(&cfg, merge_wide_kernel<D>, p, flag);
 }
 
