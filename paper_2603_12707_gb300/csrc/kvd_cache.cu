@@ -10,24 +10,6 @@ namespace kvd {
 
 namespace {
 
-// CTAs of a step kernel that builds a plan over at most `ids` page ids: one
-// where its warps hold them in a round or two (12 rows of up to 85 pages: the
-// step is 2 us shorter than with 4 or 8, which the cluster's start costs),
-// else 8 (8 rows of 2049: 9.5 us, 10.3 with 4, 14.2 with 1).
-int step_ctas(int64_t ids) { return ids <= 2048 ? 1 : 8; }
-
-// Threads per CTA of a step kernel: enough warps to copy the page ids in one
-// go (a warp has 128 in flight), 8 to 16 of them, and a thread per row where a
-// block can have one (the rows' order depends on that).  Device step of 32 /
-// 64 / 8 / 96 rows of up to 2.4k / 0.9k / 33k / 2k tokens with 256, 512 and 1024
-// threads: 5.7 5.9 6.9 / 5.5 5.8 6.9 / 6.9 6.5 7.3 / 7.5 7.0 7.7 us; without a
-// plan 1.65, 1.67 and 1.9.
-int step_threads(int64_t batch, int64_t ids, int ctas)
-{
-    if (batch > 512) return 1024;
-    return batch > 256 || ids > (int64_t)ctas * 1024 ? 512 : 256;
-}
-
 __device__ __forceinline__ void flag_error(int32_t* err, int bit) { atomicOr(err, bit); }
 
 template <int N>

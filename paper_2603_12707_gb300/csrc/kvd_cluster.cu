@@ -443,63 +443,10 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
     return cudaErrorInvalidValue;
 }
 
-// The line between the two, measured as us per layer of graph-replayed steps
-// (split plan -> clusters).  Clusters save the merge pass and its dependency
-// hop (2.3 us), but cut the rows evenly, without the plan's balancing: they
-// win up to about 45 MB of K/V per layer (LLaVA heads, 800 tokens, B 1 / 2 / 3:
-// 6.5 -> 4.3, 8.0 -> 7.1, 10.2 -> 9.7; B 4, 52 MB: 12.0 -> 13.9; Qwen heads,
-// 1500 tokens, B 4 / 8: 7.0 -> 4.3, 8.4 -> 6.3; 16/8 heads of 500, B 20: 9.1 ->
-// 8.7; B 16 of 1400, 46 MB: 10.2 -> 10.4), unless one row is so long that its
-// warps finish far behind the others (Qwen heads, 8 rows of 300 to 3800
-// tokens, 8 pages per warp: 9.8 -> 7.8; 7 of 300 to 4300, 24 MB, 9 pages: 9.3 ->
-// 8.1; 8/8 heads, 20 rows of 50 to 1500, 12
-// pages per warp: 12.1 -> 14.2; 1 row of 32000, 32 pages: 19.5 -> 21.5).
-//
-// Of the shapes, the one with the most warps per unit whose units all find a
-// slot at once, with a tenth to spare for the next launch's (LLaVA heads,
-// B 3, 96 units: 4 x 4 warps with 2 stages, 110 slots, 10.0; with 3 stages,
-// 74 slots, 13.9), but no more than about a warp per page (8 x 8 against
-// 4 x 4 warps at 7 pages: 10.2 against 3.0).
-//
-// spread: for a launch that loads nothing before its dependency wait.  Placed
-// while the clusters before it leave, it would crowd on the SMs that empty
-// first; with as many stages as let all units stay resident an SM takes no
-// more than its share of CTAs (us per call in a row, fewest stages -> most:
-// LLaVA heads, 850 tokens 5.0 -> 4.3, 40/40 heads, 500 tokens 4.0 -> 3.6, Qwen
-// heads, 8 rows of 700 5.2 -> 4.3).  A launch that does load early is better
-// off with a slot for every CTA at once (LLaVA layer 4.8 -> 5.2).
 ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
                            int64_t max_pages, bool spread)
 {
-    constexpr int64_t kMostBytes = 45000000;   // K and V of a layer
-    constexpr int kWarpsOf[][2] = {{8, 8}, {8, 4}, {4, 4}, {2, 4}, {1, 4}};
-    const int64_t units = batch * num_kv_heads;
-    const int64_t stage = 2 * (int64_t)kPageSize * D * 2;
-    const int64_t bytes = pages * num_kv_heads * stage;
-    if (bytes > kMostBytes) return ClusterShape{};
-    for (const auto& cw : kWarpsOf) {
-        ClusterShape sh;
-        sh.ctas = cw[0];
-        sh.warps = cw[1];
-        const int64_t n = (int64_t)sh.ctas * sh.warps;
-        if (n > 4 && (n / 2 >= max_pages || (n == 64 && max_pages <= 128))) continue;
-        const int64_t per_warp = (max_pages + n - 1) / n;
-        const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
-        for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
-            if (10 * (int64_t)resident_clusters(device, D, gqa, sh) < 11 * units) continue;
-            // the longest row's warps against what the layer's bytes take in
-            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB) that
-            // the layer holds, up to 25 MB, which keep the HBM busy beside them
-            const int64_t beside = std::min<int64_t>(bytes, 25000000);
-            if (per_warp * (D == 128 ? 4000000 : 2800000) > 20000000 + beside) return ClusterShape{};
-            for (ClusterShape more = sh; spread && ++more.ring <= kClusterRingBytes / stage;) {
-                if (resident_clusters(device, D, gqa, more) < units) break;
-                sh = more;
-            }
-            return sh;
-        }
-    }
-    return ClusterShape{};
+    return pick_cluster_shape(resident_clusters, device, D, gqa, num_kv_heads, batch, pages, max_pages, spread);
 }
 
 }  // namespace kvd

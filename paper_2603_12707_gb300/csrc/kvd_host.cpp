@@ -53,37 +53,6 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 void kvd::set_last_error(const char* msg) { g_last_error = msg; }
 
-int32_t kvd::auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages,
-                             int64_t max_pages, bool growing)
-{
-    const int64_t units = rows * num_kv_heads, total = pages * num_kv_heads;
-    const int64_t per_warp = gqa ? 2 : 3;
-    int64_t T = std::max<int64_t>(2, (total + per_warp * warps - 1) / (per_warp * warps));
-    if (T > (D == 128 ? 47 : 64) && max_pages > 128) T = std::max<int64_t>(40, T / 3);
-    T = std::min<int64_t>(128, T);
-    // Pages of 4 KB (d = 128) per warp.
-    const double share = (double)total / (double)warps * D / 128;
-    if (share > 30 || rows < 1) return (int32_t)T;
-    const double even = (double)max_pages * (double)rows / (double)std::max<int64_t>(1, pages);   // longest row / mean row
-    int64_t few = 0;
-    if (even <= (share < 15 ? 1.35 : 1.15)) {
-        const double want = (double)warps / (double)units * (share < 15 ? 1.06 : 1.3) + (share < 15 ? 0.0 : 0.5);
-        const int64_t items = std::max<int64_t>(1, (int64_t)want);
-        few = (max_pages + (growing ? max_pages / 8 : 0) + items - 1) / items;
-    } else if (max_pages <= 8 || (units >= warps && 10 * max_pages * warps <= 13 * total)) {
-        few = max_pages;
-    }
-    if (few >= max_pages) few = std::max<int64_t>(few, 16);
-    return (int32_t)std::max(T, std::min<int64_t>(128, few));
-}
-
-int32_t kvd::chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T)
-{
-    const bool few_units = units * kChunkCap < warps;
-    if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
-    return gqa ? kChunkCapGqa : kChunkCap;
-}
-
 CUresult kvd::encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_t rows, int D,
                               int64_t v_stride_bytes)
 {

@@ -392,6 +392,13 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
 // spread: for launches that load nothing before their dependency wait.
 ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
                            int64_t max_pages, bool spread = false);
+// The same with the number of clusters of a shape that the device holds at once as a callback.
+using ResidentClusters = int (*)(int device, int D, bool gqa, const ClusterShape& shape);
+ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bool gqa, int num_kv_heads,
+                                int64_t batch, int64_t pages, int64_t max_pages, bool spread = false);
+// CTAs of a step kernel that builds a plan over at most `ids` page ids, and its threads per CTA.
+int step_ctas(int64_t ids);
+int step_threads(int64_t batch, int64_t ids, int ctas);
 // The split pass over rows given as parameters (no append; placed early, it
 // reads nothing before its dependency wait): p.rows is written for the merge
 // pass, p.item_pages is not used.

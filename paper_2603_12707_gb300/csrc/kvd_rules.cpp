@@ -1,0 +1,118 @@
+// The choices that a call makes from sizes alone: items of a split plan,
+// clusters or a plan, launch shape of the step kernels.  Host code without
+// CUDA calls.
+#include <algorithm>
+
+#include "kvd_internal.h"
+
+namespace kvd {
+
+int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages,
+                        int64_t max_pages, bool growing)
+{
+    const int64_t units = rows * num_kv_heads, total = pages * num_kv_heads;
+    const int64_t per_warp = gqa ? 2 : 3;
+    int64_t T = std::max<int64_t>(2, (total + per_warp * warps - 1) / (per_warp * warps));
+    if (T > (D == 128 ? 47 : 64) && max_pages > 128) T = std::max<int64_t>(40, T / 3);
+    T = std::min<int64_t>(128, T);
+    // Pages of 4 KB (d = 128) per warp.
+    const double share = (double)total / (double)warps * D / 128;
+    if (share > 30 || rows < 1) return (int32_t)T;
+    const double even = (double)max_pages * (double)rows / (double)std::max<int64_t>(1, pages);   // longest row / mean row
+    int64_t few = 0;
+    if (even <= (share < 15 ? 1.35 : 1.15)) {
+        const double want = (double)warps / (double)units * (share < 15 ? 1.06 : 1.3) + (share < 15 ? 0.0 : 0.5);
+        const int64_t items = std::max<int64_t>(1, (int64_t)want);
+        few = (max_pages + (growing ? max_pages / 8 : 0) + items - 1) / items;
+    } else if (max_pages <= 8 || (units >= warps && 10 * max_pages * warps <= 13 * total)) {
+        few = max_pages;
+    }
+    if (few >= max_pages) few = std::max<int64_t>(few, 16);
+    return (int32_t)std::max(T, std::min<int64_t>(128, few));
+}
+
+int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T)
+{
+    const bool few_units = units * kChunkCap < warps;
+    if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
+    return gqa ? kChunkCapGqa : kChunkCap;
+}
+
+// The line between the two, measured as us per layer of graph-replayed steps
+// (split plan -> clusters).  Clusters save the merge pass and its dependency
+// hop (2.3 us), but cut the rows evenly, without the plan's balancing: they
+// win up to about 45 MB of K/V per layer (LLaVA heads, 800 tokens, B 1 / 2 / 3:
+// 6.5 -> 4.3, 8.0 -> 7.1, 10.2 -> 9.7; B 4, 52 MB: 12.0 -> 13.9; Qwen heads,
+// 1500 tokens, B 4 / 8: 7.0 -> 4.3, 8.4 -> 6.3; 16/8 heads of 500, B 20: 9.1 ->
+// 8.7; B 16 of 1400, 46 MB: 10.2 -> 10.4), unless one row is so long that its
+// warps finish far behind the others (Qwen heads, 8 rows of 300 to 3800
+// tokens, 8 pages per warp: 9.8 -> 7.8; 7 of 300 to 4300, 24 MB, 9 pages: 9.3 ->
+// 8.1; 8/8 heads, 20 rows of 50 to 1500, 12
+// pages per warp: 12.1 -> 14.2; 1 row of 32000, 32 pages: 19.5 -> 21.5).
+//
+// Of the shapes, the one with the most warps per unit whose units all find a
+// slot at once, with a tenth to spare for the next launch's (LLaVA heads,
+// B 3, 96 units: 4 x 4 warps with 2 stages, 110 slots, 10.0; with 3 stages,
+// 74 slots, 13.9), but no more than about a warp per page (8 x 8 against
+// 4 x 4 warps at 7 pages: 10.2 against 3.0).
+//
+// spread: for a launch that loads nothing before its dependency wait.  Placed
+// while the clusters before it leave, it would crowd on the SMs that empty
+// first; with as many stages as let all units stay resident an SM takes no
+// more than its share of CTAs (us per call in a row, fewest stages -> most:
+// LLaVA heads, 850 tokens 5.0 -> 4.3, 40/40 heads, 500 tokens 4.0 -> 3.6, Qwen
+// heads, 8 rows of 700 5.2 -> 4.3).  A launch that does load early is better
+// off with a slot for every CTA at once (LLaVA layer 4.8 -> 5.2).
+ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bool gqa, int num_kv_heads,
+                                int64_t batch, int64_t pages, int64_t max_pages, bool spread)
+{
+    constexpr int64_t kMostBytes = 45000000;   // K and V of a layer
+    constexpr int kWarpsOf[][2] = {{8, 8}, {8, 4}, {4, 4}, {2, 4}, {1, 4}};
+    const int64_t units = batch * num_kv_heads;
+    const int64_t stage = 2 * (int64_t)kPageSize * D * 2;
+    const int64_t bytes = pages * num_kv_heads * stage;
+    if (bytes > kMostBytes) return ClusterShape{};
+    for (const auto& cw : kWarpsOf) {
+        ClusterShape sh;
+        sh.ctas = cw[0];
+        sh.warps = cw[1];
+        const int64_t n = (int64_t)sh.ctas * sh.warps;
+        if (n > 4 && (n / 2 >= max_pages || (n == 64 && max_pages <= 128))) continue;
+        const int64_t per_warp = (max_pages + n - 1) / n;
+        const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
+        for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
+            if (10 * (int64_t)resident(device, D, gqa, sh) < 11 * units) continue;
+            // the longest row's warps against what the layer's bytes take in
+            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB) that
+            // the layer holds, up to 25 MB, which keep the HBM busy beside them
+            const int64_t beside = std::min<int64_t>(bytes, 25000000);
+            if (per_warp * (D == 128 ? 4000000 : 2800000) > 20000000 + beside) return ClusterShape{};
+            for (ClusterShape more = sh; spread && ++more.ring <= kClusterRingBytes / stage;) {
+                if (resident(device, D, gqa, more) < units) break;
+                sh = more;
+            }
+            return sh;
+        }
+    }
+    return ClusterShape{};
+}
+
+// CTAs of a step kernel that builds a plan over at most `ids` page ids: one
+// where its warps hold them in a round or two (12 rows of up to 85 pages: the
+// step is 2 us shorter than with 4 or 8, which the cluster's start costs),
+// else 8 (8 rows of 2049: 9.5 us, 10.3 with 4, 14.2 with 1).
+int step_ctas(int64_t ids) { return ids <= 2048 ? 1 : 8; }
+
+// Threads per CTA of a step kernel: enough warps to copy the page ids in one
+// go (a warp has 128 in flight), 8 to 16 of them, and a thread per row where a
+// block can have one (the rows' order depends on that).  Device step of 32 /
+// 64 / 8 / 96 rows of up to 2.4k / 0.9k / 33k / 2k tokens with 256, 512 and 1024
+// threads: 5.7 5.9 6.9 / 5.5 5.8 6.9 / 6.9 6.5 7.3 / 7.5 7.0 7.7 us; without a
+// plan 1.65, 1.67 and 1.9.
+int step_threads(int64_t batch, int64_t ids, int ctas)
+{
+    if (batch > 512) return 1024;
+    return batch > 256 || ids > (int64_t)ctas * 1024 ? 512 : 256;
+}
+
+}  // namespace kvd

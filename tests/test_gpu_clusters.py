@@ -1,5 +1,6 @@
 """Decode attention through thread-block clusters (small steps, no second
-pass): every cluster shape the host picks, rows that end on and around page
+pass): every cluster shape the host picks (test_rules_cpu.py checks that these
+steps pick it), rows that end on and around page
 boundaries, rows with fewer pages than the cluster has warps, and rows that
 outgrow what the shape was picked for, against the float64 oracle."""
 import numpy as np
@@ -23,10 +24,10 @@ pytestmark = pytest.mark.gpu
     (8, 8, 128, [700, 1, 16, 15]),                  # 8 of 4
     (56, 8, 128, [300, 511, 512]),
     (16, 16, 128, [300, 17, 0, 31, 250]),           # 4 of 4
-    (24, 24, 64, [100, 64, 63, 1, 47]),
+    (24, 24, 64, [100, 64, 63, 1, 47]),            # 2 of 4
     (16, 8, 128, [90, 0, 15, 16, 47, 90, 3, 2, 77, 61, 33, 32]),
-    (8, 8, 64, [60 - 3 * (b % 20) for b in range(24)]),   # 2 of 4
-    (6, 2, 64, [40 - (b % 40) for b in range(120)]),      # 1 of 4
+    (8, 8, 64, [60 - 3 * (b % 20) for b in range(24)]),   # 1 of 4
+    (6, 2, 64, [40 - (b % 40) for b in range(120)]),
 ])
 def test_cluster_shapes_match_the_oracle(kvlib, Hq, Hkv, d, lens, fused):
     cfg = wl.custom("cluster", 2, Hq, Hkv, d, len(lens), lens=lens, seed=91 + Hq + d, page_order="shuffled")

@@ -1,5 +1,6 @@
-"""The library's host-side choices, compiled alone with the host compiler (no
-GPU, no library)."""
+"""The library's host-side choices (csrc/kvd_rules.cpp), compiled alone with the
+host compiler: no GPU, no library.  The device's part of them, how many clusters
+of a shape it holds at once, is a table of what a GB300 answers."""
 import ctypes
 import os
 import subprocess
@@ -19,6 +20,68 @@ def compile_host(path, source, *files):
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, "-I", os.path.join(cuda, "include"),
                     src, *(os.path.join(CSRC, x) for x in files), "-o", lib], check=True)
     return ctypes.CDLL(lib)
+
+
+#: clusters of (CTAs, warps) with 1, 2, .. ring stages that a GB300 holds at once, by head_dim
+RESIDENT = {
+    128: {(8, 8): (15, 15, 15), (8, 4): (51, 51, 36), (4, 4): (110, 110, 74), (2, 4): (228, 228, 152),
+          (1, 4): (456, 456, 304)},
+    64: {(8, 8): (36, 36, 36, 15, 15, 15), (8, 4): (74, 74, 74, 51, 36, 36), (4, 4): (148, 148, 148, 110, 74, 74),
+         (2, 4): (304, 304, 304, 228, 152, 152), (1, 4): (608, 608, 608, 456, 304, 304)},
+}
+WARPS = 152 * 8   # resident warps of the split pass
+
+
+class Rules:
+    def __init__(self, lib):
+        self.lib = lib
+        for d, shapes in RESIDENT.items():
+            for (c, w), counts in shapes.items():
+                for r, n in enumerate(counts):
+                    lib.set_resident(d, c, w, r + 1, n)
+
+    def shape(self, hq, hkv, d, pages, spread=False):
+        """(CTAs, warps, stages) of a step over rows of these page counts; no CTAs: a split plan."""
+        out = (ctypes.c_int * 3)()
+        self.lib.shape(d, int(hq > hkv), hkv, len(pages), sum(pages), max(pages), int(spread), out)
+        return tuple(out)
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    return Rules(compile_host(str(tmp_path_factory.mktemp("rules")), """
+        #include "kvd_internal.h"
+        using namespace kvd;
+        static int known[2][9][9][8];
+        static int resident(int, int D, bool, const ClusterShape& s) { return known[D == 128][s.ctas][s.warps][s.ring]; }
+        extern "C" void set_resident(int D, int c, int w, int r, int n) { known[D == 128][c][w][r] = n; }
+        extern "C" void shape(int D, int gqa, int hkv, int rows, int pages, int max_pages, int spread, int* out)
+        {
+            const ClusterShape s = pick_cluster_shape(resident, 0, D, gqa, hkv, rows, pages, max_pages, spread);
+            out[0] = s.ctas;
+            out[1] = s.warps;
+            out[2] = s.ring;
+        }
+    """, "kvd_rules.cpp"))
+
+
+def pages_of(lens):
+    return [(n + 15) // 16 for n in lens]
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,lens,shape", [   # the steps of the GPU test of every cluster shape, after one token
+    (28, 4, 128, [2200, 33], (8, 8)),
+    (14, 2, 64, [2300, 0], (8, 8)),
+    (8, 8, 128, [700, 1, 16, 15], (8, 4)),
+    (56, 8, 128, [300, 511, 512], (8, 4)),
+    (16, 16, 128, [300, 17, 0, 31, 250], (4, 4)),
+    (24, 24, 64, [100, 64, 63, 1, 47], (2, 4)),
+    (16, 8, 128, [90, 0, 15, 16, 47, 90, 3, 2, 77, 61, 33, 32], (2, 4)),
+    (8, 8, 64, [60 - 3 * (b % 20) for b in range(24)], (1, 4)),
+    (6, 2, 64, [40 - (b % 40) for b in range(120)], (1, 4)),
+])
+def test_cluster_shapes_of_small_steps(rules, Hq, Hkv, d, lens, shape):
+    assert rules.shape(Hq, Hkv, d, pages_of([n + 1 for n in lens]))[:2] == shape
 
 
 def test_setup_runs_once_on_each_device(tmp_path):
