@@ -782,7 +782,7 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         total_units += (int64_t)np_after[b] * c->cfg.num_kv_heads;
     }
     const int32_t max_np = *std::max_element(np_after.begin(), np_after.end());
-    const int32_t T = c->split_override ? c->split_override
+    int32_t T = c->split_override ? c->split_override
                                         : auto_item_pages(c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads,
                                                           resident_warps(c), batch, total_units / c->cfg.num_kv_heads,
                                                           max_np, false);
@@ -798,17 +798,31 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
     if (!c->split_override && !c->host_only)
         shape = cluster_shape(c->device, c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, batch,
                               total_units / c->cfg.num_kv_heads, max_np);
-    const int32_t cap = chunk_cap(c->group > 1, (int64_t)batch * c->cfg.num_kv_heads, resident_warps(c), max_np, T);
+    int32_t cap = chunk_cap(c->group > 1, (int64_t)batch * c->cfg.num_kv_heads, resident_warps(c), max_np, T);
     int64_t entries = 0;
     int32_t stride = 1;
     bool split = false;
     int32_t max_chunks = 1;
-    for (int32_t b = 0; b < batch && !shape.ctas; ++b) {
-        const int nch = row_chunks(np_after[b], row_item_pages(T, rank[b], batch), cap);
-        entries += nch;
-        split = split || nch > 1;
-        max_chunks = std::max(max_chunks, nch);
-        stride = std::max(stride, (np_after[b] + nch - 1) / nch);
+    auto size_plan = [&] {
+        entries = 0;
+        stride = max_chunks = 1;
+        for (int32_t b = 0; b < batch; ++b) {
+            const int nch = row_chunks(np_after[b], row_item_pages(T, rank[b], batch), cap);
+            entries += nch;
+            max_chunks = std::max(max_chunks, nch);
+            stride = std::max(stride, (np_after[b] + nch - 1) / nch);
+        }
+        split = max_chunks > 1;
+    };
+    if (!shape.ctas) size_plan();
+    // While device steps are enabled the buffers stay: an automatic plan that
+    // does not fit is cut as device steps cut it, which always does.
+    if (!shape.ctas && c->dev_mode && !c->split_override && !c->dev_split_override && batch <= c->dev_max_batch &&
+        (entries * stride > c->item_pages_cap || entries > c->plan_cap ||
+         entries * c->cfg.num_kv_heads > c->slot_cap)) {
+        T = c->dev_item_pages;
+        cap = c->dev_chunk_cap;
+        size_plan();
     }
     if (!c->host_only && !shape.ctas)
         if (int rc = grow_scratch(c, entries, entries * c->cfg.num_kv_heads, entries * stride,

@@ -5,11 +5,12 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from oracle import PagePoolModel
 from paper_2603_12707_gb300 import kvdecode as kd
 from paper_2603_12707_gb300 import workloads as wl
 
-from _gpu_common import Tracked, assert_close, bf16_to_f64
+from _gpu_common import Tracked, assert_close, bf16_to_f64, u16
 
 pytestmark = pytest.mark.gpu
 
@@ -252,6 +253,41 @@ def test_host_step_cannot_move_buffers_under_device_steps(kvlib):
     kd.kv_cache_device_steps(h, 2, False)
     kd.kv_begin_step(h, seqs)
     assert [kd.kv_seq_info(h, s_)[0] for s_ in seqs] == [1901] * 4
+    kd.kv_cache_destroy(h)
+
+
+@pytest.mark.parametrize("held,tokens,rows", [([100, 100, 100, 100], 1600, 16), ([], 1600, 17), ([16], 1350, 12),
+                                               ([1800] * 3, 1900, 17)])
+def test_host_steps_fit_what_device_steps_reserved(kvlib, held, tokens, rows):
+    """A host-planned step of up to max_batch rows runs while device steps are
+    enabled, whatever was held when they were, in the buffers that were
+    reserved then; its result matches the oracle."""
+    lens = [tokens - 16 * (b % 3) for b in range(rows)]
+    cfg = wl.custom("fits", 1, 64, 32, 64, rows, lens=lens, seed=97)
+    h = kd.kv_cache_create(kd.make_config(1, 64, 32, 64, 17 * 121, 17, 121))
+    seqs = [kd.kv_seq_create(h) for _ in range(17)]
+    for s_, n in zip(seqs, held):
+        kd.kv_seq_reserve(h, s_, n)
+    kd.kv_cache_device_steps(h, 17)
+    ks, vs = [], []
+    for b, n in enumerate(lens):
+        kd.kv_seq_reserve(h, seqs[b], n - (held[b] if b < len(held) else 0))
+        k, v = (wl.kv_block(cfg, 0, b, n, kind, "cuda") for kind in "kv")
+        kd.kv_write_tokens(h, 0, seqs[b], 0, n, k, v)
+        ks.append(u16(k))
+        vs.append(u16(v))
+    q, kn, vn = wl.step_inputs(cfg, 0, 0, "cuda")
+    out = torch.empty_like(q)
+    kd.kv_begin_step(h, seqs[:rows])
+    kd.decode_attention_append(h, 0, rows, q, kn, vn, out)
+    torch.cuda.synchronize()
+    assert kd.kv_cache_query(h).device_error == 0
+    keep = [0, 1, rows - 1]
+    k = [np.concatenate([ks[b], u16(kn[b:b + 1])]) for b in keep]
+    v = [np.concatenate([vs[b], u16(vn[b:b + 1])]) for b in keep]
+    ref = oracle.decode_attention(u16(q)[keep], [len(x) for x in k], np.concatenate(k), np.concatenate(v))
+    vmax = np.array([np.abs(oracle.bf16_to_f64(x)).max() for x in v])
+    assert_close(bf16_to_f64(out)[keep], ref, vmax, gqa=True)
     kd.kv_cache_destroy(h)
 
 
