@@ -308,7 +308,9 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
 
 // Items per row at most: twice the usual cap when units (rows x KV heads) x the
 // usual cap would leave resident warps without an item and some row (of up
-// to max_pages pages) is long enough to use more items of T pages.
+// to max_pages pages) is long enough to use more items of T pages, and 32 if
+// it uses more than 16 (14/2 heads, 17 rows of 6700 tokens, 26 items: 19.7 us
+// a layer, cut at 16 22.9; Qwen heads, 8 rows of 3000: 11.1 and 13.1).
 // Otherwise 32 for MHA and 16 for GQA: a GQA row of at most 16 items merges
 // in one round trip with the 16-item variant, the largest whose registers
 // fit beside the resident GQA split pass (Qwen shape: 0.742 at 32, 0.769 at

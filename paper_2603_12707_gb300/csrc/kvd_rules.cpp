@@ -33,8 +33,10 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
 
 int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T)
 {
-    const bool few_units = units * kChunkCap < warps;
-    if (few_units && max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
+    if (units * kChunkCap < warps) {
+        if (max_pages > (int64_t)kChunkCap * T) return kMaxChunks;
+        if (max_pages > (int64_t)kChunkCapGqa * T) return kChunkCap;
+    }
     return gqa ? kChunkCapGqa : kChunkCap;
 }
 

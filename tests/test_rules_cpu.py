@@ -62,6 +62,10 @@ def rules(tmp_path_factory):
             out[1] = s.warps;
             out[2] = s.ring;
         }
+        extern "C" int cap(int gqa, int units, int warps, int max_pages, int T)
+        {
+            return chunk_cap(gqa, units, warps, max_pages, T);
+        }
     """, "kvd_rules.cpp"))
 
 
@@ -82,6 +86,17 @@ def pages_of(lens):
 ])
 def test_cluster_shapes_of_small_steps(rules, Hq, Hkv, d, lens, shape):
     assert rules.shape(Hq, Hkv, d, pages_of([n + 1 for n in lens]))[:2] == shape
+
+
+def test_few_units_get_the_items_that_their_rows_ask_for(rules):
+    """Units that would leave resident warps without an item at the usual cap
+    are cut into items of T pages, not fewer larger ones."""
+    for gqa in (0, 1):
+        for units in (1, 8, 32, 37):
+            for T in (2, 7, 14):
+                for pages in (1, 16 * T, 16 * T + 1, 31 * T, 32 * T, 33 * T, 64 * T):
+                    assert rules.lib.cap(gqa, units, WARPS, pages, T) >= min(64, -(-pages // T))
+    assert rules.lib.cap(1, 38, WARPS, 2000, 2) == 16 and rules.lib.cap(0, 38, WARPS, 2000, 2) == 32
 
 
 def test_setup_runs_once_on_each_device(tmp_path):
