@@ -24,6 +24,16 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
         const double want = (double)warps / (double)units * (share < 15 ? 1.06 : 1.3) + (share < 15 ? 0.0 : 0.5);
         const int64_t items = std::max<int64_t>(1, (int64_t)want);
         few = (max_pages + (growing ? max_pages / 8 : 0) + items - 1) / items;
+        // The 1.06 is for rows shorter than the longest.  Where the mean row's
+        // items outnumber the warps all the same, the few warps that work a
+        // second item cost up to 4 pages' time (d = 64: 7): items a page larger
+        // (d = 64: up to 3) if that is enough (us per layer; 32 heads, 229
+        // pages in items of 6 / 7: 15.0 / 11.9; 3 rows of 88, 7 / 8: 15.9 /
+        // 12.7; 8/8 heads at d = 64, 3 rows of 738, 14 / 15: 19.4 / 14.8; but
+        // 32 heads, 8 rows of 65, 14 / 17: 21.2 / 22.6).
+        int64_t fit = few;
+        while (share < 15 && fit < max_pages && (pages + rows * fit - 1) / (rows * fit) * units > warps) ++fit;
+        if (fit - few < 2 * 128 / D) few = fit;
     } else if (max_pages <= 8 || (units >= warps && 10 * max_pages * warps <= 13 * total)) {
         few = max_pages;
     }

@@ -47,6 +47,10 @@ class Rules:
         return tuple(out)
 
 
+    def item_pages(self, hq, hkv, d, pages, growing=False):
+        return self.lib.item_pages(d, int(hq > hkv), hkv, WARPS, len(pages), sum(pages), max(pages), int(growing))
+
+
 @pytest.fixture(scope="module")
 def rules(tmp_path_factory):
     return Rules(compile_host(str(tmp_path_factory.mktemp("rules")), """
@@ -61,6 +65,10 @@ def rules(tmp_path_factory):
             out[0] = s.ctas;
             out[1] = s.warps;
             out[2] = s.ring;
+        }
+        extern "C" int item_pages(int D, int gqa, int hkv, int warps, int rows, int pages, int max_pages, int growing)
+        {
+            return auto_item_pages(D, gqa, hkv, warps, rows, pages, max_pages, growing);
         }
         extern "C" int cap(int gqa, int units, int warps, int max_pages, int T)
         {
@@ -86,6 +94,24 @@ def pages_of(lens):
 ])
 def test_cluster_shapes_of_small_steps(rules, Hq, Hkv, d, lens, shape):
     assert rules.shape(Hq, Hkv, d, pages_of([n + 1 for n in lens]))[:2] == shape
+
+
+@pytest.mark.parametrize("growing", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,d,pages", [
+    (32, 32, 128, [229]),
+    (32, 32, 128, [91, 88, 85]),
+    (8, 8, 128, [263, 257, 250]),
+    (56, 8, 128, [571, 560, 541]),
+    (56, 8, 128, [774, 760, 742]),
+    (8, 8, 64, [738] * 3),
+    (14, 2, 128, [399 + 2 * b for b in range(17)]),
+])
+def test_one_item_per_warp_is_not_a_few_more(rules, Hq, Hkv, d, pages, growing):
+    """Even rows of short shares get one item per resident warp: with a few
+    more, some warps would work a second one while all others wait."""
+    T = rules.item_pages(Hq, Hkv, d, pages, growing)
+    items = sum(-(-n // T) for n in pages) * Hkv
+    assert 0.75 * WARPS <= items <= WARPS
 
 
 def test_few_units_get_the_items_that_their_rows_ask_for(rules):
