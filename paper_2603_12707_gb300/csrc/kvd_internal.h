@@ -286,7 +286,9 @@ CUresult encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_
 // head.  But an item costs about 0.6 pages beside its own, and a row of several
 // a merge, so where a warp's share is short (up to 30 pages of d = 128),
 //  - rows of nearly equal length are cut into one item per resident warp, or
-//    up to 1.3 for shares past 15 pages (us per layer, before -> now; 32 heads
+//    up to 1.3 for shares past 15 pages of 200 units or more (fewer, longer
+//    rows end on items too long for a second round: 32 heads, 16000 tokens
+//    45.1, at three items per warp 39.7; 3 rows of 3100 28.4 and 26.0) (us per layer, before -> now; 32 heads
 //    of 900 tokens, B 5 / 8 / 12: 17.0 -> 14.3, 22.8 -> 20.1, 30.4 -> 29.1;
 //    16/8 heads of 500, B 32: 14.9 -> 12.6; 14/2 heads at d = 64 of 1000, B
 //    128: 17.2 -> 15.2; 8/8 at d = 64 of 700, B 64: 22.1 -> 18.6);

@@ -20,7 +20,7 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
     if (share > 30 || rows < 1) return (int32_t)T;
     const double even = (double)max_pages * (double)rows / (double)std::max<int64_t>(1, pages);   // longest row / mean row
     int64_t few = 0;
-    if (even <= (share < 15 ? 1.35 : 1.15)) {
+    if (share < 15 ? even <= 1.35 : even <= 1.15 && 6 * units >= warps) {
         const double want = (double)warps / (double)units * (share < 15 ? 1.06 : 1.3) + (share < 15 ? 0.0 : 0.5);
         const int64_t items = std::max<int64_t>(1, (int64_t)want);
         few = (max_pages + (growing ? max_pages / 8 : 0) + items - 1) / items;

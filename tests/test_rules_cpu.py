@@ -114,6 +114,19 @@ def test_one_item_per_warp_is_not_a_few_more(rules, Hq, Hkv, d, pages, growing):
     assert 0.75 * WARPS <= items <= WARPS
 
 
+@pytest.mark.parametrize("growing", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,d,pages", [
+    (32, 32, 128, [1001]),
+    (32, 32, 128, [501] * 2),
+    (40, 40, 128, [404] * 2),
+    (32, 32, 128, [200, 195, 190]),
+    (14, 2, 64, [1873 - 11 * b for b in range(13)]),
+])
+def test_long_shares_of_few_units_have_several_items_per_warp(rules, Hq, Hkv, d, pages, growing):
+    T = rules.item_pages(Hq, Hkv, d, pages, growing)
+    assert T <= -(-sum(pages) * Hkv // ((2 if Hq > Hkv else 3) * WARPS))
+
+
 def test_few_units_get_the_items_that_their_rows_ask_for(rules):
     """Units that would leave resident warps without an item at the usual cap
     are cut into items of T pages, not fewer larger ones."""
