@@ -292,8 +292,13 @@ CUresult encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_
 //    of 900 tokens, B 5 / 8 / 12: 17.0 -> 14.3, 22.8 -> 20.1, 30.4 -> 29.1;
 //    16/8 heads of 500, B 32: 14.9 -> 12.6; 14/2 heads at d = 64 of 1000, B
 //    128: 17.2 -> 15.2; 8/8 at d = 64 of 700, B 64: 22.1 -> 18.6);
-//  - rows of up to 8 pages, or unequal ones of which none is much longer than
-//    a warp's share, stay whole (56/8 heads, 106 rows of up to 105 tokens:
+//  - unequal rows stay whole if none is much longer than a warp's share, or up
+//    to 8 pages and four shares.  A host's step then runs without a merge pass
+//    (rows of up to 5 pages always); a device step launches it in any case, and
+//    the line is at 2.3 shares (40/40 heads, a row of 101 tokens and 10 of
+//    10-24, whole 6.2, as items of 2 pages 4.7; 21 of up to 104 6.4 and 5.7;
+//    8/8 heads, 33 of up to 8 pages 6.9 and 4.7, device step 9.1 and 5.9; 99 of
+//    up to 6 8.1 and 7.0, device step 9.2 and 9.6) (56/8 heads, 106 rows of up to 105 tokens:
 //    13.0 -> 9.9; 32 heads, 57 rows of up to 263: 26.1 -> 23.1).
 // Longer shares gain nothing (32 heads of 900, B 24 / 32: best target within
 // 2 % of a third of the share), up to items so long that the last ones to end

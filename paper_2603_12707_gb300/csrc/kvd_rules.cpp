@@ -34,7 +34,9 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
         int64_t fit = few;
         while (share < 15 && fit < max_pages && (pages + rows * fit - 1) / (rows * fit) * units > warps) ++fit;
         if (fit - few < 2 * 128 / D) few = fit;
-    } else if (max_pages <= 8 || (units >= warps && 10 * max_pages * warps <= 13 * total)) {
+    } else if ((!growing && max_pages <= 5) ||
+               (max_pages <= 8 && 10 * max_pages * warps <= (growing ? 23 : 40) * total) ||
+               (units >= warps && 10 * max_pages * warps <= 13 * total)) {
         few = max_pages;
     }
     if (few >= max_pages) few = std::max<int64_t>(few, 16);

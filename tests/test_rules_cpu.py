@@ -127,6 +127,21 @@ def test_long_shares_of_few_units_have_several_items_per_warp(rules, Hq, Hkv, d,
     assert T <= -(-sum(pages) * Hkv // ((2 if Hq > Hkv else 3) * WARPS))
 
 
+@pytest.mark.parametrize("Hq,Hkv,d,pages,whole", [
+    (40, 40, 128, [7] + [1 + b % 2 for b in range(10)], (False, False)),
+    (8, 8, 128, [8] + [2 + b % 2 for b in range(32)], (False, False)),
+    (32, 32, 128, [7] + [1 + b % 3 for b in range(20)], (False, False)),
+    (8, 8, 128, [6] + [2 + b % 3 for b in range(98)], (True, False)),
+    (40, 40, 128, [7] + [2 + b % 3 for b in range(33)], (True, True)),
+    (16, 8, 128, [4] + [1] * 27, (True, False)),
+    (28, 4, 128, [5] + [2] * 60, (True, False)),
+])
+def test_short_unequal_rows_stay_whole_only_where_it_pays(rules, Hq, Hkv, d, pages, whole):
+    """A long row kept whole is one warp's work while the others wait; device
+    steps launch the merge pass in any case."""
+    assert tuple(rules.item_pages(Hq, Hkv, d, pages, growing) >= max(pages) for growing in (False, True)) == whole
+
+
 def test_few_units_get_the_items_that_their_rows_ask_for(rules):
     """Units that would leave resident warps without an item at the usual cap
     are cut into items of T pages, not fewer larger ones."""
