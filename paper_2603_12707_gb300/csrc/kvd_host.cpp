@@ -814,7 +814,10 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         }
         split = max_chunks > 1;
     };
-    if (!shape.ctas) size_plan();
+    size_plan();
+    if (shape.ctas && !split &&
+        whole_rows_beat_clusters(c->cfg.head_dim, c->group, batch, total_units / c->cfg.num_kv_heads, max_np))
+        shape = ClusterShape{};
     // While device steps are enabled the buffers stay: an automatic plan that
     // does not fit is cut as device steps cut it, which always does.
     if (!shape.ctas && c->dev_mode && !c->split_override && !c->dev_split_override && batch <= c->dev_max_batch &&

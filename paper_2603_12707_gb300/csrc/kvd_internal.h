@@ -405,6 +405,8 @@ ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_
 using ResidentClusters = int (*)(int device, int D, bool gqa, const ClusterShape& shape);
 ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bool gqa, int num_kv_heads,
                                 int64_t batch, int64_t pages, int64_t max_pages, bool spread = false);
+// Whether a plan that leaves every row whole is the better one where clusters would do.
+bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int64_t max_pages);
 // CTAs of a step kernel that builds a plan over at most `ids` page ids, and its threads per CTA.
 int step_ctas(int64_t ids);
 int step_threads(int64_t batch, int64_t ids, int ctas);

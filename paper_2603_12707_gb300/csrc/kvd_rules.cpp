@@ -111,6 +111,18 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
     return ClusterShape{};
 }
 
+// A plan of whole rows has no merge pass, so a row of one page is quickest as
+// one warp's item; of two for large GQA groups, whose exchange over the cluster
+// takes long, and where few rows have a second page (us per layer, clusters and
+// whole rows; 56/8 heads, 6 rows of up to 12 tokens 3.2 and 2.5; 28/4 heads, 51
+// of 8 4.1 and 2.7; 32 heads, 3 of 8 2.5 and 2.4; 14/2 heads, 60 of up to 2
+// pages 3.8 and 2.7; 16/8 heads, 43 of which one has 2 3.0 and 2.6; but 40/40
+// heads, one of 2 2.6 and 2.9, 14/2 heads at d = 64, 76 of up to 2 2.5 and 2.8).
+bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int64_t max_pages)
+{
+    return max_pages == 1 || (max_pages == 2 && ((group > 4 && D == 128) || 4 * pages <= 5 * rows));
+}
+
 // CTAs of a step kernel that builds a plan over at most `ids` page ids: one
 // where its warps hold them in a round or two (12 rows of up to 85 pages: the
 // step is 2 us shorter than with 4 or 8, which the cluster's start costs),
