@@ -52,6 +52,27 @@ int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int
     return gqa ? kChunkCapGqa : kChunkCap;
 }
 
+// Pages that a warp of the longest row may have in clusters of n warps for each
+// of `units` units, whose layer holds `bytes` of K and V: the time that takes
+// against the plan's merge pass and what the layer's bytes take in any case.
+// GQA: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB), up to 25 MB, which keep
+// the HBM busy beside them.  An MHA page is worked on the CUDA cores and takes
+// a warp about twice as long: 4 pages, and 3 and 1 more per 6 MB, up to 7, or 5
+// where half of the GPU's warps have nothing that the plan would give them (d =
+// 64: 5 and 1 more per 4.5 MB, or up to 7 with 8 warps to a CTA).  Us per layer,
+// plan and clusters, 8/8 heads: 2 rows of 3000, 6 pages 7.7 and 8.2; 6 of up to
+// 2330, 10 pages 7.6 and 10.6; 16/16, one of 2500, 5 pages 7.4 and 6.9, of
+// 5000, 10 pages 9.6 and 12.7; 40/40, 9 of up to 380, 6 pages 6.5 and 8.0, 3 of
+// up to 730, 6 pages 9.1 and 7.5; 8/8 at d = 64, 17 of up to 1080, 9 pages 10.4
+// and 7.2, 2 of 9200 and 1500, 9 pages 8.4 and 9.6.
+int64_t most_pages_per_warp(int D, bool gqa, int64_t units, int64_t n, int64_t bytes)
+{
+    if (gqa) return (20000000 + std::min<int64_t>(bytes, 25000000)) / (D == 128 ? 4000000 : 2800000);
+    if (D == 128)
+        return std::min<int64_t>(n < 64 && units * n < 600 ? 5 : 7, std::max<int64_t>(4, (17000000 + bytes) / 6000000));
+    return n == 64 ? 7 : (22500000 + bytes) / 4500000;
+}
+
 // The line between the two, measured as us per layer of graph-replayed steps
 // (split plan -> clusters).  Clusters save the merge pass and its dependency
 // hop (2.3 us), but cut the rows evenly, without the plan's balancing: they
@@ -96,11 +117,7 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
         const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
         for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
             if (10 * (int64_t)resident(device, D, gqa, sh) < 11 * units) continue;
-            // the longest row's warps against what the layer's bytes take in
-            // any case: 5 pages (d = 64: 7) and 1 more per 4 MB (2.8 MB) that
-            // the layer holds, up to 25 MB, which keep the HBM busy beside them
-            const int64_t beside = std::min<int64_t>(bytes, 25000000);
-            if (per_warp * (D == 128 ? 4000000 : 2800000) > 20000000 + beside) return ClusterShape{};
+            if (per_warp > most_pages_per_warp(D, gqa, units, n, bytes)) return ClusterShape{};
             for (ClusterShape more = sh; spread && ++more.ring <= kClusterRingBytes / stage;) {
                 if (resident(device, D, gqa, more) < units) break;
                 sh = more;

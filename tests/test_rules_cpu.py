@@ -160,6 +160,25 @@ def test_rows_of_one_or_two_pages_stay_whole(rules, d, group, pages, whole):
     assert bool(rules.lib.whole(d, group, len(pages), sum(pages), max(pages))) == whole
 
 
+@pytest.mark.parametrize("Hq,Hkv,d,lens,clusters", [
+    (8, 8, 128, [3953, 3162], False),
+    (8, 8, 128, [2330, 1500, 800, 200, 150, 100], False),
+    (40, 40, 128, [380, 190, 100, 60, 40, 30, 20, 15, 10], False),
+    (32, 32, 128, [290, 29, 40, 50, 60, 30, 35, 45, 70], False),
+    (8, 8, 64, [9200, 1500], False),
+    (8, 8, 64, [795] + [19 + b * 4 for b in range(28)], False),
+    (16, 16, 128, [5000], False),
+    (32, 32, 128, [2000], True),
+    (32, 32, 128, [900, 500, 300], True),
+    (40, 40, 128, [730, 400, 80], True),
+    (8, 8, 128, [7000], True),
+    (8, 8, 64, [1080 - 40 * b for b in range(17)], True),
+    (28, 4, 128, [4000, 2500], True),
+])
+def test_clusters_where_the_longest_rows_warps_keep_up(rules, Hq, Hkv, d, lens, clusters):
+    assert (rules.shape(Hq, Hkv, d, pages_of(lens))[0] > 0) == clusters
+
+
 def test_few_units_get_the_items_that_their_rows_ask_for(rules):
     """Units that would leave resident warps without an item at the usual cap
     are cut into items of T pages, not fewer larger ones."""
