@@ -986,7 +986,8 @@ static int launch_attention(kv_cache* c, const char* what, int32_t layer, int32_
     p.kv_map = 1;
     const bool pdl = c->chain_launches == c->launches && c->chain_stream == stream;
     // After the step kernel: placed while it runs, reads nothing before its end.
-    const bool after_step = !pdl && c->step_launches == c->launches && c->step_stream == stream;
+    const bool after_step = !pdl && c->step_launches == c->launches && c->step_stream == stream &&
+                            (c->step_cluster.ctas || place_first_layer_early(grid, resident));
     p.early = after_step ? 0 : 1;
     // A launch that appends nothing itself loads each row's last page after its
     // wait if any launch of the chain wrote new tokens, kv_append or fused and

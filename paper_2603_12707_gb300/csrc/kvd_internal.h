@@ -407,6 +407,8 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
                                 int64_t batch, int64_t pages, int64_t max_pages, bool spread = false);
 // Whether a plan that leaves every row whole is the better one where clusters would do.
 bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int64_t max_pages);
+// Whether the split pass of a step's first layer is launched early (see kvd_rules.cpp).
+bool place_first_layer_early(int64_t ctas, int64_t slots);
 // CTAs of a step kernel that builds a plan over at most `ids` page ids, and its threads per CTA.
 int step_ctas(int64_t ids);
 int step_threads(int64_t batch, int64_t ids, int ctas);

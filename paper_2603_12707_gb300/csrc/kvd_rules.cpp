@@ -140,6 +140,15 @@ bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int
     return max_pages == 1 || (max_pages == 2 && ((group > 4 && D == 128) || 4 * pages <= 5 * rows));
 }
 
+// The first layer after a step kernel may be placed while that runs and what
+// ran before it leaves, which saves up to 1 us a step.  But a split pass that
+// fills less than half of its slots then crowds on the SMs that are empty
+// first, and the layers after it, each placed where the one before the last
+// left, keep that pattern (us per layer, placed early and not; 28/4 heads, one
+// row of 20000 tokens, 256 of 1216 slots 14.3 and 13.6; 8/8 heads, one of 12000,
+// 512 slots 14.5 and 14.1; at d = 64 9.8 and 9.4; from 1216 on the same).
+bool place_first_layer_early(int64_t ctas, int64_t slots) { return 2 * ctas >= slots; }
+
 // CTAs of a step kernel that builds a plan over at most `ids` page ids: one
 // where its warps hold them in a round or two (12 rows of up to 85 pages: the
 // step is 2 us shorter than with 4 or 8, which the cluster's start costs),

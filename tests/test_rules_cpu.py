@@ -74,6 +74,7 @@ def rules(tmp_path_factory):
         {
             return whole_rows_beat_clusters(D, group, rows, pages, max_pages);
         }
+        extern "C" int early(int ctas, int slots) { return place_first_layer_early(ctas, slots); }
         extern "C" int cap(int gqa, int units, int warps, int max_pages, int T)
         {
             return chunk_cap(gqa, units, warps, max_pages, T);
@@ -177,6 +178,11 @@ def test_rows_of_one_or_two_pages_stay_whole(rules, d, group, pages, whole):
 ])
 def test_clusters_where_the_longest_rows_warps_keep_up(rules, Hq, Hkv, d, lens, clusters):
     assert (rules.shape(Hq, Hkv, d, pages_of(lens))[0] > 0) == clusters
+
+
+def test_small_grids_are_not_placed_beside_the_step_kernel(rules):
+    assert not any(rules.lib.early(n, WARPS) for n in (1, 256, 512, 607))
+    assert all(rules.lib.early(n, WARPS) for n in (608, 1216))
 
 
 def test_few_units_get_the_items_that_their_rows_ask_for(rules):
