@@ -20,6 +20,7 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
     if (share > 30 || rows < 1) return (int32_t)T;
     const double even = (double)max_pages * (double)rows / (double)std::max<int64_t>(1, pages);   // longest row / mean row
     int64_t few = 0;
+    bool whole = false;   // every row is one item
     if (share < 15 ? even <= 1.35 : even <= 1.15 && 6 * units >= warps) {
         const double want = (double)warps / (double)units * (share < 15 ? 1.06 : 1.3) + (share < 15 ? 0.0 : 0.5);
         const int64_t items = std::max<int64_t>(1, (int64_t)want);
@@ -34,12 +35,16 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
         int64_t fit = few;
         while (share < 15 && fit < max_pages && (pages + rows * fit - 1) / (rows * fit) * units > warps) ++fit;
         if (fit - few < 2 * 128 / D) few = fit;
+        whole = items == 1;
     } else if ((!growing && max_pages <= 5) ||
                (max_pages <= 8 && 10 * max_pages * warps <= (growing ? 23 : 40) * total) ||
                (units >= warps && 10 * max_pages * warps <= 13 * total)) {
         few = max_pages;
+        whole = true;
     }
-    if (few >= max_pages) few = std::max<int64_t>(few, 16);
+    // (also the last rows', whose target is a fraction; not for few units, whose
+    // rows would have too few items once they have grown)
+    if (whole) few = std::max<int64_t>(few, 16);
     return (int32_t)std::max(T, std::min<int64_t>(128, few));
 }
 

@@ -185,6 +185,17 @@ def test_small_grids_are_not_placed_beside_the_step_kernel(rules):
     assert all(rules.lib.early(n, WARPS) for n in (608, 1216))
 
 
+@pytest.mark.parametrize("Hq,Hkv,d,B", [(32, 32, 128, 1), (28, 4, 128, 8), (8, 8, 64, 4), (14, 2, 64, 13), (32, 32, 128, 12)])
+def test_rows_that_start_short_fill_the_gpu_when_grown(rules, Hq, Hkv, d, B):
+    """Device steps keep the target size of the lengths held when they were
+    enabled: few units of a page each still get as many items as 60 grown
+    pages make, up to three per warp or the cap."""
+    for held in (1, 2, 4):
+        T = rules.item_pages(Hq, Hkv, d, [held] * B, True)
+        items = min(-(-60 // T), rules.lib.cap(int(Hq > Hkv), B * Hkv, WARPS, 256, T)) * B * Hkv
+        assert items >= min(WARPS, 30 * B * Hkv, 16 * B * Hkv if Hq > Hkv else WARPS)
+
+
 def test_few_units_get_the_items_that_their_rows_ask_for(rules):
     """Units that would leave resident warps without an item at the usual cap
     are cut into items of T pages, not fewer larger ones."""
