@@ -444,9 +444,9 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
 }
 
 ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
-                           int64_t max_pages, bool spread)
+                           int64_t max_pages, bool spread, int64_t limit)
 {
-    return pick_cluster_shape(resident_clusters, device, D, gqa, num_kv_heads, batch, pages, max_pages, spread);
+    return pick_cluster_shape(resident_clusters, device, D, gqa, num_kv_heads, batch, pages, max_pages, spread, limit);
 }
 
 }  // namespace kvd

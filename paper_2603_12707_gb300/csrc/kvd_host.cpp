@@ -1135,12 +1135,14 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     a.err = c->err;
     a.step_no = c->step_no;
     // The rows' lengths are the device's: judge the step by the pages held
-    // when device steps were enabled, or by full rows if there were none.
+    // when device steps were enabled, or by full rows if there were none, and
+    // by what the rows may grow to: a captured step keeps its shape.
     ClusterShape shape;
     if (!c->dev_split_override) {
         const int64_t row = c->dev_seqs ? c->dev_row_pages + 1 : c->cfg.max_pages_per_seq;
         const int64_t pages = c->dev_seqs ? (c->dev_pages * batch + c->dev_seqs - 1) / c->dev_seqs : row * batch;
-        shape = cluster_shape(c->device, c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, batch, pages, row);
+        shape = cluster_shape(c->device, c->cfg.head_dim, c->group > 1, c->cfg.num_kv_heads, batch, pages, row, false,
+                              std::min<int64_t>(c->cfg.max_pages_per_seq, c->cfg.num_pages));
     }
     a.no_plan = shape.ctas ? 1 : 0;
     c->last_stream = st;

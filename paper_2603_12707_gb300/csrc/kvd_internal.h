@@ -399,12 +399,14 @@ cudaError_t launch_cluster(int D, bool gqa, bool fused, bool pdl, const ClusterS
 // Clusters for `batch` rows of num_kv_heads that hold `pages` pages per KV
 // head in all and at most max_pages in one row, or ctas == 0: the split plan.
 // spread: for launches that load nothing before their dependency wait.
+// limit: pages that a row may grow to while the shape stays (0: none does).
 ClusterShape cluster_shape(int device, int D, bool gqa, int num_kv_heads, int64_t batch, int64_t pages,
-                           int64_t max_pages, bool spread = false);
+                           int64_t max_pages, bool spread = false, int64_t limit = 0);
 // The same with the number of clusters of a shape that the device holds at once as a callback.
 using ResidentClusters = int (*)(int device, int D, bool gqa, const ClusterShape& shape);
 ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bool gqa, int num_kv_heads,
-                                int64_t batch, int64_t pages, int64_t max_pages, bool spread = false);
+                                int64_t batch, int64_t pages, int64_t max_pages, bool spread = false,
+                                int64_t limit = 0);
 // Whether a plan that leaves every row whole is the better one where clusters would do.
 bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int64_t max_pages);
 // Whether the split pass of a step's first layer is launched early (see kvd_rules.cpp).

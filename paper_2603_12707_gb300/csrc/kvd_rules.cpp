@@ -103,8 +103,27 @@ int64_t most_pages_per_warp(int D, bool gqa, int64_t units, int64_t n, int64_t b
 // LLaVA heads, 850 tokens 5.0 -> 4.3, 40/40 heads, 500 tokens 4.0 -> 3.6, Qwen
 // heads, 8 rows of 700 5.2 -> 4.3).  A launch that does load early is better
 // off with a slot for every CTA at once (LLaVA layer 4.8 -> 5.2).
+//
+// limit: the pages that a row may grow to while the shape stays (device steps
+// and the graphs captured of them; 0 for a step that picks its own).  Warps and
+// stages then serve rows of half of that, and a step whose longest row could
+// still fall far behind runs from the plan, which follows the lengths.  A shape
+// picked for one page a row, graph kept while the rows grow to 2000 / 8000
+// tokens: LLaVA heads, one row 43 / 165 us a layer, Qwen heads, 8 rows 33 / 119
+// (plan 10.3 / 22.8 and 11.0 / 22.7).  Rows that all grow are within 6 % of the
+// plan or faster; most_grown bounds one row of `limit` pages among short ones
+// (us, clusters and plan; Qwen heads, 8 rows, clusters of 32 warps, 4000 / 8000
+// / 16000 tokens 6.6 and 7.0, 10.3 and 9.5, 18.2 and 13.3; 24 rows, 16 warps,
+// 8000 19.7 and 17.9; 56/8 heads, 20 rows, 8 warps, 1000 / 2000 7.2 and 7.3,
+// 11.5 and 9.2; LLaVA heads, 2 rows, 16 warps, 1000 / 2000 5.5 and 7.3, 9.9 and
+// 9.4; 8/8 heads, 4 rows, 32 warps, 2000 / 4000 5.3 and 6.0, 9.2 and 7.9).
+// Clusters of 64 GQA warps cut a row as the plan does (28/4 heads, 32000 tokens
+// 19.8 and 18.8), and the heads of a single row that fill the GPU are bound by
+// their bytes (LLaVA heads, 16000 tokens 41.4 and 39.7).  Short rows of long
+// tables pay: LLaVA heads, one of 16 / 50 tokens 2.9 / 3.1, with a shape of
+// their own 2.5 / 2.5 (plan 4.0 / 5.2).
 ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bool gqa, int num_kv_heads,
-                                int64_t batch, int64_t pages, int64_t max_pages, bool spread)
+                                int64_t batch, int64_t pages, int64_t max_pages, bool spread, int64_t limit)
 {
     constexpr int64_t kMostBytes = 45000000;   // K and V of a layer
     constexpr int kWarpsOf[][2] = {{8, 8}, {8, 4}, {4, 4}, {2, 4}, {1, 4}};
@@ -112,17 +131,27 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
     const int64_t stage = 2 * (int64_t)kPageSize * D * 2;
     const int64_t bytes = pages * num_kv_heads * stage;
     if (bytes > kMostBytes) return ClusterShape{};
+    const int64_t row = std::max(max_pages, (limit + 1) / 2);   // pages that warps and stages are chosen for
+    auto most_grown = [&](int64_t n) -> int64_t {
+        if (gqa) {
+            if (n == 64 || (n == 32 && D == 64 && units >= 38)) return limit;
+            return n == 32 ? 16 : n == 16 ? 32 : n == 8 ? 9 : 8;
+        }
+        if (units * n > 900 && (batch == 1 || n == 32)) return batch == 1 ? limit : D == 128 ? 8 : 18;
+        return D == 128 ? (n == 16 ? 6 : 4) : n == 64 ? 9 : n == 16 ? 7 : 5;
+    };
     for (const auto& cw : kWarpsOf) {
         ClusterShape sh;
         sh.ctas = cw[0];
         sh.warps = cw[1];
         const int64_t n = (int64_t)sh.ctas * sh.warps;
-        if (n > 4 && (n / 2 >= max_pages || (n == 64 && max_pages <= 128))) continue;
-        const int64_t per_warp = (max_pages + n - 1) / n;
-        const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, per_warp));
+        if (n > 4 && (n / 2 >= row || (n == 64 && row <= 128))) continue;
+        const int ring = (int)std::min<int64_t>(kClusterRingBytes / stage, std::max<int64_t>(1, (row + n - 1) / n));
         for (sh.ring = ring; sh.ring >= std::min(ring, 2); --sh.ring) {
             if (10 * (int64_t)resident(device, D, gqa, sh) < 11 * units) continue;
-            if (per_warp > most_pages_per_warp(D, gqa, units, n, bytes)) return ClusterShape{};
+            const int64_t most = most_pages_per_warp(D, gqa, units, n, bytes);
+            if ((max_pages + n - 1) / n > most) return ClusterShape{};
+            if (limit > max_pages && (limit + n - 1) / n > std::max(most, most_grown(n))) return ClusterShape{};
             for (ClusterShape more = sh; spread && ++more.ring <= kClusterRingBytes / stage;) {
                 if (resident(device, D, gqa, more) < units) break;
                 sh = more;

@@ -45,7 +45,7 @@ def test_cluster_shapes_match_the_oracle(kvlib, Hq, Hkv, d, lens, fused):
     t.close()
 
 
-@pytest.mark.parametrize("Hq,Hkv,d", [(4, 4, 128), (14, 2, 64)])
+@pytest.mark.parametrize("Hq,Hkv,d", [(4, 4, 128), (14, 2, 64), (14, 2, 128)])   # a plan, and clusters of 64 warps
 def test_rows_that_outgrow_the_shape_and_a_failed_row(kvlib, Hq, Hkv, d):
     """Device steps pick their clusters from the rows held when they are
     enabled (a page each); then a row grows to 9000 tokens, far past the

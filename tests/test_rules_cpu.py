@@ -40,10 +40,10 @@ class Rules:
                 for r, n in enumerate(counts):
                     lib.set_resident(d, c, w, r + 1, n)
 
-    def shape(self, hq, hkv, d, pages, spread=False):
+    def shape(self, hq, hkv, d, pages, spread=False, limit=0):
         """(CTAs, warps, stages) of a step over rows of these page counts; no CTAs: a split plan."""
         out = (ctypes.c_int * 3)()
-        self.lib.shape(d, int(hq > hkv), hkv, len(pages), sum(pages), max(pages), int(spread), out)
+        self.lib.shape(d, int(hq > hkv), hkv, len(pages), sum(pages), max(pages), int(spread), limit, out)
         return tuple(out)
 
 
@@ -59,9 +59,10 @@ def rules(tmp_path_factory):
         static int known[2][9][9][8];
         static int resident(int, int D, bool, const ClusterShape& s) { return known[D == 128][s.ctas][s.warps][s.ring]; }
         extern "C" void set_resident(int D, int c, int w, int r, int n) { known[D == 128][c][w][r] = n; }
-        extern "C" void shape(int D, int gqa, int hkv, int rows, int pages, int max_pages, int spread, int* out)
+        extern "C" void shape(int D, int gqa, int hkv, int rows, int pages, int max_pages, int spread, int limit,
+                              int* out)
         {
-            const ClusterShape s = pick_cluster_shape(resident, 0, D, gqa, hkv, rows, pages, max_pages, spread);
+            const ClusterShape s = pick_cluster_shape(resident, 0, D, gqa, hkv, rows, pages, max_pages, spread, limit);
             out[0] = s.ctas;
             out[1] = s.warps;
             out[2] = s.ring;
@@ -194,6 +195,31 @@ def test_rows_that_start_short_fill_the_gpu_when_grown(rules, Hq, Hkv, d, B):
         T = rules.item_pages(Hq, Hkv, d, [held] * B, True)
         items = min(-(-60 // T), rules.lib.cap(int(Hq > Hkv), B * Hkv, WARPS, 256, T)) * B * Hkv
         assert items >= min(WARPS, 30 * B * Hkv, 16 * B * Hkv if Hq > Hkv else WARPS)
+@pytest.mark.parametrize("Hq,Hkv,d,B", [(32, 32, 128, 1), (28, 4, 128, 1), (28, 4, 128, 4), (28, 4, 128, 8), (40, 40, 128, 1),
+                                        (8, 8, 64, 4), (14, 2, 64, 8), (32, 32, 128, 3), (8, 8, 128, 4), (6, 2, 64, 60)])
+@pytest.mark.parametrize("limit", [20, 64, 200, 256, 512, 2048, 8192])
+def test_a_shape_that_stays_serves_grown_rows(rules, Hq, Hkv, d, B, limit):
+    """Device steps keep the clusters they started with (a captured graph
+    does), so those picked for a page a row have the warps, and the stages,
+    that rows of `limit` pages need; else the step runs from a plan."""
+    for held in (1, 4, 10):
+        c, w, r = rules.shape(Hq, Hkv, d, [held] * B, limit=limit)
+        if c == 0:
+            continue
+        n = c * w
+        if limit > 2 * n:
+            assert r >= 2
+        items = 64 if B * Hkv * 32 < WARPS else 16 if Hq > Hkv else 32   # of the plan, for one long row
+        assert -(-limit // n) <= max(18, -(-limit // items)) or (B == 1 and Hkv * n > 900)
+    assert rules.shape(Hq, Hkv, d, [10] * B, limit=11) == rules.shape(Hq, Hkv, d, [10] * B)
+
+
+def test_clusters_of_long_tables(rules):
+    assert rules.shape(32, 32, 128, [4], limit=256) == (8, 4, 3)     # one request in a 4096-token context
+    assert rules.shape(28, 4, 128, [4] * 2, limit=2048) == (8, 8, 3)
+    assert rules.shape(28, 4, 128, [4] * 8, limit=512) == (8, 4, 3)
+    assert rules.shape(28, 4, 128, [4] * 8, limit=2048) == (0, 0, 0)
+    assert rules.shape(32, 32, 128, [4] * 3, limit=256) == (0, 0, 0)
 
 
 def test_few_units_get_the_items_that_their_rows_ask_for(rules):
