@@ -349,6 +349,9 @@ struct OncePerDevice {
     }
 };
 
+int32_t noalloc_chunk_cap(bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages, int64_t max_pages,
+                          int32_t T);
+
 // Message returned by kv_last_error() on the calling thread.
 void set_last_error(const char* msg);
 

@@ -271,7 +271,7 @@ extern "C" KVC_API int decode_attention_noalloc(const void* k_pool, const void* 
     };
     const int64_t T_step = auto_item_pages(head_dim, G > 1, num_kv_heads, warps, batch, total_pages, max_np, false);
     auto cut_as_step = [&](int64_t size) {
-        return cut(size, chunk_cap(G > 1, (int64_t)batch * num_kv_heads, warps, max_np, (int32_t)size), true);
+        return cut(size, noalloc_chunk_cap(G > 1, num_kv_heads, warps, batch, total_pages, max_np, (int32_t)size), true);
     };
     if (!cut_as_step(T_step) && !cut_as_step(std::max(T, T_step)) && !cut(T, kChunkCap, false))
         return fail(KVC_ERR_UNSUPPORTED, "the batch does not fit the static scratch");

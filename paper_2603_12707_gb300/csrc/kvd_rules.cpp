@@ -57,6 +57,18 @@ int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int
     return gqa ? kChunkCapGqa : kChunkCap;
 }
 
+// The allocation-free call's: with a row of more than 32 shares (pages per
+// warp) 32 items for GQA too, as that row decides (us a call, 16 and 32; 28/4
+// heads, 12 rows of 5400 tokens and one of 21500 52 and 36; 16/8, 6 of 3600 to
+// 28600 65 and 57; 14/2, 25 of 288 and one of 11500 24 and 15; the Qwen-shaped
+// batch, whose longest row has 27 shares, stays at 16).
+int32_t noalloc_chunk_cap(bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages, int64_t max_pages,
+                          int32_t T)
+{
+    const int32_t cap = chunk_cap(gqa, rows * num_kv_heads, warps, max_pages, T);
+    return max_pages * warps > 32 * pages * num_kv_heads ? std::max(cap, kChunkCap) : cap;
+}
+
 // Pages that a warp of the longest row may have in clusters of n warps for each
 // of `units` units, whose layer holds `bytes` of K and V: the time that takes
 // against the plan's merge pass and what the layer's bytes take in any case.

@@ -75,6 +75,10 @@ def rules(tmp_path_factory):
         {
             return whole_rows_beat_clusters(D, group, rows, pages, max_pages);
         }
+        extern "C" int noalloc_cap(int gqa, int hkv, int warps, int rows, int pages, int max_pages, int T)
+        {
+            return noalloc_chunk_cap(gqa, hkv, warps, rows, pages, max_pages, T);
+        }
         extern "C" int early(int ctas, int slots) { return place_first_layer_early(ctas, slots); }
         extern "C" int cap(int gqa, int units, int warps, int max_pages, int T)
         {
@@ -231,6 +235,18 @@ def test_few_units_get_the_items_that_their_rows_ask_for(rules):
                 for pages in (1, 16 * T, 16 * T + 1, 31 * T, 32 * T, 33 * T, 64 * T):
                     assert rules.lib.cap(gqa, units, WARPS, pages, T) >= min(64, -(-pages // T))
     assert rules.lib.cap(1, 38, WARPS, 2000, 2) == 16 and rules.lib.cap(0, 38, WARPS, 2000, 2) == 32
+
+
+@pytest.mark.parametrize("Hq,Hkv,pages,cap", [
+    (28, 4, [1347] + [337] * 12, 32),
+    (16, 8, [1786, 1500, 900, 600, 400, 228], 32),
+    (14, 2, [721] + [18] * 25, 32),
+    (28, 4, [288, 270, 260, 160, 150, 140] + [60] * 26, 16),
+    (28, 4, [300] * 20, 16),
+    (8, 8, [721] + [18] * 70, 32),
+])
+def test_the_allocation_free_call_cuts_a_long_row_into_32(rules, Hq, Hkv, pages, cap):
+    assert rules.lib.noalloc_cap(int(Hq > Hkv), Hkv, WARPS, len(pages), sum(pages), max(pages), 8) == cap
 
 
 def test_setup_runs_once_on_each_device(tmp_path):
