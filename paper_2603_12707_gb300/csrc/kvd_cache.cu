@@ -61,8 +61,8 @@ __device__ int block_exclusive_scan(int v, int* total)
 //
 // CTA 0 orders and counts; all CTAs then write entries and page lists, the
 // rows spread over their warps, reading what CTA 0 found from its shared
-// memory.  Step kernel, one CTA against this: 32 rows of up to 288 pages 10.4
-// and 8.6 us, 96 rows of up to 512 18.5 and 12.3, 194 short rows 16.6 and 10.4.
+// memory.  Device step, one CTA of 1024 threads and eight: 32 rows of 288 pages
+// 10.3 and 5.8 us, 96 of 128 15.7 and 7.8, 188 of one page 12.0 and 8.2.
 template <class RowAt>
 __device__ int build_split_plan(int batch, int item_pages, int chunk_cap, int max_entries, RowAt row_at,
                                 PlanEntry* plan, int2* rows, const int32_t* page_table, int max_pages,
@@ -211,8 +211,7 @@ __global__ void __launch_bounds__(1024) step_device_kernel(const StepDevArgs a)
     const bool small = a.batch <= (int)blockDim.x;
     const bool lead = cluster_ctarank() == 0;   // the other CTAs only help to write the plan
     // The stack's top pages, one per thread, load along with the rows' lengths
-    // (with the threads above and the early arrival in build_split_plan, the
-    // steps named there take 5.2 / 5.8 / 6.4 / 6.5 us; 6.9 / 7.8 / 7.7 / 7.8 before).
+    // (with the early arrival in build_split_plan 1 us of a step of 96 rows).
     const int top0 = lead ? *a.free_top : 0;
     if (lead && threadIdx.x < top0) s_free[threadIdx.x] = a.free_pages[top0 - 1 - threadIdx.x];
     int carry = 0;
@@ -614,9 +613,8 @@ cudaError_t launch_seq_op(const SeqOpArgs& a, bool pdl, cudaStream_t st)
 
 cudaError_t launch_step_device(const StepDevArgs& a, cudaStream_t st)
 {
-    const int64_t ids = a.no_plan ? 0 : (int64_t)a.batch * a.max_pages;
-    const int ctas = step_ctas(ids);
-    return launch_cluster_of(ctas, step_threads(a.batch, ids, ctas), step_device_kernel, st, a);
+    const int64_t ids = a.no_plan ? 0 : a.pages;
+    return launch_cluster_of(step_ctas(a.batch, ids), step_threads(a.batch, ids), step_device_kernel, st, a);
 }
 
 cudaError_t launch_scatter_i32(int32_t* base, const int32_t* idx, const int32_t* val, int n, bool pdl, cudaStream_t st)
@@ -628,9 +626,8 @@ cudaError_t launch_scatter_i32(int32_t* base, const int32_t* idx, const int32_t*
 
 cudaError_t launch_step(const StepPatch& patch, const PlanArgs& plan, cudaStream_t st)
 {
-    const int64_t ids = plan.build && !plan.no_plan ? (int64_t)plan.batch * plan.max_pages : 0;
-    const int ctas = step_ctas(ids);
-    return launch_cluster_of(ctas, step_threads(plan.batch, ids, ctas), step_kernel, st, patch, plan);
+    const int64_t ids = plan.build && !plan.no_plan ? plan.pages : 0;
+    return launch_cluster_of(step_ctas(plan.batch, ids), step_threads(plan.batch, ids), step_kernel, st, patch, plan);
 }
 
 cudaError_t launch_token_copy(const TokenCopyArgs& a, bool pdl, cudaStream_t st)

@@ -857,6 +857,7 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         pa.plan = c->plan;
         pa.rows = c->rows;
         pa.chunk_cap = cap;
+        pa.pages = total_units / c->cfg.num_kv_heads;
         pa.page_ids = c->item_pages;
         pa.page_stride = stride;
         pa.err = c->err;
@@ -1130,6 +1131,7 @@ int kv_begin_step_device(kv_cache* c, int32_t batch, const int32_t* seq_ids, voi
     a.rows = c->rows;
     a.n_entries = c->d_small + 1;
     a.chunk_cap = c->dev_chunk_cap;
+    a.pages = std::min<int64_t>((int64_t)batch * c->cfg.max_pages_per_seq, c->cfg.num_pages);
     a.page_ids = c->item_pages;
     a.page_stride = c->dev_stride;
     a.err = c->err;

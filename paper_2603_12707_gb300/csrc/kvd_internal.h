@@ -112,6 +112,7 @@ struct PlanArgs {
     PlanEntry* plan;     // [n_entries]
     int2* rows;          // [batch]: (first partial slot, items) of each batch row
     int32_t chunk_cap;   // items per row at most (kChunkCap or kMaxChunks)
+    int64_t pages;       // of all rows: what the launch is sized for
     int32_t* page_ids;   // [entries][page_stride]: page ids of each entry's pages
     int32_t page_stride;
     int32_t* err;
@@ -136,6 +137,7 @@ struct StepDevArgs {
     int2* rows;
     int32_t* n_entries;       // out: plan entries of the step
     int32_t chunk_cap;        // items per row at most (kChunkCap or kMaxChunks)
+    int64_t pages;            // that the rows may hold in all: what the launch is sized for
     int32_t* page_ids;        // [max_entries][page_stride]: page ids of each entry's pages
     int32_t page_stride;
     int32_t* err;
@@ -414,9 +416,10 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
 bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int64_t max_pages);
 // Whether the split pass of a step's first layer is launched early (see kvd_rules.cpp).
 bool place_first_layer_early(int64_t ctas, int64_t slots);
-// CTAs of a step kernel that builds a plan over at most `ids` page ids, and its threads per CTA.
-int step_ctas(int64_t ids);
-int step_threads(int64_t batch, int64_t ids, int ctas);
+// CTAs, and threads per CTA, of a step kernel over `rows` rows that builds a
+// plan of `ids` page ids (0: no plan).
+int step_ctas(int64_t rows, int64_t ids);
+int step_threads(int64_t rows, int64_t ids);
 // The split pass over rows given as parameters (no append; placed early, it
 // reads nothing before its dependency wait): p.rows is written for the merge
 // pass, p.item_pages is not used.

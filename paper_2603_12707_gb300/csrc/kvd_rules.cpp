@@ -195,22 +195,25 @@ bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int
 // 512 slots 14.5 and 14.1; at d = 64 9.8 and 9.4; from 1216 on the same).
 bool place_first_layer_early(int64_t ctas, int64_t slots) { return 2 * ctas >= slots; }
 
-// CTAs of a step kernel that builds a plan over at most `ids` page ids: one
-// where its warps hold them in a round or two (12 rows of up to 85 pages: the
-// step is 2 us shorter than with 4 or 8, which the cluster's start costs),
-// else 8 (8 rows of 2049: 9.5 us, 10.3 with 4, 14.2 with 1).
-int step_ctas(int64_t ids) { return ids <= 2048 ? 1 : 8; }
+// A step kernel that builds a plan is a cluster of 8 CTAs, but for a few short
+// rows, which one CTA handles before the cluster has met.  Each warp takes a
+// row at a time, or 128 page ids of one, so 8 warps a CTA, 16 for more than 64
+// rows, and a thread per row where a block can have one (the rows' order
+// depends on that).  us a step, one CTA of 256 / 512 / 1024 threads and 8 of 256 /
+// 512 / 1024: 1 row of 50 pages 3.9 4.1 4.7 and 4.7 5.1 6.0; 16 of 4 4.8 4.4 5.2
+// and 4.9 5.2 6.4; 12 of 85 5.7 5.1 5.4 and 4.8 5.2 6.4; 64 of 8 9.7 7.3 6.8 and
+// 5.2 5.7 7.1; 188 of 1 22.0 14.8 12.0 and 8.5 8.2 8.3; 96 of 128 24.4 17.2 15.7
+// and 8.6 7.8 8.1; 8 of 2049 16.9 11.9 10.6 and 6.3 6.1 7.0; 500 of 4 - 37.0 29.0
+// and - 16.1 15.8.  Without a plan (no ids) one CTA, 256 / 512 / 1024 threads: 1.7
+// 1.7 1.9.
+int step_ctas(int64_t rows, int64_t ids) { return ids == 0 || (rows <= 16 && ids <= 1024) ? 1 : 8; }
 
-// Threads per CTA of a step kernel: enough warps to copy the page ids in one
-// go (a warp has 128 in flight), 8 to 16 of them, and a thread per row where a
-// block can have one (the rows' order depends on that).  Device step of 32 /
-// 64 / 8 / 96 rows of up to 2.4k / 0.9k / 33k / 2k tokens with 256, 512 and 1024
-// threads: 5.7 5.9 6.9 / 5.5 5.8 6.9 / 6.9 6.5 7.3 / 7.5 7.0 7.7 us; without a
-// plan 1.65, 1.67 and 1.9.
-int step_threads(int64_t batch, int64_t ids, int ctas)
+int step_threads(int64_t rows, int64_t ids)
 {
-    if (batch > 512) return 1024;
-    return batch > 256 || ids > (int64_t)ctas * 1024 ? 512 : 256;
+    if (rows > 512) return 1024;
+    if (rows > 256) return 512;
+    if (ids == 0) return 256;
+    return rows > (step_ctas(rows, ids) == 1 ? 8 : 64) ? 512 : 256;
 }
 
 }  // namespace kvd

@@ -79,6 +79,11 @@ def rules(tmp_path_factory):
         {
             return noalloc_chunk_cap(gqa, hkv, warps, rows, pages, max_pages, T);
         }
+        extern "C" int step_launch(int rows, int64_t ids, int* threads)
+        {
+            *threads = step_threads(rows, ids);
+            return step_ctas(rows, ids);
+        }
         extern "C" int early(int ctas, int slots) { return place_first_layer_early(ctas, slots); }
         extern "C" int cap(int gqa, int units, int warps, int max_pages, int T)
         {
@@ -247,6 +252,25 @@ def test_few_units_get_the_items_that_their_rows_ask_for(rules):
 ])
 def test_the_allocation_free_call_cuts_a_long_row_into_32(rules, Hq, Hkv, pages, cap):
     assert rules.lib.noalloc_cap(int(Hq > Hkv), Hkv, WARPS, len(pages), sum(pages), max(pages), 8) == cap
+
+
+def test_step_kernels_have_warps_for_their_rows(rules):
+    """Many short rows need warps as many long ones do; a row needs a thread of
+    its own unless the block has 1024."""
+    def launch(rows, ids):
+        t = ctypes.c_int()
+        return rules.lib.step_launch(rows, ctypes.c_int64(ids), ctypes.byref(t)), t.value
+
+    for rows in (1, 8, 9, 16, 17, 64, 65, 141, 188, 256, 257, 512, 513, 1024, 3000):
+        for per_row in (0, 1, 3, 60, 2049):
+            c, t = launch(rows, rows * per_row)
+            assert t in (256, 512, 1024) and c in (1, 8) and (t >= rows or t == 1024)
+            if per_row == 0:
+                assert c == 1
+            else:
+                assert c * t // 32 >= min(rows, 128) // 2
+    assert launch(12, 12 * 128) == launch(12, 12 * 2048)
+    assert launch(188, 188)[0] == 8
 
 
 def test_setup_runs_once_on_each_device(tmp_path):
