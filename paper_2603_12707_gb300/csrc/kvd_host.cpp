@@ -816,7 +816,8 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
     };
     size_plan();
     if (shape.ctas && !split &&
-        whole_rows_beat_clusters(c->cfg.head_dim, c->group, batch, total_units / c->cfg.num_kv_heads, max_np))
+        whole_rows_beat_clusters(c->cfg.head_dim, c->group, c->cfg.num_kv_heads, batch,
+                                 total_units / c->cfg.num_kv_heads, max_np))
         shape = ClusterShape{};
     // While device steps are enabled the buffers stay: an automatic plan that
     // does not fit is cut as device steps cut it, which always does.

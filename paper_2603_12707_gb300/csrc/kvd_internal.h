@@ -413,7 +413,7 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
                                 int64_t batch, int64_t pages, int64_t max_pages, bool spread = false,
                                 int64_t limit = 0);
 // Whether a plan that leaves every row whole is the better one where clusters would do.
-bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int64_t max_pages);
+bool whole_rows_beat_clusters(int D, int group, int num_kv_heads, int64_t rows, int64_t pages, int64_t max_pages);
 // Whether the split pass of a step's first layer is launched early (see kvd_rules.cpp).
 bool place_first_layer_early(int64_t ctas, int64_t slots);
 // CTAs, and threads per CTA, of a step kernel over `rows` rows that builds a

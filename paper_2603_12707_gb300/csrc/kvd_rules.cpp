@@ -57,8 +57,8 @@ int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int
     return gqa ? kChunkCapGqa : kChunkCap;
 }
 
-// The allocation-free call's: with a row of more than 32 shares (pages per
-// warp) 32 items for GQA too, as that row decides (us a call, 16 and 32; 28/4
+// The allocation-free call's: with a row of more than 256 pages and 32 shares
+// (pages per warp) 32 items for GQA too, as that row decides (us a call, 16 and 32; 28/4
 // heads, 12 rows of 5400 tokens and one of 21500 52 and 36; 16/8, 6 of 3600 to
 // 28600 65 and 57; 14/2, 25 of 288 and one of 11500 24 and 15; the Qwen-shaped
 // batch, whose longest row has 27 shares, stays at 16).
@@ -66,7 +66,7 @@ int32_t noalloc_chunk_cap(bool gqa, int num_kv_heads, int64_t warps, int64_t row
                           int32_t T)
 {
     const int32_t cap = chunk_cap(gqa, rows * num_kv_heads, warps, max_pages, T);
-    return max_pages * warps > 32 * pages * num_kv_heads ? std::max(cap, kChunkCap) : cap;
+    return max_pages > 256 && max_pages * warps > 32 * pages * num_kv_heads ? std::max(cap, kChunkCap) : cap;
 }
 
 // Pages that a warp of the longest row may have in clusters of n warps for each
@@ -87,7 +87,7 @@ int64_t most_pages_per_warp(int D, bool gqa, int64_t units, int64_t n, int64_t b
     if (gqa) return (20000000 + std::min<int64_t>(bytes, 25000000)) / (D == 128 ? 4000000 : 2800000);
     if (D == 128)
         return std::min<int64_t>(n < 64 && units * n < 600 ? 5 : 7, std::max<int64_t>(4, (17000000 + bytes) / 6000000));
-    return n == 64 ? 7 : (22500000 + bytes) / 4500000;
+    return n == 64 ? 7 : (24000000 + bytes) / 4500000;
 }
 
 // The line between the two, measured as us per layer of graph-replayed steps
@@ -180,9 +180,11 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
 // whole rows; 56/8 heads, 6 rows of up to 12 tokens 3.2 and 2.5; 28/4 heads, 51
 // of 8 4.1 and 2.7; 32 heads, 3 of 8 2.5 and 2.4; 14/2 heads, 60 of up to 2
 // pages 3.8 and 2.7; 16/8 heads, 43 of which one has 2 3.0 and 2.6; but 40/40
-// heads, one of 2 2.6 and 2.9, 14/2 heads at d = 64, 76 of up to 2 2.5 and 2.8).
-bool whole_rows_beat_clusters(int D, int group, int64_t rows, int64_t pages, int64_t max_pages)
+// heads, one of 2 2.6 and 2.9; d = 64, 14/2 heads, 76 of up to 2 2.5 and 2.8, up
+// to 100 units of one page 2.1-2.4 and 2.2-2.7).
+bool whole_rows_beat_clusters(int D, int group, int num_kv_heads, int64_t rows, int64_t pages, int64_t max_pages)
 {
+    if (D == 64 && rows * num_kv_heads <= 100) return false;
     return max_pages == 1 || (max_pages == 2 && ((group > 4 && D == 128) || 4 * pages <= 5 * rows));
 }
 

@@ -71,9 +71,9 @@ def rules(tmp_path_factory):
         {
             return auto_item_pages(D, gqa, hkv, warps, rows, pages, max_pages, growing);
         }
-        extern "C" int whole(int D, int group, int rows, int pages, int max_pages)
+        extern "C" int whole(int D, int group, int hkv, int rows, int pages, int max_pages)
         {
-            return whole_rows_beat_clusters(D, group, rows, pages, max_pages);
+            return whole_rows_beat_clusters(D, group, hkv, rows, pages, max_pages);
         }
         extern "C" int noalloc_cap(int gqa, int hkv, int warps, int rows, int pages, int max_pages, int T)
         {
@@ -157,18 +157,19 @@ def test_short_unequal_rows_stay_whole_only_where_it_pays(rules, Hq, Hkv, d, pag
     assert tuple(rules.item_pages(Hq, Hkv, d, pages, growing) >= max(pages) for growing in (False, True)) == whole
 
 
-@pytest.mark.parametrize("d,group,pages,whole", [
-    (128, 7, [1] * 51, True),
-    (128, 1, [1], True),
-    (64, 7, [1, 1], True),
-    (128, 7, [2, 1, 2], True),
-    (128, 2, [2] + [1] * 42, True),
-    (128, 1, [2], False),
-    (64, 7, [2, 1] * 38, False),
-    (128, 7, [3] + [1] * 60, False),
+@pytest.mark.parametrize("d,group,hkv,pages,whole", [
+    (128, 7, 4, [1] * 51, True),
+    (128, 1, 32, [1], True),
+    (64, 7, 2, [1, 1], False),
+    (64, 7, 2, [1] * 111, True),
+    (128, 7, 4, [2, 1, 2], True),
+    (128, 2, 8, [2] + [1] * 42, True),
+    (128, 1, 40, [2], False),
+    (64, 7, 2, [2, 1] * 38, False),
+    (128, 7, 2, [3] + [1] * 60, False),
 ])
-def test_rows_of_one_or_two_pages_stay_whole(rules, d, group, pages, whole):
-    assert bool(rules.lib.whole(d, group, len(pages), sum(pages), max(pages))) == whole
+def test_rows_of_one_or_two_pages_stay_whole(rules, d, group, hkv, pages, whole):
+    assert bool(rules.lib.whole(d, group, hkv, len(pages), sum(pages), max(pages))) == whole
 
 
 @pytest.mark.parametrize("Hq,Hkv,d,lens,clusters", [
