@@ -387,7 +387,7 @@ cudaError_t decode_variant_info(int D, bool gqa, DecodeVariant* v);
 // (it lets the next kernel start at once and waits for the split pass).
 // max_chunks: an upper bound on the items of any row of the step (<= kMaxChunks).
 // split_regs_per_subpartition: registers the resident split pass holds on
-// each of an SM's four schedulers (0: nothing resident beside it).
+// each of an SM's four schedulers.
 cudaError_t launch_merge(int D, bool pdl, int max_chunks, int num_sms, int split_regs_per_subpartition,
                          const DecodeParams& p, cudaStream_t st);
 // fused: the append + attention kernel.  pdl: launched with programmatic
