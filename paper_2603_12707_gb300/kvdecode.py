@@ -107,10 +107,10 @@ def load():
 def _ptr(x):
     if x is None:
         return None
-    if isinstance(x, array.array):
-        return x.buffer_info()[0]
     if hasattr(x, "data_ptr"):
         return x.data_ptr()
+    if isinstance(x, array.array):
+        return x.buffer_info()[0]
     if isinstance(x, ctypes.Array):
         return ctypes.addressof(x)
     return int(x)
