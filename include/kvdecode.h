@@ -129,8 +129,9 @@ KVC_API int kv_cache_pool(kv_cache *cache, int32_t layer, void **k_pool, void **
 /* Override the target split size (pages per work item of decode_attention)
  * used by later kv_begin_step calls; 0 restores the automatic choice.
  * Range 0 .. 1024.  A row of n pages is cut into ceil(n / T') items of
- * near-equal size, T' = max(T, ceil(n / 32)): never more than 32 items per
- * (sequence, KV head).  With an override every step runs from a split plan;
+ * near-equal size, T' = max(T, ceil(n / cap)), where the shorter rows of a
+ * batch take fractions of T and cap is 32, 16 with several query heads per KV
+ * head, up to 64 where few rows have to fill the GPU.  With an override every step runs from a split plan;
  * the automatic choice runs small steps without one (decode_attention). */
 KVC_API int kv_cache_set_split_pages(kv_cache *cache, int32_t pages);
 
@@ -239,9 +240,10 @@ KVC_API int kv_append(kv_cache *cache, int32_t layer, int32_t batch, const void 
  * merges the partial results of every (sequence, KV head) cut into several
  * items by log-sum-exp.  A step with little to read (up to about 45 MB of K
  * and V per layer; kv_begin_step decides by the step's lengths,
- * kv_begin_step_device by those held when device steps were enabled) has no
- * plan: one thread-block cluster per (sequence, KV head) does both in one
- * launch. */
+ * kv_begin_step_device, whose graphs outlive them, by those held when device
+ * steps were enabled and by how long max_pages_per_seq and the pool let a
+ * sequence become) has no plan: one thread-block cluster per (sequence, KV
+ * head) does both in one launch. */
 KVC_API int decode_attention(kv_cache *cache, int32_t layer, int32_t batch, const void *q, void *out,
                      float softmax_scale, void *stream);
 
@@ -255,14 +257,19 @@ KVC_API int decode_attention(kv_cache *cache, int32_t layer, int32_t batch, cons
  * kv_append, the kernel is launched with programmatic dependent launch: it
  * may start, and stream this layer's cached pages (positions < s_b), while
  * that launch is finishing; it reads q, k_new and v_new and writes anything
- * only after the kernel before it has completed.  After any other call of
- * this library it is an ordinary launch.  The same holds for decode_attention
- * (which, where a launch chained before it appended tokens, reads each row's
- * last page only once that has completed) and for kv_append (which reads and
- * writes nothing before the kernel before it has).  So a kernel the caller
- * enqueues between two layers must not write the cache's pages (a foreign
- * kernel could only race with the early reads if it signalled its dependents
- * early). */
+ * only after the kernel before it has completed.  The same holds for
+ * decode_attention (which, where a launch chained before it appended tokens,
+ * reads each row's last page only once that has completed).  So a kernel the
+ * caller enqueues between two layers must not write the cache's pages (a
+ * foreign kernel could only race with the early reads if it signalled its
+ * dependents early).
+ * These are the only launches that read anything early.  Others carry the
+ * launch attribute too, are placed while what precedes them on the stream
+ * finishes, and read and write nothing before that has completed: the
+ * attention launch right after kv_begin_step or kv_begin_step_device, the
+ * step kernels of those two, kv_append after an attention launch,
+ * kv_seq_reserve, kv_seq_free, kv_write_tokens, kv_read_tokens and
+ * kv_write_varlen after one another, and decode_attention_noalloc. */
 KVC_API int decode_attention_append(kv_cache *cache, int32_t layer, int32_t batch, const void *q,
                                     const void *k_new, const void *v_new, void *out,
                                     float softmax_scale, void *stream);
@@ -277,7 +284,9 @@ KVC_API int decode_attention_append(kv_cache *cache, int32_t layer, int32_t batc
  * replayed every step with no host work (the role CUDA graphs play in the
  * paper's engine, Sec. 5.4).  Enabling reserves plan, page-list and partial
  * buffers for up to max_batch sequences at the longest page-table row, and
- * fixes the work-item size from the pages currently held.  While enabled,
+ * fixes the work-item size and the choice between clusters and a plan from
+ * the pages currently held (decode_attention), so a max_pages_per_seq far
+ * above what sequences reach costs small batches some speed.  While enabled,
  * admitting and closing sequences needs no host synchronisation:
  * kv_seq_create is host bookkeeping, kv_seq_reserve and kv_seq_free are
  * kernels on their stream, and kv_write_tokens, kv_write_varlen and
@@ -291,8 +300,8 @@ KVC_API int decode_attention_append(kv_cache *cache, int32_t layer, int32_t batc
  * state back on a stream the cache owns.  Graphs captured while device
  * steps are enabled stay valid until they are disabled, enabled again (which
  * may resize the buffers) or the cache is destroyed: meanwhile a host-planned
- * step that would need larger buffers fails with KVC_ERR_INVALID instead of
- * moving them. */
+ * step of more than max_batch sequences, or with a set split size, that would
+ * need larger buffers fails with KVC_ERR_INVALID instead of moving them. */
 KVC_API int kv_cache_device_steps(kv_cache *cache, int32_t max_batch, int32_t enable, void *stream);
 
 /* kv_begin_step with everything on the device: seq_ids is DEVICE memory
@@ -331,10 +340,11 @@ KVC_API int kv_cache_sync(kv_cache *cache);
  *                   cleared by this call), or NULL to discard them
  * Work space is a 16 MiB array in this library's device code, held by every
  * GPU that loads the library until the process exits.  batch <= 1024.
- * Work items are enlarged (doubled, up to 1024 pages each) until the split
- * plan and partial results fit the 16 MiB (one item per row needs no
- * partials at all); KVC_ERR_UNSUPPORTED, with nothing enqueued, if they
- * still do not fit at 1024 pages.  The first call on
+ * Work items are enlarged (doubled, up to 1024 pages each) until a split plan
+ * with its page lists and the partial results would fit the 16 MiB (one item
+ * per row needs no partials at all); KVC_ERR_UNSUPPORTED, with nothing
+ * enqueued, if they still do not at 1024 pages.  (The call itself keeps only
+ * the partials there; the limit is that of the plan.)  The first call on
  * each device looks up the array's device address (cudaGetSymbolAddress);
  * make that first call before any stream capture.  Every call uses the same
  * array and leaves its work counter at zero, as it found it, so calls that
