@@ -282,48 +282,10 @@ CUresult encode_tile_map(void* encode_fn, CUtensorMap* map, void* k_pool, int64_
 // Target pages per work item of a step of `rows` rows that hold `pages` pages
 // per KV head in all and at most max_pages in one row; growing: the rows will
 // outgrow these numbers by some tokens (device steps fix the target once).
-//
-// Items end at about the same time on all warps if there are some of them per
-// warp: three for MHA, two for GQA, whose items leave a partial per query
-// head.  But an item costs about 0.6 pages beside its own, and a row of several
-// a merge, so where a warp's share is short (up to 30 pages of d = 128),
-//  - rows of nearly equal length are cut into one item per resident warp, or
-//    up to 1.3 for shares past 15 pages of 200 units or more (fewer, longer
-//    rows end on items too long for a second round: 32 heads, 16000 tokens
-//    45.1, at three items per warp 39.7; 3 rows of 3100 28.4 and 26.0) (us per layer, before -> now; 32 heads
-//    of 900 tokens, B 5 / 8 / 12: 17.0 -> 14.3, 22.8 -> 20.1, 30.4 -> 29.1;
-//    16/8 heads of 500, B 32: 14.9 -> 12.6; 14/2 heads at d = 64 of 1000, B
-//    128: 17.2 -> 15.2; 8/8 at d = 64 of 700, B 64: 22.1 -> 18.6);
-//  - unequal rows stay whole if none is much longer than a warp's share, or up
-//    to 8 pages and four shares.  A host's step then runs without a merge pass
-//    (rows of up to 5 pages always); a device step launches it in any case, and
-//    the line is at 2.3 shares (40/40 heads, a row of 101 tokens and 10 of
-//    10-24, whole 6.2, as items of 2 pages 4.7; 21 of up to 104 6.4 and 5.7;
-//    8/8 heads, 33 of up to 8 pages 6.9 and 4.7, device step 9.1 and 5.9; 99 of
-//    up to 6 8.1 and 7.0, device step 9.2 and 9.6) (56/8 heads, 106 rows of up to 105 tokens:
-//    13.0 -> 9.9; 32 heads, 57 rows of up to 263: 26.1 -> 23.1).
-// Longer shares gain nothing (32 heads of 900, B 24 / 32: best target within
-// 2 % of a third of the share), up to items so long that the last ones to end
-// leave the others idle: targets from 48 pages (d = 64: 65) for rows past 128
-// become a third of that, at least 40 and at most 128 (whole batches, ms; 32
-// heads, 96 rows of 128-8192 tokens, 128 -> 53: 13.82 -> 13.49, 40 13.50, 64
-// 13.50, 96 13.55; 256 such rows, a third of 424: 128 54.14 a step, 40 54.50; 78 rows of up to 4581 7.97 -> 7.75, 48 7.79, 64 7.88; 16/8
-// heads, 149 rows of up to 4606, 55 -> 40: 5.79 -> 5.60; 8/8 at d = 64, 37 rows
-// of up to 27861, 87 -> 40: 6.04 -> 5.97.  Not below: 56/8 heads, 117 rows of up
-// to 4592, 47 -> 40: 5.93 -> 5.97; d = 64, 202 rows, 51 -> 40: 8.05 -> 8.11; nor
-// for 161 rows of up to 68 pages, 60 -> 40: 4.22 -> 4.23).
 int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages, int64_t max_pages,
                         bool growing);
 
-// Items per row at most: twice the usual cap when units (rows x KV heads) x the
-// usual cap would leave resident warps without an item and some row (of up
-// to max_pages pages) is long enough to use more items of T pages, and 32 if
-// it uses more than 16 (14/2 heads, 17 rows of 6700 tokens, 26 items: 19.7 us
-// a layer, cut at 16 22.9; Qwen heads, 8 rows of 3000: 11.1 and 13.1).
-// Otherwise 32 for MHA and 16 for GQA: a GQA row of at most 16 items merges
-// in one round trip with the 16-item variant, the largest whose registers
-// fit beside the resident GQA split pass (Qwen shape: 0.742 at 32, 0.769 at
-// 16, 0.756 at 24, 0.686 at 12).
+// Items per row at most, for `units` rows x KV heads.
 int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T);
 
 // A setup that belongs to a device (a kernel's attributes do), done once on

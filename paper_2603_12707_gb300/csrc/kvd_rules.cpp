@@ -7,6 +7,39 @@
 
 namespace kvd {
 
+// Items end at about the same time on all warps if there are some of them per
+// warp: three for MHA, two for GQA, whose items leave a partial per query
+// head.  But an item costs about 0.6 pages beside its own, and a row of several
+// a merge, so where a warp's share is short (up to 30 pages of d = 128)
+//  - rows of nearly equal length are cut into one item per resident warp, or
+//    up to 1.3 for shares past 15 pages of 200 units or more;
+//  - unequal rows stay whole if none is much longer than a warp's share, or up
+//    to 8 pages and four shares.  A host's step then runs without a merge pass
+//    (rows of up to 5 pages always); a device step launches it in any case, and
+//    the line is at 2.3 shares.
+// Longer shares gain nothing (32 heads of 900, B 24 / 32: best target within
+// 2 % of a third of the share), up to items so long that the last ones to end
+// leave the others idle: targets from 48 pages (d = 64: 65) for rows past 128
+// become a third of that, at least 40 and at most 128.
+//
+// us per layer of host steps, three (GQA two) items per warp and the rule.
+// Equal rows: 32 heads of 900 tokens, B 5 / 8 / 12 16.6 and 13.2, 21.9 and 18.9,
+// 29.2 and 26.8; 16/8 heads of 500, B 32 13.8 and 11.8; 14/2 at d = 64 of 1000, B
+// 128 15.3 and 12.8; 8/8 at d = 64 of 700, B 64 21.5 and 17.0.  The 1.06 against
+// 1.0: 32 heads, 8 rows of 760 to 1000 19.8 and 18.3, nine other batches within
+// 2 % of each other up to 1.15; the 1.3 against 1.0 within 3 %, 2.0 up to 5 %
+// slower; fewer than 200 units: 32 heads, 16000 tokens 39.7 and 45.1, 3 rows of
+// 3100 26.0 and 28.4.  Whole rows: 56/8 heads, 106 of up to 105 tokens 12.5 and
+// 8.1; 32 heads, 57 of up to 248 23.3 and 20.2; 8/8 at d = 64, 256 of up to 300
+// (1.13 shares) 19.7 and 14.8; but 40/40 heads, a row of 101 tokens and 10 of
+// 10-24 4.7 and, whole, 6.2; 8/8 heads, 33 of up to 8 pages 4.7 and 6.9, device
+// steps 5.9 and 9.1.  At least 16, so that whole rows of 2 pages are not halved
+// where the last rows take fractions: 56/8 heads, 152 such rows 6.4 and 3.7.
+// Long items: 32 heads, 96 rows of up to 8192 tokens, 94 / 40 / 48 / 64 pages
+// 385 379 380 376, 128 / 42 691 680; 78 of up to 4581, 73 / 40 / 48 297 293 299;
+// 16/8 heads, 149 of up to 4606, 53 / 40 / 64 154 147 151; not below: 56/8 heads,
+// 117 of up to 4592, 37 / 40 108 107; 8/8 at d = 64, 37 of up to 27861, 52 / 40
+// 111 110.
 int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_t rows, int64_t pages,
                         int64_t max_pages, bool growing)
 {
@@ -48,6 +81,14 @@ int32_t auto_item_pages(int D, bool gqa, int num_kv_heads, int64_t warps, int64_
     return (int32_t)std::max(T, std::min<int64_t>(128, few));
 }
 
+// Twice the usual cap when units x the usual cap would leave resident warps
+// without an item and some row is long enough to use more items of T pages,
+// and 32 if it uses more than 16 (14/2 heads, 17 rows of 6700 tokens, 26 items
+// 19.8 us a layer, cut at 16 22.9; Qwen heads, 8 rows of 3000 11.1 and 13.2).
+// Otherwise 32 for MHA and 16 for GQA: a GQA row of at most 16 items merges
+// in one round trip with the 16-item variant, the largest whose registers
+// fit beside the resident GQA split pass (Qwen shape, of the copy rate: 0.742
+// at 32, 0.769 at 16, 0.756 at 24, 0.686 at 12).
 int32_t chunk_cap(bool gqa, int64_t units, int64_t warps, int64_t max_pages, int32_t T)
 {
     if (units * kChunkCap < warps) {
