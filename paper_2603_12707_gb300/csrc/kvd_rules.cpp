@@ -34,7 +34,7 @@ namespace kvd {
 // (1.13 shares) 19.7 and 14.8; but 40/40 heads, a row of 101 tokens and 10 of
 // 10-24 4.7 and, whole, 6.2; 8/8 heads, 33 of up to 8 pages 4.7 and 6.9, device
 // steps 5.9 and 9.1.  At least 16, so that whole rows of 2 pages are not halved
-// where the last rows take fractions: 56/8 heads, 152 such rows 6.4 and 3.7.
+// where the last rows take fractions (56/8 heads, 152 such rows 1.7 times as long).
 // Long items: 32 heads, 96 rows of up to 8192 tokens, 94 / 40 / 48 / 64 pages
 // 385 379 380 376, 128 / 42 691 680; 78 of up to 4581, 73 / 40 / 48 297 293 299;
 // 16/8 heads, 149 of up to 4606, 53 / 40 / 64 154 147 151; not below: 56/8 heads,
