@@ -229,11 +229,16 @@ struct MhaCompute {
 // ------------------------------------------------------------ GQA, bf16 MMA
 // S^T[16 tokens][8 heads] = K . q^T and O^T[D][8 heads] += V^T . P^T with
 // mma.m16n8k16; accumulator columns of a lane are heads 2*(lane&3) and +1.
-template <int D>
+//
+// kNarrowQ: up to how many heads q is read with 4-byte loads in the fragment
+// layout, which take an L1 wavefront per head and instruction; more heads are
+// read 16 bytes at a time and transposed.  In the split pass at d = 64 the
+// transpose costs more than its 8 instructions save (14/2 heads, us per layer,
+// 4 and 8 narrow heads: 3 rows of one page 2.4 and 2.2, 90 rows of up to 2250
+// tokens 13.1 and 12.9); in clusters it does not (13 rows of 300 2.9 and 3.0).
+template <int D, int kNarrowQ = 4>
 struct GqaCompute {
     static constexpr int KS = D / 16;
-    // The 4-byte loads take an L1 wavefront per head and instruction.
-    static constexpr int kNarrowQ = 4;
     int G;
     uint32_t qb[KS][2];
     float m0, m1, l0, l1;
@@ -538,7 +543,7 @@ __global__ void __launch_bounds__(kWarps * 32)
     uint32_t pending = 0;  // bit s: stage s has a load in flight that was not waited on
     bool ok = true;
 
-    using Comp = typename std::conditional<GQA, GqaCompute<D>, MhaCompute<D>>::type;
+    using Comp = typename std::conditional<GQA, GqaCompute<D, D == 64 ? 8 : 4>, MhaCompute<D>>::type;
     Comp comp;
     // Chained launches depend programmatically on the previous kernel: until
     // griddep_wait() only the plan, page table and cache pages (none of which

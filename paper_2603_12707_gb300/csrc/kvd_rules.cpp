@@ -221,11 +221,11 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
 // whole rows; 56/8 heads, 6 rows of up to 12 tokens 3.2 and 2.5; 28/4 heads, 51
 // of 8 4.1 and 2.7; 32 heads, 3 of 8 2.5 and 2.4; 14/2 heads, 60 of up to 2
 // pages 3.8 and 2.7; 16/8 heads, 43 of which one has 2 3.0 and 2.6; but 40/40
-// heads, one of 2 2.6 and 2.9; d = 64, 14/2 heads, 76 of up to 2 2.5 and 2.8, up
-// to 100 units of one page 2.1-2.4 and 2.2-2.7).
+// heads, one of 2 2.6 and 2.9; d = 64, 14/2 heads, 76 of up to 2 2.5 and 2.8, 6/2
+// and 8/8 heads, up to 100 units of one page 2.1-2.3 and 2.2-2.4).
 bool whole_rows_beat_clusters(int D, int group, int num_kv_heads, int64_t rows, int64_t pages, int64_t max_pages)
 {
-    if (D == 64 && rows * num_kv_heads <= 100) return false;
+    if (D == 64 && group <= 4 && rows * num_kv_heads <= 100) return false;
     return max_pages == 1 || (max_pages == 2 && ((group > 4 && D == 128) || 4 * pages <= 5 * rows));
 }
 

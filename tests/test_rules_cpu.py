@@ -160,7 +160,8 @@ def test_short_unequal_rows_stay_whole_only_where_it_pays(rules, Hq, Hkv, d, pag
 @pytest.mark.parametrize("d,group,hkv,pages,whole", [
     (128, 7, 4, [1] * 51, True),
     (128, 1, 32, [1], True),
-    (64, 7, 2, [1, 1], False),
+    (64, 7, 2, [1, 1], True),
+    (64, 3, 2, [1, 1], False),
     (64, 7, 2, [1] * 111, True),
     (128, 7, 4, [2, 1, 2], True),
     (128, 2, 8, [2] + [1] * 42, True),
