@@ -815,15 +815,27 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         split = max_chunks > 1;
     };
     size_plan();
+    // Clusters need no plan buffers: a plan takes their place only where its
+    // buffers are there or may grow now.
+    auto fits = [&] {
+        return entries * stride <= c->item_pages_cap && entries <= c->plan_cap &&
+               entries * c->cfg.num_kv_heads <= c->slot_cap;
+    };
+    auto may_grow = [&] {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        return !c->dev_mode &&
+               cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &capture) == cudaSuccess &&
+               capture == cudaStreamCaptureStatusNone;
+    };
     if (shape.ctas && !split &&
         whole_rows_beat_clusters(c->cfg.head_dim, c->group, c->cfg.num_kv_heads, batch,
-                                 total_units / c->cfg.num_kv_heads, max_np))
+                                 total_units / c->cfg.num_kv_heads, max_np) &&
+        (fits() || may_grow()))
         shape = ClusterShape{};
     // While device steps are enabled the buffers stay: an automatic plan that
     // does not fit is cut as device steps cut it, which always does.
     if (!shape.ctas && c->dev_mode && !c->split_override && !c->dev_split_override && batch <= c->dev_max_batch &&
-        (entries * stride > c->item_pages_cap || entries > c->plan_cap ||
-         entries * c->cfg.num_kv_heads > c->slot_cap)) {
+        !fits()) {
         T = c->dev_item_pages;
         cap = c->dev_chunk_cap;
         size_plan();

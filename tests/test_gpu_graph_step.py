@@ -256,6 +256,43 @@ def test_host_step_cannot_move_buffers_under_device_steps(kvlib):
     kd.kv_cache_destroy(h)
 
 
+@pytest.mark.parametrize("way", ["captured", "device steps of one row"])
+def test_one_page_rows_without_plan_buffers(kvlib, way):
+    """A host step of one-page rows runs as a plan of whole rows; where its
+    buffers are not there and may not be allocated (the cache's first step in a
+    stream capture, or more rows than device steps reserved) as clusters."""
+    B, H, d = 100, 2, 128
+    cfg = wl.custom("first", 1, H, H, d, B, lens=[1 + b % 15 for b in range(B)], seed=31)
+    t = Tracked(cfg, extra_tokens=4, keep_rows=[0, 1, B - 1])
+    h, s = t.sess.h, torch.cuda.Stream()
+    q, kn, vn = wl.step_inputs(cfg, 0, 0, "cuda")
+    out = torch.zeros_like(q)
+    torch.cuda.synchronize()
+
+    def step():
+        kd.kv_begin_step(h, t.sess.seq_ids, s)
+        kd.decode_attention_append(h, 0, B, q, kn, vn, out, 0.0, s)
+
+    if way == "captured":
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            step()
+        with torch.cuda.stream(s):
+            g.replay()
+    else:
+        kd.kv_cache_device_steps(h, 1, True, s)
+        step()
+    s.synchronize()
+    assert t.sess.query().device_error == 0
+    ks = [np.concatenate([u16(wl.kv_block(cfg, 0, b, 1 + b % 15, "k", "cuda")), u16(kn[b:b + 1])]) for b in (0, 1, B - 1)]
+    vs = [np.concatenate([u16(wl.kv_block(cfg, 0, b, 1 + b % 15, "v", "cuda")), u16(vn[b:b + 1])]) for b in (0, 1, B - 1)]
+    ref = oracle.decode_attention(u16(q)[[0, 1, B - 1]], [len(x) for x in ks], np.concatenate(ks), np.concatenate(vs))
+    vmax = np.array([np.abs(oracle.bf16_to_f64(x)).max() for x in vs])
+    assert_close(bf16_to_f64(out)[[0, 1, B - 1]], ref, vmax, gqa=False)
+    t.sess.lens += 1
+    t.close()
+
+
 @pytest.mark.parametrize("held,tokens,rows", [([100, 100, 100, 100], 1600, 16), ([], 1600, 17), ([16], 1350, 12),
                                                ([1800] * 3, 1900, 17)])
 def test_host_steps_fit_what_device_steps_reserved(kvlib, held, tokens, rows):
