@@ -120,6 +120,7 @@ struct kv_cache {
     float* part_o = nullptr;
     float2* part_ml = nullptr;
     int64_t slot_cap = 0;
+    std::vector<void*> kept;                    // plan buffers from or before stream captures, freed with the cache
     std::vector<CUtensorMap> tmaps;             // [L]: K and V of a layer
 
     // device-side steps (kv_begin_step_device): free stack on the device
@@ -211,6 +212,38 @@ int64_t resident_warps(const kv_cache* c)
     return (int64_t)std::max(1, c->num_sms) * std::max(1, c->variant.ctas_per_sm) * std::max(1, c->variant.warps);
 }
 
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone;
+}
+
+// A plan buffer of `bytes` in place of *buf.  In a stream capture it is
+// allocated at once: one that the graph allocates exists only from its first
+// replay on, and calls outside the graph use the same buffer.  The old one may
+// belong to work before the capture, and is kept until the cache is destroyed.
+int replace_buffer(kv_cache* c, void** buf, size_t bytes, cudaStream_t st)
+{
+    const bool capture = capturing(st);
+    const bool held = std::find(c->kept.begin(), c->kept.end(), *buf) != c->kept.end();
+    if (*buf && !held) {
+        if (capture) c->kept.push_back(*buf);
+        else KVD_CUDA(cudaFreeAsync(*buf, st));
+    }
+    *buf = nullptr;
+    if (!capture) {
+        KVD_CUDA(cudaMallocAsync(buf, bytes, st));
+        return KVC_OK;
+    }
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    KVD_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaMalloc(buf, bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    KVD_CUDA(e);
+    c->kept.push_back(*buf);
+    return KVC_OK;
+}
+
 int grow_scratch(kv_cache* c, int64_t entries, int64_t slots, int64_t page_ids, cudaStream_t st)
 {
     // While device steps are enabled, captured graphs may hold these buffers'
@@ -221,30 +254,22 @@ int grow_scratch(kv_cache* c, int64_t entries, int64_t slots, int64_t page_ids, 
                     "captured since may use them: disable device steps first");
     if (page_ids > c->item_pages_cap) {
         const int64_t cap = std::max<int64_t>(page_ids, c->item_pages_cap + c->item_pages_cap / 2);
-        if (c->item_pages) KVD_CUDA(cudaFreeAsync(c->item_pages, st));
-        c->item_pages = nullptr;
         c->item_pages_cap = 0;
-        KVD_CUDA(cudaMallocAsync((void**)&c->item_pages, (size_t)cap * sizeof(int32_t), st));
+        if (int rc = replace_buffer(c, (void**)&c->item_pages, (size_t)cap * sizeof(int32_t), st)) return rc;
         c->item_pages_cap = cap;
     }
     if (entries > c->plan_cap) {
         const int64_t cap = std::max<int64_t>(entries, c->plan_cap + c->plan_cap / 2);
-        if (c->plan) KVD_CUDA(cudaFreeAsync(c->plan, st));
-        c->plan = nullptr;
         c->plan_cap = 0;
-        KVD_CUDA(cudaMallocAsync((void**)&c->plan, (size_t)cap * sizeof(PlanEntry), st));
+        if (int rc = replace_buffer(c, (void**)&c->plan, (size_t)cap * sizeof(PlanEntry), st)) return rc;
         c->plan_cap = cap;
     }
     if (slots > c->slot_cap) {
         const int64_t cap = std::max<int64_t>(slots, c->slot_cap + c->slot_cap / 2);
-        if (c->part_o) KVD_CUDA(cudaFreeAsync(c->part_o, st));
-        if (c->part_ml) KVD_CUDA(cudaFreeAsync(c->part_ml, st));
-        c->part_o = nullptr;
-        c->part_ml = nullptr;
         c->slot_cap = 0;
         const size_t G = (size_t)c->group, D = (size_t)c->cfg.head_dim;
-        KVD_CUDA(cudaMallocAsync((void**)&c->part_o, (size_t)cap * G * D * sizeof(float), st));
-        KVD_CUDA(cudaMallocAsync((void**)&c->part_ml, (size_t)cap * G * sizeof(float2), st));
+        if (int rc = replace_buffer(c, (void**)&c->part_o, (size_t)cap * G * D * sizeof(float), st)) return rc;
+        if (int rc = replace_buffer(c, (void**)&c->part_ml, (size_t)cap * G * sizeof(float2), st)) return rc;
         c->slot_cap = cap;
     }
     return KVC_OK;
@@ -261,12 +286,11 @@ void release_device(kv_cache* c)
     cudaFree(c->start_flags);
     cudaFree(c->step_no);
     cudaFree(c->err);
-    cudaFree(c->plan);
-    cudaFree(c->item_pages);
     cudaFree(c->d_free);
     cudaFree(c->d_small);
-    cudaFree(c->part_o);
-    cudaFree(c->part_ml);
+    for (void* p : {(void*)c->plan, (void*)c->item_pages, (void*)c->part_o, (void*)c->part_ml})
+        if (std::find(c->kept.begin(), c->kept.end(), p) == c->kept.end()) cudaFree(p);
+    for (void* p : c->kept) cudaFree(p);
 }
 
 // Wait for the cache's stream (the stream of its latest call; the caller
@@ -821,12 +845,7 @@ int kv_begin_step(kv_cache* c, int32_t batch, const int32_t* seq_ids, void* stre
         return entries * stride <= c->item_pages_cap && entries <= c->plan_cap &&
                entries * c->cfg.num_kv_heads <= c->slot_cap;
     };
-    auto may_grow = [&] {
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        return !c->dev_mode &&
-               cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &capture) == cudaSuccess &&
-               capture == cudaStreamCaptureStatusNone;
-    };
+    auto may_grow = [&] { return !c->dev_mode && !capturing(static_cast<cudaStream_t>(stream)); };
     if (shape.ctas && !split &&
         whole_rows_beat_clusters(c->cfg.head_dim, c->group, c->cfg.num_kv_heads, batch,
                                  total_units / c->cfg.num_kv_heads, max_np) &&

@@ -256,6 +256,41 @@ def test_host_step_cannot_move_buffers_under_device_steps(kvlib):
     kd.kv_cache_destroy(h)
 
 
+@pytest.mark.parametrize("eager_first", [False, True])
+@pytest.mark.parametrize("replay", [False, True])
+def test_plan_buffers_that_a_capture_brings_are_there_outside_it(kvlib, eager_first, replay):
+    """A captured host step whose plan needs buffers the cache has not got (or
+    larger ones than an eager step brought): a step after it, with the graph
+    replayed or not, finds them."""
+    cfg = wl.custom("capbuf", 1, 8, 8, 128, 6, lens=[300 + 40 * b for b in range(6)], seed=37)
+    t = Tracked(cfg, extra_tokens=8, split_pages=8 if eager_first else 2)
+    h, s = t.sess.h, torch.cuda.Stream()
+    q, kn, vn = wl.step_inputs(cfg, 0, 0, "cuda")
+    out, ref = torch.zeros_like(q), torch.zeros_like(q)
+    torch.cuda.synchronize()
+    if eager_first:
+        kd.kv_begin_step(h, t.sess.seq_ids, s)
+        kd.decode_attention_append(h, 0, 6, q, kn, vn, out, 0.0, s)
+        s.synchronize()
+        kd.kv_cache_set_split_pages(h, 2)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        kd.kv_begin_step(h, t.sess.seq_ids, s)
+        kd.decode_attention_append(h, 0, 6, q, kn, vn, out, 0.0, s)
+    if replay:
+        with torch.cuda.stream(s):
+            g.replay()
+    kd.kv_cache_set_split_pages(h, 4)
+    kd.kv_begin_step(h, t.sess.seq_ids, s)
+    kd.kv_append(h, 0, 6, kn, vn, s)
+    kd.decode_attention(h, 0, 6, q, out, 0.0, s)
+    kd.decode_attention_append(h, 0, 6, q, kn, vn, ref, 0.0, s)
+    s.synchronize()
+    assert t.sess.query().device_error == 0 and float(out.abs().max()) > 0 and torch.equal(out, ref)
+    t.sess.lens += 3 if eager_first else 2
+    t.close()
+
+
 @pytest.mark.parametrize("way", ["captured", "device steps of one row"])
 def test_one_page_rows_without_plan_buffers(kvlib, way):
     """A host step of one-page rows runs as a plan of whole rows; where its
