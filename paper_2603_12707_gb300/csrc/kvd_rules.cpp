@@ -188,7 +188,7 @@ ClusterShape pick_cluster_shape(ResidentClusters resident, int device, int D, bo
     auto most_grown = [&](int64_t n) -> int64_t {
         if (gqa) {
             if (n == 64 || (n == 32 && D == 64 && units >= 38)) return limit;
-            return n == 32 ? 16 : n == 16 ? 32 : n == 8 ? 9 : 8;
+            return n == 32 ? 17 : n == 16 ? 33 : n == 8 ? 9 : 8;
         }
         if (units * n > 900 && (batch == 1 || n == 32)) return batch == 1 ? limit : D == 128 ? 8 : 18;
         return D == 128 ? (n == 16 ? 6 : 4) : n == 64 ? 9 : n == 16 ? 7 : 5;

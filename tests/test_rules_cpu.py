@@ -229,6 +229,7 @@ def test_clusters_of_long_tables(rules):
     assert rules.shape(32, 32, 128, [4], limit=256) == (8, 4, 3)     # one request in a 4096-token context
     assert rules.shape(28, 4, 128, [4] * 2, limit=2048) == (8, 8, 3)
     assert rules.shape(28, 4, 128, [4] * 8, limit=512) == (8, 4, 3)
+    assert rules.shape(28, 4, 128, [4] * 8, limit=520) == (8, 4, 3)  # 8192 tokens and a little room
     assert rules.shape(28, 4, 128, [4] * 8, limit=2048) == (0, 0, 0)
     assert rules.shape(32, 32, 128, [4] * 3, limit=256) == (0, 0, 0)
 
